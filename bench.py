@@ -52,9 +52,9 @@ NBODY_TRAFFIC = 2311424.0
 FF2_TRAFFIC = 15.17e6
 FF_TRAFFIC = 15.2e6
 # float32 lane operations (FADD, FMUL, FFMA each 1; a packed instruction 2) per ordered pair that
-# the float-float evaluation issues, counted by ncu on the packed mutual kernel: the emulation's
+# the float-float evaluation by pairs of triangles issues, counted in its source: the emulation's
 # cost, against 20 / 28 flops of the method's own arithmetic
-FF_OPS_PAIR = {"laplace": 97.7, "yukawa": 145.7}
+FF_OPS_PAIR = {"laplace": 58.0, "yukawa": 82.0}
 # the oracle's measured full solve of this workload on one host (x86-64, 8 cores: dense BEM
 # set-up and the default-tolerance solve, written by tests/golden/make_golden.py), against which
 # the sampled CPU model was checked once on that host
@@ -361,19 +361,15 @@ def run_pbfb(args):
                               traffic=None if tree else NBODY_TRAFFIC,
                               peak_basis=peak_basis))
         lff, msff = prof["nbodyff_launches"], prof["nbodyff_ms"]
-        packed_ff = tuned.get("ff_kernel") == 4
         if lff:
-            cands.append(dict(kernel="k_nbody_ffm2 (float-float far field of the Newton residual, mutual pairs, "
-                                     "2 targets per thread)" if packed_ff else
-                                     "k_nbody_ffm (float-float far field of the Newton residual, mutual pairs)",
+            cands.append(dict(kernel="k_pairs_ff (float-float far field of the Newton residual by pairs of triangles)",
                               launches=lff, ms=msff, pairs=prof["nbodyff_pairs"],
                               flops=prof["nbodyff_pairs"] * fpair,
                               lane_ops=prof["nbodyff_pairs"] * 0.5 * (FF_OPS_PAIR["laplace"] + FF_OPS_PAIR["yukawa"]),
-                              peak=peak32, traffic=FF2_TRAFFIC if packed_ff else FF_TRAFFIC,
-                              peak_basis=peak_basis))
+                              peak=peak32, traffic=None, peak_basis=peak_basis))
     else:
         l64, ms64 = prof["nbody64_launches"], prof["nbody64_ms"]
-        cands.append(dict(kernel="k_nbody_f64", launches=l64, ms=ms64, pairs=prof["nbody64_pairs"],
+        cands.append(dict(kernel="k_pairs_f64", launches=l64, ms=ms64, pairs=prof["nbody64_pairs"],
                           flops=prof["nbody64_pairs"] * fpair,
                           peak=1.25, traffic=None, peak_basis="fp64 nominal 1.25 TFLOP/s (GB300)"))
 
@@ -385,7 +381,7 @@ def run_pbfb(args):
         if c.get("lane_ops") and avg_ms > 0:
             peak_lanes = sm_count * FP32_LANES * sm_mhz * 1e6 / 1e12
             a = (c["lane_ops"] / launches) / (avg_ms * 1e-3) / 1e12
-            emu = {"note": "float-float emulation: float32 lane operations issued per ordered pair (ncu) "
+            emu = {"note": "float-float emulation: float32 lane operations issued per ordered pair (source count) "
                            f"{FF_OPS_PAIR['laplace']} Laplace / {FF_OPS_PAIR['yukawa']} Yukawa against the "
                            "method's 20 / 28 flops",
                    "achieved": a, "peak": peak_lanes, "unit": "T float32 lane-ops/s", "frac": a / peak_lanes}

@@ -383,10 +383,11 @@ typedef struct pbfb_tuning {
                                         2: mutual pairs, each point pair evaluated once for
                                         both directions (4 targets per thread; blocks_per_sm
                                         counts one-warp blocks) */
-  int32_t ff_blocks_per_sm;          /* float-float far field source splits: 1..64 */
-  int32_t ff_kernel;                 /* float-float far field: 1 one target per thread,
-                                        2 two per thread (float2), 3 mutual pairs, 4 mutual
-                                        pairs with two targets per thread (float2) */
+  int32_t ff_blocks_per_sm;          /* float-float far field: an eighth of its tasks per SM
+                                        (ff_kernel 1: source splits), 1..64 */
+  int32_t ff_kernel;                 /* float-float far field: 1 one target per thread; 0, 2, 3
+                                        and 4 pairs of triangles, each pair of points evaluated
+                                        once for both directions (float2) */
   int32_t spmv_lanes;                /* lanes per row of the operator's SpMV: 4, 8, 16 */
   int32_t spmv_block;                /* threads per block of that SpMV: 128, 256, 512 */
   int32_t pcg_blocks_per_sm;         /* blocks per SM of the cooperative inner PCG: 1..32
@@ -428,8 +429,8 @@ int pbfb_apply_tuning(pbfb_mesh* mesh, const pbfb_tuning* t);
  * candidate shape of the float32 far field (targets per thread 1/2/4, packed
  * or not, 8/16/32 blocks per SM of source splits; or mutual pairs with
  * 16/32/64 one-warp blocks per SM) and of the float-float far
- * field (4/8/16 blocks per SM; one or two targets per thread, or mutual
- * pairs evaluated once for both directions) on both
+ * field (4/8/16/24 blocks per SM; one target per thread, or pairs of
+ * triangles) on both
  * surfaces of this mesh at the current parameters, and of the operator's
  * SpMV (4/8/16 lanes per row x 128/256/512 threads) and of the cooperative
  * inner PCG of the block preconditioner (1/2/4/8 blocks per SM or all that

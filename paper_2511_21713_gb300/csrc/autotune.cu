@@ -151,7 +151,7 @@ int autotune(Mesh* m, int reps, pbfb_tuning* best_out, double* ms_out) {
     }
   }
   // float-float far field
-  for (int kind : {1, 2, 3, 4})
+  for (int kind : {1, 4})
     for (int bps : {4, 8, 16, 24}) {
       pbfb_tuning t = best;
       t.ff_kernel = kind;

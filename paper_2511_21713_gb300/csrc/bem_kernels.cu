@@ -273,6 +273,15 @@ __global__ void k_pair_corrections(int npair, const int* __restrict__ pt_, const
     }
     double g, dl;
     K.eval(X, Y, ns, g, dl);
+    // the far field's plane distance: from the trial triangle's first point, 0 within a triangle
+    {
+      const double d0 = X[0] - Y[0], d1 = X[1] - Y[1], d2 = X[2] - Y[2];
+      const double r2 = d0 * d0 + d1 * d1 + d2 * d2, r = sqrt(r2);
+      const double D = t == s ? 0.0
+                              : fma(ns[2], X[2] - qx[2 * nqt + QS * s],
+                                    fma(ns[1], X[1] - qx[nqt + QS * s], ns[0] * (X[0] - qx[QS * s])));
+      dl = D * (1.0 + kappa * r) * g / r2;
+    }
     double W = qw[QS * t + q] * qw[QS * s + p];
     for (int a = 0; a < 3; ++a)
       for (int b = 0; b < 3; ++b) {
@@ -308,9 +317,8 @@ __global__ void k_pair_corrections(int npair, const int* __restrict__ pt_, const
 __global__ void k_sources(int nt, const int* __restrict__ tri, const int* __restrict__ vmap,
                           const double* __restrict__ lam, const double* __restrict__ u, int u_local,
                           const double* __restrict__ qw, const double* __restrict__ nrm,
-                          const float4* __restrict__ qpf, const double* __restrict__ qx, double cs, double cd,
-                          int want64, float4* __restrict__ spos, float4* __restrict__ sdl,
-                          double* __restrict__ s64) {
+                          const float4* __restrict__ qpf, double cs, double cd, float4* __restrict__ spos,
+                          float4* __restrict__ sdl) {
   int j = blockIdx.x * blockDim.x + threadIdx.x;
   int nq = QS * nt;
   if (j >= nq) return;
@@ -325,20 +333,10 @@ __global__ void k_sources(int nt, const int* __restrict__ tri, const int* __rest
   double w = qw[j];
   double sv = cs * w * lh, mu = cd * w * uh;
   double n0 = nrm[t], n1 = nrm[nt + t], n2 = nrm[2 * nt + t];
-  if (want64) {
-    s64[j] = qx[j];
-    s64[nq + j] = qx[nq + j];
-    s64[2 * nq + j] = qx[2 * nq + j];
-    s64[3 * nq + j] = sv;
-    s64[4 * nq + j] = mu * n0;
-    s64[5 * nq + j] = mu * n1;
-    s64[6 * nq + j] = mu * n2;
-  } else {
-    float4 p = qpf[j];
-    p.w = (float)sv;
-    spos[j] = p;
-    sdl[j] = make_float4((float)(mu * n0), (float)(mu * n1), (float)(mu * n2), 0.f);
-  }
+  float4 p = qpf[j];
+  p.w = (float)sv;
+  spos[j] = p;
+  sdl[j] = make_float4((float)(mu * n0), (float)(mu * n1), (float)(mu * n2), 0.f);
 }
 
 // float32 N-body: targets = sources = the nq quadrature points.  Block = NT threads, each
@@ -569,7 +567,7 @@ __global__ void __launch_bounds__(NT) k_nbody_f32x2(int nq, const float4* __rest
 }
 
 // Mutual float32 N-body for the GMRES operator: every unordered pair of points evaluated once
-// for both directions (the organisation of k_nbody_ffm, with one-warp blocks).  Block (rg, cg)
+// for both directions, with one-warp blocks.  Block (rg, cg)
 // is one warp; it holds 4 targets per lane (I * 128 + lane + 32 k) as two f32x2 pairs, streams
 // the 128 points of tile J through shared memory, and at step s lane l takes point (l + s) mod
 // 128, so the 32 lanes update distinct source-side sums (warp-synchronous, fixed order).  Pair
@@ -725,47 +723,6 @@ __global__ void __launch_bounds__(32) k_nbody_f32m(int nq, int G, const float4* 
   }
 }
 
-// float64 N-body, same organisation (one target per thread).
-template <int NT, bool YUK>
-__global__ void __launch_bounds__(NT) k_nbody_f64(int nq, const double* __restrict__ s64, double kappa,
-                                                  int per_split, double* __restrict__ out) {
-  __shared__ double sh[7][NT];
-  const int i = blockIdx.x * NT + threadIdx.x;
-  const int ii = i < nq ? i : 0;
-  const double x = s64[ii], y = s64[nq + ii], z = s64[2 * nq + ii];
-  const int sb = blockIdx.y * per_split;
-  const int se = min(nq, sb + per_split);
-  double acc = 0.0;
-  for (int s0 = sb; s0 < se; s0 += NT) {
-    int j = s0 + threadIdx.x;
-    if (j < se) {
-      for (int c = 0; c < 7; ++c) sh[c][threadIdx.x] = s64[c * nq + j];
-    } else {
-      sh[0][threadIdx.x] = sh[1][threadIdx.x] = sh[2][threadIdx.x] = 1e150;
-      for (int c = 3; c < 7; ++c) sh[c][threadIdx.x] = 0.0;
-    }
-    __syncthreads();
-    const int cnt = min(NT, se - s0);
-    for (int jj = 0; jj < cnt; ++jj) {
-      if (s0 + jj == i) continue;
-      double dx = x - sh[0][jj], dy = y - sh[1][jj], dz = z - sh[2][jj];
-      double r2 = dx * dx + dy * dy + dz * dz;
-      double ri = rsqrt(r2);
-      double nd = sh[4][jj] * dx + sh[5][jj] * dy + sh[6][jj] * dz;
-      double ri2 = ri * ri;
-      if (YUK) {
-        double r = r2 * ri;
-        double e = exp(-kappa * r);
-        acc += (sh[3][jj] + nd * (1.0 + kappa * r) * ri2) * e * ri;
-      } else {
-        acc += (sh[3][jj] + nd * ri2) * ri;
-      }
-    }
-    __syncthreads();
-  }
-  if (i < nq) out[(int64_t)blockIdx.y * nq + i] = acc;
-}
-
 // ---------------------------------------------------------------- float-float far field
 //
 // The Newton residual needs a far field accurate to float64 level, but the float64 rate of
@@ -886,7 +843,7 @@ __global__ void k_sources_ff(int nt, const int* __restrict__ tri, const int* __r
   for (int d = 0; d < 3; ++d) {
     const double yq = rint(y[d] / grid) * grid;  // on the grid: exact in float32
     yh[d] = (float)yq;
-    yl[d] = (float)(y[d] - yq);
+    yl[d] = (float)(rint((y[d] - yq) / (grid * 0x1p-24)) * (grid * 0x1p-24));
     mh[d] = (float)mm[d];
     ml[d] = (float)(mm[d] - (double)mh[d]);
   }
@@ -960,470 +917,6 @@ __global__ void __launch_bounds__(NT) k_nbody_ff(int nq, const float4* __restric
     __syncthreads();
   }
   if (i < nq) out[(int64_t)blockIdx.y * nq + i] = acc64;
-}
-
-// Packed float-float N-body: two targets per thread, every float-float operation applied to both
-// with the Blackwell float2 arithmetic (__fadd2_rn / __fmul2_rn / __ffma2_rn, per component the
-// same rounding as the scalar _rn operations), halving the issue slots of k_nbody_ff.  Each lane
-// performs the scalar kernel's operation sequence under the same source split (results agree to
-// float-float rounding).  Sources are staged pre-duplicated; tiles holding one of the thread's
-// own targets take the scalar path for the coincident-point test.
-struct ffv { float2 h, l; };
-__device__ __forceinline__ float2 vdup(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __fadd2_rn(a, vneg(b)); }
-__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-
-__device__ __forceinline__ ffv v_two_sum(float2 a, float2 b) {
-  float2 s = vadd(a, b);
-  float2 bb = vsub(s, a);
-  float2 e = vadd(vsub(a, vsub(s, bb)), vsub(b, bb));
-  return {s, e};
-}
-__device__ __forceinline__ ffv v_fast_two_sum(float2 a, float2 b) {
-  float2 s = vadd(a, b);
-  return {s, vsub(b, vsub(s, a))};
-}
-__device__ __forceinline__ ffv v_add(ffv a, ffv b) {
-  ffv s = v_two_sum(a.h, b.h);
-  float2 lo = vadd(s.l, vadd(a.l, b.l));
-  return v_fast_two_sum(s.h, lo);
-}
-__device__ __forceinline__ ffv v_mul(ffv a, ffv b) {
-  float2 p = vmul(a.h, b.h);
-  float2 e = vfma(a.h, b.h, vneg(p));
-  e = vfma(a.h, b.l, e);
-  e = vfma(a.l, b.h, e);
-  return v_fast_two_sum(p, e);
-}
-__device__ __forceinline__ ffv v_sq(ffv a) {
-  float2 p = vmul(a.h, a.h);
-  float2 e = vfma(a.h, a.h, vneg(p));
-  e = vfma(vadd(a.h, a.h), a.l, e);
-  return v_fast_two_sum(p, e);
-}
-__device__ __forceinline__ ffv v_diff(float2 xh, float2 xl, float2 yh, float2 yl) {
-  return v_fast_two_sum(vsub(xh, yh), vsub(xl, yl));
-}
-__device__ __forceinline__ ffv v_dot3(ffv a0, ffv a1, ffv a2, ffv b0, ffv b1, ffv b2) {
-  float2 p0 = vmul(a0.h, b0.h), p1 = vmul(a1.h, b1.h), p2 = vmul(a2.h, b2.h);
-  float2 e0 = vfma(a0.l, b0.h, vfma(a0.h, b0.l, vfma(a0.h, b0.h, vneg(p0))));
-  float2 e1 = vfma(a1.l, b1.h, vfma(a1.h, b1.l, vfma(a1.h, b1.h, vneg(p1))));
-  float2 e2 = vfma(a2.l, b2.h, vfma(a2.h, b2.l, vfma(a2.h, b2.h, vneg(p2))));
-  ffv s1 = v_two_sum(p0, p1);
-  ffv s2 = v_two_sum(s1.h, p2);
-  float2 lo = vadd(vadd(s1.l, s2.l), vadd(vadd(e0, e1), e2));
-  return v_fast_two_sum(s2.h, lo);
-}
-__device__ __forceinline__ ffv v_rsqrt(ffv r) {
-  float2 y0 = make_float2(rsqrtf(r.h.x), rsqrtf(r.h.y));
-  float2 t = vmul(y0, y0);
-  float2 te = vfma(y0, y0, vneg(t));
-  float2 a = vmul(r.h, t);
-  float2 ae = vfma(r.h, t, vneg(a));
-  float2 z = vadd(vsub(a, vdup(1.0f)), vfma(r.l, t, vfma(r.h, te, ae)));
-  return v_fast_two_sum(y0, vmul(vmul(vdup(-0.5f), y0), z));
-}
-// exp(-x) per lane as ff_expm; the table index is clamped and the lanes with x >= FF_XMAX give 0
-__device__ __forceinline__ ffv v_expm(ffv x, const float2* __restrict__ tab_hi) {
-  float2 xs = vmul(x.h, vdup(256.0f));
-  int k0 = __float2int_rd(xs.x), k1 = __float2int_rd(xs.y);
-  k0 = min(max(k0, 0), FF_TABLE_HI * 16 - 1);
-  k1 = min(max(k1, 0), FF_TABLE_HI * 16 - 1);
-  float2 kf = vmul(make_float2((float)k0, (float)k1), vdup(0.00390625f));
-  ffv f = v_fast_two_sum(vsub(x.h, kf), x.l);
-  ffv f2 = v_sq(f);
-  float2 p2 = vmul(f.h, vfma(f.h, vfma(f.h, vdup(-1.0f / 120.0f), vdup(1.0f / 24.0f)), vdup(-1.0f / 6.0f)));
-  ffv one_minus = v_two_sum(vdup(1.0f), vneg(f.h));
-  one_minus = v_fast_two_sum(one_minus.h, vsub(one_minus.l, f.l));
-  ffv tail = v_fast_two_sum(vmul(vdup(0.5f), f2.h), vfma(f2.h, p2, vmul(vdup(0.5f), f2.l)));
-  ffv ef = v_add(one_minus, tail);
-  const float2 a0 = tab_hi[k0 >> 4], a1 = tab_hi[k1 >> 4];
-  const float2 b0 = c_ff_exp_lo[k0 & 15], b1 = c_ff_exp_lo[k1 & 15];
-  ffv r = v_mul(v_mul(ef, ffv{make_float2(a0.x, a1.x), make_float2(a0.y, a1.y)}),
-                ffv{make_float2(b0.x, b1.x), make_float2(b0.y, b1.y)});
-  if (x.h.x >= FF_XMAX) r.h.x = r.l.x = 0.f;
-  if (x.h.y >= FF_XMAX) r.h.y = r.l.y = 0.f;
-  return r;
-}
-
-// per source, duplicated: yh.x yh.y | yh.z sh | yl.x yl.y | yl.z sl | mh.x mh.y | mh.z ml.x | ml.y ml.z
-template <bool YUK>
-__device__ __forceinline__ ffv v_pair(const float4* __restrict__ q, const float2 (&th)[3], const float2 (&tl)[3],
-                                      ffv kap, const float2* __restrict__ tab) {
-  const float4 c0 = q[0], c1 = q[1], c2 = q[2], c3 = q[3], c4 = q[4], c5 = q[5], c6 = q[6];
-  const float2 pxh = make_float2(c0.x, c0.y), pyh = make_float2(c0.z, c0.w);
-  const float2 pzh = make_float2(c1.x, c1.y), sh = make_float2(c1.z, c1.w);
-  const float2 pxl = make_float2(c2.x, c2.y), pyl = make_float2(c2.z, c2.w);
-  const float2 pzl = make_float2(c3.x, c3.y), sl = make_float2(c3.z, c3.w);
-  const ffv mx{make_float2(c4.x, c4.y), make_float2(c5.z, c5.w)};
-  const ffv my{make_float2(c4.z, c4.w), make_float2(c6.x, c6.y)};
-  const ffv mz{make_float2(c5.x, c5.y), make_float2(c6.z, c6.w)};
-  ffv d0 = v_diff(th[0], tl[0], pxh, pxl);
-  ffv d1 = v_diff(th[1], tl[1], pyh, pyl);
-  ffv d2 = v_diff(th[2], tl[2], pzh, pzl);
-  ffv r2 = v_dot3(d0, d1, d2, d0, d1, d2);
-  ffv ri = v_rsqrt(r2);
-  ffv nd = v_dot3(mx, my, mz, d0, d1, d2);
-  ffv ri2 = v_sq(ri);
-  if (YUK) {
-    ffv r = v_mul(r2, ri);
-    ffv x = v_mul(kap, r);
-    ffv e = v_expm(x, tab);
-    ffv one_x = v_two_sum(vdup(1.0f), x.h);
-    one_x = v_fast_two_sum(one_x.h, vadd(one_x.l, x.l));
-    ffv t = v_add(ffv{sh, sl}, v_mul(v_mul(nd, one_x), ri2));
-    return v_mul(t, v_mul(e, ri));
-  }
-  ffv t = v_add(ffv{sh, sl}, v_mul(nd, ri2));
-  return v_mul(t, ri);
-}
-
-template <int NT, bool YUK>
-__global__ void __launch_bounds__(NT) k_nbody_ff2(int nq, const float4* __restrict__ tgt,
-                                                  const float4* __restrict__ src, float kh, float kl,
-                                                  const float2* __restrict__ tab_hi, int per_split,
-                                                  double* __restrict__ out) {
-  __shared__ float4 shv[NT][7];   // duplicated (packed) copies
-  __shared__ float4 shs[4][NT];   // scalar copies for the tiles that hold the thread's own targets
-  __shared__ float2 tab[YUK ? FF_TABLE_HI : 1];
-  if (YUK)
-    for (int k = threadIdx.x; k < FF_TABLE_HI; k += NT) tab[k] = tab_hi[k];
-  const int t0 = blockIdx.x * 2 * NT;
-  const int i0 = t0 + threadIdx.x, i1 = t0 + NT + threadIdx.x;
-  const int c0 = i0 < nq ? i0 : 0, c1 = i1 < nq ? i1 : 0;
-  const float4 a0 = tgt[2 * c0], b0 = tgt[2 * c0 + 1];
-  const float4 a1 = tgt[2 * c1], b1 = tgt[2 * c1 + 1];
-  const float2 th[3] = {make_float2(a0.x, a1.x), make_float2(a0.y, a1.y), make_float2(a0.z, a1.z)};
-  const float2 tl[3] = {make_float2(b0.x, b1.x), make_float2(b0.y, b1.y), make_float2(b0.z, b1.z)};
-  const float ths0[3] = {a0.x, a0.y, a0.z}, tls0[3] = {b0.x, b0.y, b0.z};
-  const float ths1[3] = {a1.x, a1.y, a1.z}, tls1[3] = {b1.x, b1.y, b1.z};
-  const ffv kapv{vdup(kh), vdup(kl)};
-  const ff kap{kh, kl};
-  const int sb = blockIdx.y * per_split;
-  const int se = min(nq, sb + per_split);
-  double acc0 = 0.0, acc1 = 0.0;
-  for (int s0 = sb; s0 < se; s0 += NT) {
-    const int j = s0 + threadIdx.x;
-    float4 c[4];
-    if (j < se) {
-      for (int k = 0; k < 4; ++k) c[k] = src[4 * j + k];
-    } else {  // never read: the loops below stop at se
-      c[0] = c[1] = c[2] = c[3] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    for (int k = 0; k < 4; ++k) shs[k][threadIdx.x] = c[k];
-    shv[threadIdx.x][0] = make_float4(c[0].x, c[0].x, c[0].y, c[0].y);
-    shv[threadIdx.x][1] = make_float4(c[0].z, c[0].z, c[0].w, c[0].w);
-    shv[threadIdx.x][2] = make_float4(c[1].x, c[1].x, c[1].y, c[1].y);
-    shv[threadIdx.x][3] = make_float4(c[1].z, c[1].z, c[1].w, c[1].w);
-    shv[threadIdx.x][4] = make_float4(c[2].x, c[2].x, c[2].y, c[2].y);
-    shv[threadIdx.x][5] = make_float4(c[2].z, c[2].z, c[3].x, c[3].x);
-    shv[threadIdx.x][6] = make_float4(c[3].y, c[3].y, c[3].z, c[3].z);
-    __syncthreads();
-    const int cnt = min(NT, se - s0);
-    const bool diag = (s0 < t0 + 2 * NT) && (s0 + NT > t0);
-    if (!diag) {
-      ffv acc{vdup(0.f), vdup(0.f)};
-      for (int jj = 0; jj < cnt; ++jj) acc = v_add(acc, v_pair<YUK>(shv[jj], th, tl, kapv, tab));
-      acc0 += (double)acc.h.x + (double)acc.l.x;
-      acc1 += (double)acc.h.y + (double)acc.l.y;
-    } else {
-      ff s0acc{0.f, 0.f}, s1acc{0.f, 0.f};
-      for (int jj = 0; jj < cnt; ++jj) {
-        if (s0 + jj != i0)
-          s0acc = ff_add(s0acc, ff_pair<YUK>(shs[0][jj], shs[1][jj], shs[2][jj], shs[3][jj], ths0, tls0, kap, tab));
-        if (s0 + jj != i1)
-          s1acc = ff_add(s1acc, ff_pair<YUK>(shs[0][jj], shs[1][jj], shs[2][jj], shs[3][jj], ths1, tls1, kap, tab));
-      }
-      acc0 += (double)s0acc.h + (double)s0acc.l;
-      acc1 += (double)s1acc.h + (double)s1acc.l;
-    }
-    __syncthreads();
-  }
-  if (i0 < nq) out[(int64_t)blockIdx.y * nq + i0] = acc0;
-  if (i1 < nq) out[(int64_t)blockIdx.y * nq + i1] = acc1;
-}
-
-// Mutual float-float N-body: every unordered pair of points is evaluated once for both
-// directions.  The pair (i, j) shares d = x_i - y_j, 1/r and, for the Yukawa kernel, exp(-kappa r);
-// with f = (1 + kappa r) / r^2 and g = exp(-kappa r) / r it contributes
-//   (s_j + (m_j . d) f) g  to target i   and   (s_i - (m_i . d) f) g  to target j,
-// saving the shared part of the float-float work (about 30% of the operations).
-//
-// Points are cut into tiles of MT = 128 and the tiles into G groups; block (rg, cg), rg <= cg, takes
-// every tile pair (I in rg, J in cg, I < J) and the diagonal tiles I = J (one direction, coincident
-// point skipped).  Target-side sums stay in registers and go to PI[cg][i]; source-side sums are
-// accumulated in shared memory per tile pair and added to PJ[rg][j], which only this block touches.
-// Within a tile pair, step s of the 128 takes source 32 ((w + s / 32) mod 4) + (lane + s) mod 32 in
-// warp w: the warps work on disjoint quarters of the source tile between barriers and the lanes of
-// a warp on distinct sources, so the shared-memory sums have no races and a fixed order.  The
-// final value of a point is the fixed-order sum of its 2 G partials (k_mutual_sum).
-constexpr int MT = 128;
-
-template <bool YUK>
-__device__ __forceinline__ void ff_mutual(const float4& ah, const float4& al, const float4& amh, const float4& aml,
-                                          const float4& bh, const float4& bl, const float4& bmh, const float4& bml,
-                                          ff kap, const float2* __restrict__ tab, ff& to_a, ff& to_b) {
-  // a = target (x, s, m), b = source (y, s, m); float4 (x, y, z, s) hi / lo, (mx, my, mz, -) hi / lo
-  ff d0 = ff_diff(ah.x, al.x, bh.x, bl.x);
-  ff d1 = ff_diff(ah.y, al.y, bh.y, bl.y);
-  ff d2 = ff_diff(ah.z, al.z, bh.z, bl.z);
-  ff r2 = ff_dot3(d0, d1, d2, d0, d1, d2);
-  ff ri = ff_rsqrt(r2);
-  ff ri2 = ff_sq(ri);
-  ff f, g;
-  if (YUK) {
-    ff r = ff_mul(r2, ri);
-    ff x = ff_mul(kap, r);
-    ff e = ff_expm(x, tab);
-    ff one_x = two_sum(1.0f, x.h);
-    one_x = fast_two_sum(one_x.h, __fadd_rn(one_x.l, x.l));
-    f = ff_mul(one_x, ri2);
-    g = ff_mul(e, ri);
-  } else {
-    f = ri2;
-    g = ri;
-  }
-  ff ndb = ff_dot3(ff{bmh.x, bml.x}, ff{bmh.y, bml.y}, ff{bmh.z, bml.z}, d0, d1, d2);
-  ff nda = ff_dot3(ff{amh.x, aml.x}, ff{amh.y, aml.y}, ff{amh.z, aml.z}, d0, d1, d2);
-  ff fb = ff_mul(ndb, f), fa = ff_mul(nda, f);
-  to_a = ff_mul(ff_add(ff{bh.w, bl.w}, fb), g);
-  to_b = ff_mul(ff_add(ff{ah.w, al.w}, ff{-fa.h, -fa.l}), g);
-}
-
-template <bool YUK>
-__global__ void __launch_bounds__(MT) k_nbody_ffm(int nq, int G, const float4* __restrict__ src, float kh, float kl,
-                                                  const float2* __restrict__ tab_hi, double* __restrict__ PI,
-                                                  double* __restrict__ PJ) {
-  __shared__ float4 sb[4][MT];              // source tile: (y, s) hi, (y, s) lo, m hi, m lo
-  __shared__ float2 acc_j[MT];              // source-side float-float sums of the current tile pair
-  __shared__ float2 tab[YUK ? FF_TABLE_HI : 1];
-  if (YUK)
-    for (int k = threadIdx.x; k < FF_TABLE_HI; k += MT) tab[k] = tab_hi[k];
-  // block -> (rg, cg), rg <= cg
-  int t = blockIdx.x, rg = 0;
-  while (t >= G - rg) {
-    t -= G - rg;
-    ++rg;
-  }
-  const int cg = rg + t;
-  const int nT = (nq + MT - 1) / MT;
-  const int tpg = (nT + G - 1) / G;
-  const int i0g = rg * tpg, i1g = min(nT, (rg + 1) * tpg);
-  const int j0g = cg * tpg, j1g = min(nT, (cg + 1) * tpg);
-  const ff kap{kh, kl};
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int I = i0g; I < i1g; ++I) {
-    const int i = I * MT + threadIdx.x;
-    const bool iv = i < nq;
-    // invalid targets sit far away with zero strength
-    float4 ah = iv ? src[4 * i] : make_float4(2e15f, 0.f, 0.f, 0.f);
-    float4 al = iv ? src[4 * i + 1] : make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 amh = iv ? src[4 * i + 2] : make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 aml = iv ? src[4 * i + 3] : make_float4(0.f, 0.f, 0.f, 0.f);
-    double acc64 = 0.0;
-    for (int J = max(I, j0g); J < j1g; ++J) {
-      const int jl = J * MT + threadIdx.x;
-      __syncthreads();  // the previous tile's readers are done
-      if (jl < nq) {
-        for (int c = 0; c < 4; ++c) sb[c][threadIdx.x] = src[4 * jl + c];
-      } else {
-        sb[0][threadIdx.x] = make_float4(1e15f, 0.f, 0.f, 0.f);
-        sb[1][threadIdx.x] = sb[2][threadIdx.x] = sb[3][threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-      acc_j[threadIdx.x] = make_float2(0.f, 0.f);
-      __syncthreads();
-      const int cnt = min(MT, nq - J * MT);
-      ff acc{0.f, 0.f};
-      if (J == I) {
-        // diagonal tile: target side only, coincident point skipped
-        const float th[3] = {ah.x, ah.y, ah.z}, tl[3] = {al.x, al.y, al.z};
-        for (int jj = 0; jj < cnt; ++jj) {
-          if (jj == (int)threadIdx.x) continue;
-          acc = ff_add(acc, ff_pair<YUK>(sb[0][jj], sb[1][jj], sb[2][jj], sb[3][jj], th, tl, kap, tab));
-        }
-      } else {
-        for (int ph = 0; ph < 4; ++ph) {
-          const int base = 32 * ((warp + ph) & 3);
-          for (int k = 0; k < 32; ++k) {
-            const int jj = base + ((lane + k) & 31);
-            ff ta, tb;
-            ff_mutual<YUK>(ah, al, amh, aml, sb[0][jj], sb[1][jj], sb[2][jj], sb[3][jj], kap, tab, ta, tb);
-            // running sums kept as (high, low) with the low parts and TwoSum errors added plainly
-            // (at most 128 terms per tile pair, converted to float64 at its end)
-            const ff sa = two_sum(acc.h, ta.h);
-            acc = ff{sa.h, __fadd_rn(acc.l, __fadd_rn(sa.l, ta.l))};
-            const float2 o = acc_j[jj];
-            const ff sj = two_sum(o.x, tb.h);
-            acc_j[jj] = make_float2(sj.h, __fadd_rn(o.y, __fadd_rn(sj.l, tb.l)));
-            __syncwarp();
-          }
-          __syncthreads();
-        }
-        // source-side sums of this tile pair into PJ[rg][j]
-        if (jl < nq) {
-          const float2 o = acc_j[threadIdx.x];
-          PJ[(int64_t)rg * nq + jl] += (double)o.x + (double)o.y;
-        }
-      }
-      acc64 += (double)acc.h + (double)acc.l;
-    }
-    if (iv) PI[(int64_t)cg * nq + i] = acc64;
-  }
-}
-
-// Packed mutual float-float N-body: k_nbody_ffm's pair organisation with two targets per thread
-// on the float2 instructions.  Tiles hold MT2 = 256 points (targets i and i + 128 of a tile in one
-// thread); a thread evaluates each source of the tile pair against both of its targets at once
-// (the per-lane operation sequence of ff_mutual, so every pair value equals the scalar kernel's),
-// adds the two lanes' source-side contributions and folds them into the tile's shared sums.  The
-// 256 sources are visited in 8 chunks of 32: in phase p warp w takes chunk (w + p) mod 8 (the 4
-// warps on distinct chunks between barriers) and lane l at step k source (l + k) mod 32 of it.
-// Diagonal tiles take the scalar one-direction path with the coincident point skipped.
-constexpr int MT2 = 2 * MT;
-
-template <bool YUK>
-__device__ __forceinline__ void v_mutual(const float2 (&ah)[3], const float2 (&al)[3], const ffv (&am)[3],
-                                         const ffv& as, const float4& bh, const float4& bl, const float4& bmh,
-                                         const float4& bml, ffv kap, const float2* __restrict__ tab, ffv& to_a,
-                                         ffv& to_b) {
-  ffv d0 = v_diff(ah[0], al[0], vdup(bh.x), vdup(bl.x));
-  ffv d1 = v_diff(ah[1], al[1], vdup(bh.y), vdup(bl.y));
-  ffv d2 = v_diff(ah[2], al[2], vdup(bh.z), vdup(bl.z));
-  ffv r2 = v_dot3(d0, d1, d2, d0, d1, d2);
-  ffv ri = v_rsqrt(r2);
-  ffv ri2 = v_sq(ri);
-  ffv f, g;
-  if (YUK) {
-    ffv r = v_mul(r2, ri);
-    ffv x = v_mul(kap, r);
-    ffv e = v_expm(x, tab);
-    ffv one_x = v_two_sum(vdup(1.0f), x.h);
-    one_x = v_fast_two_sum(one_x.h, vadd(one_x.l, x.l));
-    f = v_mul(one_x, ri2);
-    g = v_mul(e, ri);
-  } else {
-    f = ri2;
-    g = ri;
-  }
-  ffv ndb = v_dot3(ffv{vdup(bmh.x), vdup(bml.x)}, ffv{vdup(bmh.y), vdup(bml.y)}, ffv{vdup(bmh.z), vdup(bml.z)}, d0,
-                   d1, d2);
-  ffv nda = v_dot3(am[0], am[1], am[2], d0, d1, d2);
-  ffv fb = v_mul(ndb, f), fa = v_mul(nda, f);
-  to_a = v_mul(v_add(ffv{vdup(bh.w), vdup(bl.w)}, fb), g);
-  to_b = v_mul(v_add(as, ffv{vneg(fa.h), vneg(fa.l)}), g);
-}
-
-template <bool YUK>
-__global__ void __launch_bounds__(MT) k_nbody_ffm2(int nq, int G, const float4* __restrict__ src, float kh,
-                                                   float kl, const float2* __restrict__ tab_hi,
-                                                   double* __restrict__ PI, double* __restrict__ PJ) {
-  __shared__ float4 sb[4][MT2];             // source tile: (y, s) hi, (y, s) lo, m hi, m lo
-  __shared__ float2 acc_j[MT2];             // source-side float-float sums of the current tile pair
-  __shared__ float2 tab[YUK ? FF_TABLE_HI : 1];
-  if (YUK)
-    for (int k = threadIdx.x; k < FF_TABLE_HI; k += MT) tab[k] = tab_hi[k];
-  int t = blockIdx.x, rg = 0;
-  while (t >= G - rg) {
-    t -= G - rg;
-    ++rg;
-  }
-  const int cg = rg + t;
-  const int nT = (nq + MT2 - 1) / MT2;
-  const int tpg = (nT + G - 1) / G;
-  const int i0g = rg * tpg, i1g = min(nT, (rg + 1) * tpg);
-  const int j0g = cg * tpg, j1g = min(nT, (cg + 1) * tpg);
-  const ff kap{kh, kl};
-  const ffv kapv{vdup(kh), vdup(kl)};
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int I = i0g; I < i1g; ++I) {
-    const int i0 = I * MT2 + threadIdx.x, i1 = i0 + MT;
-    const bool v0 = i0 < nq, v1 = i1 < nq;
-    // invalid targets sit far away with zero strength
-    const float4 a0h = v0 ? src[4 * i0] : make_float4(2e15f, 0.f, 0.f, 0.f);
-    const float4 a0l = v0 ? src[4 * i0 + 1] : zero4;
-    const float4 a0mh = v0 ? src[4 * i0 + 2] : zero4;
-    const float4 a0ml = v0 ? src[4 * i0 + 3] : zero4;
-    const float4 a1h = v1 ? src[4 * i1] : make_float4(2e15f, 0.f, 0.f, 0.f);
-    const float4 a1l = v1 ? src[4 * i1 + 1] : zero4;
-    const float4 a1mh = v1 ? src[4 * i1 + 2] : zero4;
-    const float4 a1ml = v1 ? src[4 * i1 + 3] : zero4;
-    const float2 ah[3] = {make_float2(a0h.x, a1h.x), make_float2(a0h.y, a1h.y), make_float2(a0h.z, a1h.z)};
-    const float2 al[3] = {make_float2(a0l.x, a1l.x), make_float2(a0l.y, a1l.y), make_float2(a0l.z, a1l.z)};
-    const ffv am[3] = {ffv{make_float2(a0mh.x, a1mh.x), make_float2(a0ml.x, a1ml.x)},
-                       ffv{make_float2(a0mh.y, a1mh.y), make_float2(a0ml.y, a1ml.y)},
-                       ffv{make_float2(a0mh.z, a1mh.z), make_float2(a0ml.z, a1ml.z)}};
-    const ffv as{make_float2(a0h.w, a1h.w), make_float2(a0l.w, a1l.w)};
-    double acc0 = 0.0, acc1 = 0.0;
-    for (int J = max(I, j0g); J < j1g; ++J) {
-      __syncthreads();  // the previous tile's readers are done
-      for (int h = 0; h < 2; ++h) {
-        const int slot = h * MT + threadIdx.x;
-        const int jl = J * MT2 + slot;
-        if (jl < nq) {
-          for (int c = 0; c < 4; ++c) sb[c][slot] = src[4 * jl + c];
-        } else {
-          sb[0][slot] = make_float4(1e15f, 0.f, 0.f, 0.f);
-          sb[1][slot] = sb[2][slot] = sb[3][slot] = zero4;
-        }
-        acc_j[slot] = make_float2(0.f, 0.f);
-      }
-      __syncthreads();
-      if (J == I) {
-        // diagonal tile: target side only, coincident point skipped (scalar, per target)
-        const int cnt = min(MT2, nq - J * MT2);
-        for (int q = 0; q < 2; ++q) {
-          const float4& xh = q == 0 ? a0h : a1h;
-          const float4& xl = q == 0 ? a0l : a1l;
-          const float th[3] = {xh.x, xh.y, xh.z}, tl[3] = {xl.x, xl.y, xl.z};
-          const int self = q * MT + (int)threadIdx.x;
-          ff acc{0.f, 0.f};
-          for (int jj = 0; jj < cnt; ++jj) {
-            if (jj == self) continue;
-            acc = ff_add(acc, ff_pair<YUK>(sb[0][jj], sb[1][jj], sb[2][jj], sb[3][jj], th, tl, kap, tab));
-          }
-          (q == 0 ? acc0 : acc1) += (double)acc.h + (double)acc.l;
-        }
-      } else {
-        ffv acc{vdup(0.f), vdup(0.f)};
-        for (int ph = 0; ph < 8; ++ph) {
-          const int base = 32 * ((warp + ph) & 7);
-          for (int k = 0; k < 32; ++k) {
-            const int jj = base + ((lane + k) & 31);
-            ffv ta, tb;
-            v_mutual<YUK>(ah, al, am, as, sb[0][jj], sb[1][jj], sb[2][jj], sb[3][jj], kapv, tab, ta, tb);
-            // running sums kept as (high, low) with the low parts and TwoSum errors added plainly
-            // (at most 256 terms per tile pair, converted to float64 at its end)
-            const ffv sa = v_two_sum(acc.h, ta.h);
-            acc = ffv{sa.h, vadd(acc.l, vadd(sa.l, ta.l))};
-            const ff tbs = two_sum(tb.h.x, tb.h.y);
-            const float tbl = __fadd_rn(tbs.l, __fadd_rn(tb.l.x, tb.l.y));
-            const float2 o = acc_j[jj];
-            const ff sj = two_sum(o.x, tbs.h);
-            acc_j[jj] = make_float2(sj.h, __fadd_rn(o.y, __fadd_rn(sj.l, tbl)));
-            __syncwarp();
-          }
-          __syncthreads();
-        }
-        // source-side sums of this tile pair into PJ[rg][j]
-        for (int h = 0; h < 2; ++h) {
-          const int slot = h * MT + threadIdx.x;
-          const int jl = J * MT2 + slot;
-          if (jl < nq) {
-            const float2 o = acc_j[slot];
-            PJ[(int64_t)rg * nq + jl] += (double)o.x + (double)o.y;
-          }
-        }
-        acc0 += (double)acc.h.x + (double)acc.l.x;
-        acc1 += (double)acc.h.y + (double)acc.l.y;
-      }
-    }
-    if (v0) PI[(int64_t)cg * nq + i0] = acc0;
-    if (v1) PI[(int64_t)cg * nq + i1] = acc1;
-  }
 }
 
 // out[i] = sum over c of PI[c][i] + sum over r of PJ[r][i] (fixed order)
@@ -1750,34 +1243,23 @@ int launch_bem_far(Mesh* m, Surface* s, const double* x, const double* lam, doub
   const int u_local = (x != nullptr && x == lam) ? 1 : 0;
   const double* uvec = (cd != 0.0) ? x : nullptr;
   const double* lvec = (cs != 0.0) ? lam : nullptr;
-  const bool f64 = precision == PBFB_FP64;
   if (precision == PBFB_FLOAT2) return launch_bem_far_ff(m, s, x, lam, cs, cd, kappa, y, accumulate);
+  if (precision == PBFB_FP64) {
+    double* v;
+    PB_TRY(launch_pairs(m, s, x, lam, cs * INV4PI, cd * INV4PI, kappa, true, &v));
+    return test_reduce(m, s, v, 1, y, accumulate);
+  }
   k_sources<<<blocks_for(nq, 256), 256, 0, m->stream>>>(s->nt, s->tri.p, s->vmap.p, lvec, uvec, u_local, s->qw.p,
-                                                        s->nrm.p, s->qpf.p, s->qx.p, cs * INV4PI, cd * INV4PI,
-                                                        f64 ? 1 : 0, s->spos.p, s->sdl.p, s->s64.p);
+                                                        s->nrm.p, s->qpf.p, cs * INV4PI, cd * INV4PI, s->spos.p,
+                                                        s->sdl.p);
   PB_LAUNCHED(m);
   cudaEvent_t ev;
-  KernelClassTimer& tm = f64 ? m->t_nbody64 : m->t_nbody;
+  KernelClassTimer& tm = m->t_nbody;
   timer_begin(m, tm, &ev);
   int nsplit;
   double* vals = s->val.p;
   double tree_pairs = -1.0;
-  if (f64) {
-    constexpr int NT = 128;
-    int ntb = blocks_for(nq, NT);
-    nsplit = std::max(1, std::min(blocks_for(4 * 152, ntb), blocks_for(nq, 4 * NT)));
-    int per = blocks_for(blocks_for(nq, nsplit), NT) * NT;
-    nsplit = blocks_for(nq, per);
-    dim3 grid(ntb, nsplit);
-    if ((size_t)nsplit * nq > s->val.n) {
-      set_error("far-field split buffer too small");
-      return PBFB_ERR_STATE;
-    }
-    if (yuk)
-      k_nbody_f64<NT, true><<<grid, NT, 0, m->stream>>>(nq, s->s64.p, kappa, per, s->val.p);
-    else
-      k_nbody_f64<NT, false><<<grid, NT, 0, m->stream>>>(nq, s->s64.p, kappa, per, s->val.p);
-  } else if (use_tree(m, s)) {
+  if (use_tree(m, s)) {
     PB_TRY(launch_tree_far(m, s, kappa, s->spos.p, s->sdl.p, s->val.p, &tree_pairs));
     nsplit = 1;
   } else {
@@ -1823,7 +1305,7 @@ int launch_bem_far(Mesh* m, Surface* s, const double* x, const double* lam, doub
   PB_LAUNCHED(m);
   const double pairs = tree_pairs >= 0.0 ? tree_pairs : (double)nq * (double)nq;
   timer_end(m, tm, ev, pairs);
-  if (!f64) m->nbody_flops += (yuk ? 24.0 : 18.0) * pairs;
+  m->nbody_flops += (yuk ? 24.0 : 18.0) * pairs;
   return test_reduce(m, s, vals, nsplit, y, accumulate);
 }
 
@@ -1832,54 +1314,28 @@ int launch_bem_far_ff(Mesh* m, Surface* s, const double* x, const double* lam, d
   const int nq = s->nq;
   const bool yuk = kappa != 0.0;
   const int u_local = (x != nullptr && x == lam) ? 1 : 0;
+  // by pairs of triangles; ff_kernel = 1 asks for the one-target-per-thread sum.  Lengths are scaled by kappa
+  // there: a Yukawa kernel with kappa below 1e-8 (no physical ionic strength; the scaled 1/r^3 nears the end of
+  // float32's range) takes the float64 form.
+  if (m->tune_ff_kernel != 1) {
+    double* v;
+    PB_TRY(launch_pairs(m, s, x, lam, cs * INV4PI, cd * INV4PI, kappa, kappa > 0.0 && kappa < 1e-8, &v));
+    return test_reduce(m, s, v, 1, y, accumulate);
+  }
   PB_TRY(ff_exp_table(m));
   if (s->ffsrc.n < 4 * (size_t)nq) PB_TRY(s->ffsrc.alloc(4 * (size_t)nq));
   if (s->fftgt.n < 2 * (size_t)nq) PB_TRY(s->fftgt.alloc(2 * (size_t)nq));
   k_sources_ff<<<blocks_for(nq, 256), 256, 0, m->stream>>>(
       s->nt, s->tri.p, s->vmap.p, cs != 0.0 ? lam : nullptr, cd != 0.0 ? x : nullptr, u_local, s->qw.p, s->nrm.p,
-      s->qx.p, s->ctr[0], s->ctr[1], s->ctr[2], cs * INV4PI, cd * INV4PI, s->ff_q, s->ffsrc.p, s->fftgt.p);
+      s->qx.p, s->ctr[0], s->ctr[1], s->ctr[2], cs * INV4PI, cd * INV4PI, ff_grid(s, 1.0), s->ffsrc.p, s->fftgt.p);
   PB_LAUNCHED(m);
   cudaEvent_t ev;
   timer_begin(m, m->t_nbodyff, &ev);
   constexpr int NT = 128;
-  // kernel: 1 one target per thread, 2 two targets per thread (float2), 3 mutual pairs, 4 mutual
-  // pairs with two targets per thread (float2);
-  // built-in choice: packed mutual for large surfaces (5 % faster than 3 on GB300: the float32
-  // pipe, not issue, bounds both), two targets per thread otherwise
-  const int kind = m->tune_ff_kernel > 0 ? m->tune_ff_kernel : (nq >= 16384 ? 4 : 2);
-  const int bps = m->tune_ff_bps > 0 ? m->tune_ff_bps : 8;  // GB300 sweep: 8 blocks per SM of source splits
+  const int bps = m->tune_ff_bps > 0 ? m->tune_ff_bps : 8;
   const float kh = (float)kappa, kl = (float)(kappa - (double)kh);
-  if (kind == 3 || kind == 4) {
-    // tile groups: G (G + 1) / 2 blocks, about bps blocks per SM (built-in 16: two waves, which
-    // measured faster than one full wave or fewer, larger tiles); 2 G + 1 partial rows
-    const int nT = blocks_for(nq, kind == 4 ? MT2 : MT);
-    int G = (int)std::sqrt(2.0 * (m->tune_ff_bps > 0 ? m->tune_ff_bps : 16) * 152.0);
-    G = std::max(1, std::min(G, nT));
-    PB_TRY(ensure(s->mval, (size_t)(2 * G + 1) * nq));
-    double* PI = s->mval.p;
-    double* PJ = s->mval.p + (size_t)G * nq;
-    double* out = s->mval.p + (size_t)2 * G * nq;
-    PB_CUDA(cudaMemsetAsync(s->mval.p, 0, (size_t)2 * G * nq * sizeof(double), m->stream));
-    const int nblk = G * (G + 1) / 2;
-    if (kind == 4 && yuk)
-      k_nbody_ffm2<true><<<nblk, MT, 0, m->stream>>>(nq, G, s->ffsrc.p, kh, kl, m->ff_tab.p, PI, PJ);
-    else if (kind == 4)
-      k_nbody_ffm2<false><<<nblk, MT, 0, m->stream>>>(nq, G, s->ffsrc.p, kh, kl, m->ff_tab.p, PI, PJ);
-    else if (yuk)
-      k_nbody_ffm<true><<<nblk, MT, 0, m->stream>>>(nq, G, s->ffsrc.p, kh, kl, m->ff_tab.p, PI, PJ);
-    else
-      k_nbody_ffm<false><<<nblk, MT, 0, m->stream>>>(nq, G, s->ffsrc.p, kh, kl, m->ff_tab.p, PI, PJ);
-    PB_LAUNCHED(m);
-    k_mutual_sum<<<blocks_for(nq, 256), 256, 0, m->stream>>>(nq, G, PI, PJ, out);
-    PB_LAUNCHED(m);
-    timer_end(m, m->t_nbodyff, ev, (double)nq * (double)nq);
-    return test_reduce(m, s, out, 1, y, accumulate);
-  }
-  const bool pk = kind == 2;
-  const int ntb = blocks_for(nq, pk ? 2 * NT : NT);
-  // source splits from the packed grid in both variants, so that they sum in the same order
-  const int ntb2 = blocks_for(nq, 2 * NT);
-  int nsplit = std::max(1, std::min(blocks_for(bps * 152, ntb2), blocks_for(nq, 4 * NT)));
+  const int ntb = blocks_for(nq, NT);
+  int nsplit = std::max(1, std::min(blocks_for(bps * 152, ntb), blocks_for(nq, 4 * NT)));
   const int per = blocks_for(blocks_for(nq, nsplit), NT) * NT;
   nsplit = blocks_for(nq, per);
   if ((size_t)nsplit * nq > s->val.n) {
@@ -1887,11 +1343,7 @@ int launch_bem_far_ff(Mesh* m, Surface* s, const double* x, const double* lam, d
     return PBFB_ERR_STATE;
   }
   dim3 grid(ntb, nsplit);
-  if (pk && yuk)
-    k_nbody_ff2<NT, true><<<grid, NT, 0, m->stream>>>(nq, s->fftgt.p, s->ffsrc.p, kh, kl, m->ff_tab.p, per, s->val.p);
-  else if (pk)
-    k_nbody_ff2<NT, false><<<grid, NT, 0, m->stream>>>(nq, s->fftgt.p, s->ffsrc.p, kh, kl, m->ff_tab.p, per, s->val.p);
-  else if (yuk)
+  if (yuk)
     k_nbody_ff<NT, true><<<grid, NT, 0, m->stream>>>(nq, s->fftgt.p, s->ffsrc.p, kh, kl, m->ff_tab.p, per, s->val.p);
   else
     k_nbody_ff<NT, false><<<grid, NT, 0, m->stream>>>(nq, s->fftgt.p, s->ffsrc.p, kh, kl, m->ff_tab.p, per, s->val.p);
@@ -1991,7 +1443,7 @@ int bem_apply_noalloc(Mesh* m, int which, int op, const double* x, double* y) {
   const double cs = op == 0 ? 1.0 : 0.0, cd = op == 1 ? 1.0 : 0.0;
   k_sources<<<blocks_for(nq, 256), 256, 0, m->stream>>>(s->nt, s->tri.p, s->vmap.p, cs != 0.0 ? x : nullptr,
                                                         cd != 0.0 ? x : nullptr, 1, s->qw.p, s->nrm.p, s->qpf.p,
-                                                        s->qx.p, cs * INV4PI, cd * INV4PI, 0, spos, sdl, nullptr);
+                                                        cs * INV4PI, cd * INV4PI, spos, sdl);
   PB_LAUNCHED(m);
   // The split kernels and targets per thread of pbfb_bem_apply (launch_bem_far), with its split
   // rules (whole waves of resident blocks when blocks_per_sm is 0), capped at NOALLOC_SPLITS

@@ -245,9 +245,8 @@ int build_surface(Mesh* m, Surface* s, const std::vector<int>& gtri, const std::
     for (int d = 0; d < 3; ++d) c[d] += xyz_h[3 * (size_t)v + d];
   for (int d = 0; d < 3; ++d) s->ctr[d] = c[d] / verts.size();
   {
-    // float-float coordinates: high parts on the grid 2^-k with every difference of two high
-    // parts below 2^24 steps, hence exact in float32 (quadrature points lie within the
-    // triangles, so within the largest vertex distance from the centre)
+    // largest vertex distance from the centre: the quadrature points lie within the triangles (float-float
+    // coordinates, ff_grid)
     double rmax = 0.0;
     for (int v : verts) {
       double r2 = 0.0;
@@ -257,8 +256,7 @@ int build_surface(Mesh* m, Surface* s, const std::vector<int>& gtri, const std::
       }
       rmax = std::max(rmax, std::sqrt(r2));
     }
-    const int k = (int)std::floor(24.0 - std::log2(2.0 * rmax * 1.01 + 1e-300)) - 1;
-    s->ff_q = std::ldexp(1.0, -k);
+    s->rmax = rmax;
   }
   s->nt = nt;
   s->nv = (int)verts.size();
@@ -355,7 +353,6 @@ int build_surface(Mesh* m, Surface* s, const std::vector<int>& gtri, const std::
   PB_TRY(s->diagV.alloc(s->nv));
   PB_TRY(s->spos.alloc(s->nq));
   PB_TRY(s->sdl.alloc(s->nq));
-  PB_TRY(s->s64.alloc(7 * (size_t)s->nq));
   // far-field partial-sum buffer: enough source splits for every launch shape of launch_bem_far
   PB_TRY(s->val.alloc(far_splits_max(s->nq) * (size_t)s->nq));
   return PBFB_OK;
@@ -690,6 +687,7 @@ int mesh_create(const double* xyz, int nv, const int* tets, int64_t nt, const in
   }
   PB_TRY(init_quadrature());
   PB_TRY(init_dense_attributes());
+  PB_TRY(init_pair_attributes());
   Mesh* m = new Mesh();
   int st = PBFB_OK;
   auto fail = [&](int s) {

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <cmath>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -112,7 +113,7 @@ struct Surface {
   DBuf<double> area;        // nt
   DBuf<float4> qpf;         // nq float (x, y, z, 0) relative to ctr
   double ctr[3] = {0, 0, 0};
-  double ff_q = 0.0;            // grid of the float-float coordinates' high parts (a power of 2)
+  double rmax = 0.0;            // largest vertex distance from ctr
   // test reduction: per vertex list of (tri*3 + a)
   DBuf<int> inc_ptr, inc_idx;
   // special pairs
@@ -132,11 +133,15 @@ struct Surface {
   bool built = false;
   // far-field work buffers
   DBuf<float4> spos, sdl;       // float32 sources
-  DBuf<double> s64;             // float64 sources: 7 * nq (x, y, z, s, mx, my, mz)
   DBuf<double> val;             // nsplit * nq target potentials
   DBuf<float4> ffsrc, fftgt;    // float-float sources (4 float4) and targets (2 float4) per point
   int nsplit = 1;
-  DBuf<double> mval;            // mutual float32 far field: 2 G partial rows + the sum
+  DBuf<double> mval;            // mutual far fields: partial rows + the sum
+  // tile layouts of the far fields by triangle pairs (bem_pairs.cu): geometry (float-float, for lengths
+  // scaled by pgeo_scale; float64) and strengths
+  DBuf<float> pgeo, psrc;
+  DBuf<double> pgeo64, psrc64;
+  double pgeo_scale = 0.0;
   SurfaceTree tree;             // treecode plan of the float32 far field (built on first use)
   // dense single layer (float32, ld x ld): -V^-1 once inverted (bem_dense.cu)
   DBuf<float> vinv;
@@ -224,9 +229,8 @@ struct Mesh {
   int tune_tpt = 0;                 // float32 far field: targets per thread (0 = heuristic)
   int tune_bps = 0;                 // float32 far field: target blocks per SM for the source split
   int tune_packed = 0;              // float32 far field: 1 = packed f32x2 kernel
-  int tune_ff_kernel = 0;           // float-float far field: 1 one target per thread, 2 two (float2),
-                                    // 3 mutual pairs (0 = mutual for large surfaces, else 2)
-  int tune_ff_bps = 0;              // float-float far field: target blocks per SM (0 = built-in)
+  int tune_ff_kernel = 0;           // float-float far field: 1 one target per thread, else pairs of triangles
+  int tune_ff_bps = 0;              // float-float far field: tasks / 8 (blocks for kernel 1) per SM (0 = built-in)
   int tune_tree = 0;                // float32 far field: 0 built-in (treecode from TREE_MIN_POINTS
                                     // points), 1 direct sum, 2 treecode
   int spmv_lanes = 0;               // lanes per row of the operator's sparse part (0 = 8; 4, 8, 16)
@@ -249,6 +253,8 @@ struct Mesh {
   bool timing = false;
   KernelClassTimer t_nbody, t_nbody64, t_nbodyff, t_spmv, t_elem, t_dense;
   DBuf<float2> ff_tab;      // float-float exp table of the Yukawa kernel
+  DBuf<float2> pair_tab;    // float-float exp tables of the far field by triangle pairs
+  DBuf<double> pair_tab64;  // its float64 table of 2^-k/2048
   DBuf<float4> fx_tab;      // float-float exp / sinh / cosh (j/32) tables of the element kernels
   double nbody_flops = 0.0;  // float32 far-field flops issued (18 per Laplace pair, 24 per Yukawa pair)
   double setup_ms[4] = {0, 0, 0, 0};  // mesh_create: validation, surfaces, operator pattern, device set-up
@@ -336,6 +342,26 @@ int launch_coulomb(Mesh* m);
 // reaction potentials of x_L and x_NL at the charges: ur_dev[0, nq) and ur_dev[nq, 2 nq)
 int launch_reaction_potentials(Mesh* m, const double* xL, const double* xNL, double* ur_dev);
 int bem_apply_noalloc(Mesh* m, int which, int op, const double* x, double* y);
+
+// Grid of the float-float coordinates' high parts for lengths scaled by `scale` (a power of 2): differences
+// of two of them are below 2^24 steps, hence exact in float32.  Low parts lie on its 2^-25th part, within half
+// a step, so that they are float32 numbers and most differences of two of them are exact too: the pair
+// arithmetic then sees the same (rounded) points in every pair.
+inline double ff_grid(const Surface* s, double scale) {
+  return std::ldexp(1.0, -(int)std::floor(24.0 - std::log2(2.0 * s->rmax * scale * 1.01 + 1e-300)));
+}
+
+// ---- bem_pairs.cu: far fields of the accurate precisions by pairs of triangles
+struct PairSplit {
+  int nT, tpg, G, K, nsub, ntask;  // tiles, tiles per group, groups, step parts, point shares, tasks
+  size_t rows;                     // rows of partial sums
+};
+void pair_split(int nt, int want, bool f64, PairSplit* S);
+size_t pair_work(int64_t nt);
+// far-field potentials at the quadrature points (float64 if f64, else float-float); *val: device, nq
+int launch_pairs(Mesh* m, Surface* s, const double* x, const double* lam, double cs, double cd, double kappa, bool f64,
+                 double** val);
+int init_pair_attributes();
 
 // ---- treecode.cu: hierarchical float32 far field
 constexpr int TREE_MIN_POINTS = 65536;  // built-in: treecode for surfaces of at least this many points
