@@ -8,7 +8,7 @@
 // points of the surface (an N-body sum, coincident points excluded) and reduces the
 // target potentials against the test functions.  Touching and close triangle pairs
 // are corrected by a precomputed sparse matrix holding, per P1 pair (i, j), the
-// difference between the accurate rule of the pair's class and the 6 x 6 rule:
+// difference between the accurate rule of the pair's class and the 6 x 6 rule (bem_corrections.cu):
 //   identical / common edge / common vertex: Sauter-Schwab (Sauter & Schwab,
 //     Boundary Element Methods, 2011, Sec. 5.2), 5 Gauss-Legendre points per variable;
 //   near (no shared vertex, centroid distance < 2 max(h_tau, h_sigma)): 6 points on
@@ -29,46 +29,7 @@ namespace pbfb {
 
 namespace {
 
-constexpr int NGL = 5;       // Gauss-Legendre points per Sauter-Schwab variable
-constexpr int NSUB = 96;     // 16 sub-triangles x 6 points
 constexpr double INV4PI = 0.079577471545947667884;
-
-__constant__ double c_gl_x[NGL];
-__constant__ double c_gl_w[NGL];
-__constant__ double c_sub_b[NSUB][3];
-__constant__ double c_sub_w[NSUB];
-
-// Gauss-Legendre nodes on [-1, 1] by Newton's method on the three-term recurrence of
-// P_n, mapped to [0, 1].
-void gauss_legendre01(int n, double* x01, double* w01) {
-  for (int i = 0; i < n; ++i) {
-    double z = std::cos(M_PI * (i + 0.75) / (n + 0.5));
-    double pp = 0.0;
-    for (int it = 0; it < 100; ++it) {
-      double p0 = 1.0, p1 = z;
-      for (int k = 2; k <= n; ++k) {
-        double p2 = ((2.0 * k - 1.0) * z * p1 - (k - 1.0) * p0) / k;
-        p0 = p1;
-        p1 = p2;
-      }
-      pp = n * (z * p1 - p0) / (z * z - 1.0);
-      double dz = p1 / pp;
-      z -= dz;
-      if (std::fabs(dz) < 1e-16) break;
-    }
-    {
-      double p0 = 1.0, p1 = z;
-      for (int k = 2; k <= n; ++k) {
-        double p2 = ((2.0 * k - 1.0) * z * p1 - (k - 1.0) * p0) / k;
-        p0 = p1;
-        p1 = p2;
-      }
-      pp = n * (z * p1 - p0) / (z * z - 1.0);
-    }
-    x01[i] = 0.5 * (1.0 - z);
-    w01[i] = 1.0 / ((1.0 - z * z) * pp * pp);  // (2 / ((1 - z^2) P'^2)) / 2
-  }
-}
 
 // ---------------------------------------------------------------- geometry
 
@@ -106,208 +67,9 @@ __global__ void k_surface_geometry(const double* __restrict__ xyz, int nvtot, co
   }
 }
 
-// ---------------------------------------------------------------- near-field corrections
-
-struct PairKer {
-  double kappa;
-  __device__ __forceinline__ void eval(const double* x, const double* y, const double* n, double& g,
-                                       double& dl) const {
-    double d0 = x[0] - y[0], d1 = x[1] - y[1], d2 = x[2] - y[2];
-    double r2 = d0 * d0 + d1 * d1 + d2 * d2;
-    double r = sqrt(r2);
-    double e = exp(-kappa * r);
-    g = e * INV4PI / r;
-    dl = (n[0] * d0 + n[1] * d1 + n[2] * d2) * (1.0 + kappa * r) * e * INV4PI / (r2 * r);
-  }
-};
-
-// Sauter-Schwab reference points of region `reg` for class `cls` at (xi, e1, e2, e3):
-// returns the two points (s1, s2) in {0 <= s2 <= s1 <= 1} and the Jacobian of the map.
-__device__ __forceinline__ double ss_point(int cls, int reg, double xi, double e1, double e2, double e3,
-                                           double& x1, double& x2, double& y1, double& y2) {
-  if (cls == PAIR_IDENTICAL) {
-    double a1, a2, b1, b2;
-    int base = reg >> 1;
-    if (base == 0) {
-      a1 = xi; a2 = xi * (1.0 - e1 + e1 * e2);
-      b1 = xi * (1.0 - e1 * e2 * e3); b2 = xi * (1.0 - e1);
-    } else if (base == 1) {
-      a1 = xi; a2 = xi * e1 * (1.0 - e2 + e2 * e3);
-      b1 = xi * (1.0 - e1 * e2); b2 = xi * e1 * (1.0 - e2);
-    } else {
-      a1 = xi * (1.0 - e1 * e2 * e3); a2 = xi * e1 * (1.0 - e2 * e3);
-      b1 = xi; b2 = xi * e1 * (1.0 - e2);
-    }
-    if (reg & 1) { x1 = b1; x2 = b2; y1 = a1; y2 = a2; }
-    else { x1 = a1; x2 = a2; y1 = b1; y2 = b2; }
-    return xi * xi * xi * e1 * e1 * e2;
-  }
-  if (cls == PAIR_EDGE) {
-    double j = xi * xi * xi * e1 * e1;
-    switch (reg) {
-      case 0:
-        x1 = xi; x2 = xi * e1 * e3; y1 = xi * (1.0 - e1 * e2); y2 = xi * e1 * (1.0 - e2);
-        return j;
-      case 1:
-        x1 = xi; x2 = xi * e1; y1 = xi * (1.0 - e1 * e2 * e3); y2 = xi * e1 * e2 * (1.0 - e3);
-        return j * e2;
-      case 2:
-        x1 = xi * (1.0 - e1 * e2); x2 = xi * e1 * (1.0 - e2); y1 = xi; y2 = xi * e1 * e2 * e3;
-        return j * e2;
-      case 3:
-        x1 = xi * (1.0 - e1 * e2 * e3); x2 = xi * e1 * e2 * (1.0 - e3); y1 = xi; y2 = xi * e1;
-        return j * e2;
-      default:
-        x1 = xi * (1.0 - e1 * e2 * e3); x2 = xi * e1 * (1.0 - e2 * e3); y1 = xi; y2 = xi * e1 * e2;
-        return j * e2;
-    }
-  }
-  // common vertex
-  if (reg == 0) { x1 = xi; x2 = xi * e1; y1 = xi * e2; y2 = xi * e2 * e3; }
-  else { x1 = xi * e2; x2 = xi * e2 * e3; y1 = xi; y2 = xi * e1; }
-  return xi * xi * xi * e2;
-}
-
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
-}
-
-// One warp per special pair.  Outputs, per pair, 9 entries in stored local vertex
-// order (a of the test triangle, b of the trial one):
-//   corrV/corrK = accurate rule - 6x6 rule (coincident points excluded),
-//   fullV = accurate single-layer value (for the operator diagonal),
-//   mass = P1 mass entries (identical pairs only).
-__global__ void k_pair_corrections(int npair, const int* __restrict__ pt_, const int* __restrict__ ps_,
-                                   const int* __restrict__ cls_, const int* __restrict__ perm_,
-                                   const int* __restrict__ tri, const int* __restrict__ vmap,
-                                   const double* __restrict__ xyz, int nvtot, const double* __restrict__ nrm,
-                                   const double* __restrict__ area, const double* __restrict__ qx,
-                                   const double* __restrict__ qw, int nt, double kappa,
-                                   double* __restrict__ corrV, double* __restrict__ corrK,
-                                   double* __restrict__ fullV, double* __restrict__ mass) {
-  int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
-  if (warp >= npair) return;
-  const int t = pt_[warp], s = ps_[warp], cls = cls_[warp];
-  int pt[3], ps[3];
-  for (int a = 0; a < 3; ++a) {
-    pt[a] = perm_[6 * warp + a];
-    ps[a] = perm_[6 * warp + 3 + a];
-  }
-  double Pt[3][3], Ps[3][3];  // corners in rule order
-  for (int a = 0; a < 3; ++a) {
-    int vt = vmap[tri[3 * t + pt[a]]], vs = vmap[tri[3 * s + ps[a]]];
-    for (int d = 0; d < 3; ++d) {
-      Pt[a][d] = xyz[d * nvtot + vt];
-      Ps[a][d] = xyz[d * nvtot + vs];
-    }
-  }
-  double ns[3] = {nrm[s], nrm[nt + s], nrm[2 * nt + s]};
-  double At = area[t], As = area[s];
-  PairKer K{kappa};
-  double SL[9], DL[9];
-  for (int k = 0; k < 9; ++k) SL[k] = DL[k] = 0.0;
-  if (cls != PAIR_NEAR) {
-    int nreg = cls == PAIR_IDENTICAL ? 6 : (cls == PAIR_EDGE ? 5 : 2);
-    int npts = nreg * NGL * NGL * NGL * NGL;
-    for (int k = lane; k < npts; k += 32) {
-      int reg = k / (NGL * NGL * NGL * NGL);
-      int i = k - reg * (NGL * NGL * NGL * NGL);
-      int i0 = i / (NGL * NGL * NGL), i1 = (i / (NGL * NGL)) % NGL, i2 = (i / NGL) % NGL, i3 = i % NGL;
-      double x1, x2, y1, y2;
-      double jac = ss_point(cls, reg, c_gl_x[i0], c_gl_x[i1], c_gl_x[i2], c_gl_x[i3], x1, x2, y1, y2);
-      double W = jac * c_gl_w[i0] * c_gl_w[i1] * c_gl_w[i2] * c_gl_w[i3];
-      double bx[3] = {1.0 - x1, x1 - x2, x2}, by[3] = {1.0 - y1, y1 - y2, y2};
-      double X[3], Y[3];
-      for (int d = 0; d < 3; ++d) {
-        X[d] = bx[0] * Pt[0][d] + bx[1] * Pt[1][d] + bx[2] * Pt[2][d];
-        Y[d] = by[0] * Ps[0][d] + by[1] * Ps[1][d] + by[2] * Ps[2][d];
-      }
-      double g, dl;
-      K.eval(X, Y, ns, g, dl);
-      g *= W;
-      dl *= W;
-      for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) {
-          SL[3 * a + b] += g * bx[a] * by[b];
-          DL[3 * a + b] += dl * bx[a] * by[b];
-        }
-    }
-    double jac = 4.0 * At * As;
-    for (int k = 0; k < 9; ++k) {
-      SL[k] *= jac;
-      DL[k] *= jac;
-    }
-  } else {
-    for (int k = lane; k < QS * NSUB; k += 32) {
-      int q = k / NSUB, p = k - q * NSUB;
-      double X[3], Y[3];
-      for (int d = 0; d < 3; ++d) {
-        X[d] = c_tri_b[q][0] * Pt[0][d] + c_tri_b[q][1] * Pt[1][d] + c_tri_b[q][2] * Pt[2][d];
-        Y[d] = c_sub_b[p][0] * Ps[0][d] + c_sub_b[p][1] * Ps[1][d] + c_sub_b[p][2] * Ps[2][d];
-      }
-      double g, dl;
-      K.eval(X, Y, ns, g, dl);
-      double W = c_tri_w[q] * c_sub_w[p] * At * As;
-      g *= W;
-      dl *= W;
-      for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) {
-          SL[3 * a + b] += g * c_tri_b[q][a] * c_sub_b[p][b];
-          DL[3 * a + b] += dl * c_tri_b[q][a] * c_sub_b[p][b];
-        }
-    }
-  }
-  // 6 x 6 rule in stored order (what the far-field sum adds), coincident points excluded
-  double RS[9], RD[9];
-  for (int k = 0; k < 9; ++k) RS[k] = RD[k] = 0.0;
-  int nqt = QS * nt;
-  for (int k = lane; k < QS * QS; k += 32) {
-    int q = k / QS, p = k - q * QS;
-    if (t == s && q == p) continue;
-    double X[3], Y[3];
-    for (int d = 0; d < 3; ++d) {
-      X[d] = qx[d * nqt + QS * t + q];
-      Y[d] = qx[d * nqt + QS * s + p];
-    }
-    double g, dl;
-    K.eval(X, Y, ns, g, dl);
-    // the far field's plane distance: from the trial triangle's first point, 0 within a triangle
-    {
-      const double d0 = X[0] - Y[0], d1 = X[1] - Y[1], d2 = X[2] - Y[2];
-      const double r2 = d0 * d0 + d1 * d1 + d2 * d2, r = sqrt(r2);
-      const double D = t == s ? 0.0
-                              : fma(ns[2], X[2] - qx[2 * nqt + QS * s],
-                                    fma(ns[1], X[1] - qx[nqt + QS * s], ns[0] * (X[0] - qx[QS * s])));
-      dl = D * (1.0 + kappa * r) * g / r2;
-    }
-    double W = qw[QS * t + q] * qw[QS * s + p];
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b) {
-        RS[3 * a + b] += W * g * c_tri_b[q][a] * c_tri_b[p][b];
-        RD[3 * a + b] += W * dl * c_tri_b[q][a] * c_tri_b[p][b];
-      }
-  }
-  for (int k = 0; k < 9; ++k) {
-    SL[k] = warp_sum(SL[k]);
-    DL[k] = warp_sum(DL[k]);
-    RS[k] = warp_sum(RS[k]);
-    RD[k] = warp_sum(RD[k]);
-  }
-  if (lane == 0) {
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b) {
-        int o = 9 * warp + 3 * pt[a] + ps[b];  // rule order -> stored order
-        int r = 3 * a + b;
-        fullV[o] = SL[r];
-        corrV[o] = SL[r] - RS[3 * pt[a] + ps[b]];
-        corrK[o] = DL[r] - RD[3 * pt[a] + ps[b]];
-      }
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b)
-        mass[9 * warp + 3 * a + b] = (cls == PAIR_IDENTICAL) ? At * (a == b ? 2.0 : 1.0) / 12.0 : 0.0;
-  }
 }
 
 // ---------------------------------------------------------------- far field
@@ -1068,40 +830,7 @@ int init_quadrature() {
   static bool done = false;
   std::lock_guard<std::mutex> lk(mu);
   if (done) return PBFB_OK;
-  double x[NGL], w[NGL];
-  gauss_legendre01(NGL, x, w);
-  PB_CUDA(cudaMemcpyToSymbol(c_gl_x, x, sizeof(x)));
-  PB_CUDA(cudaMemcpyToSymbol(c_gl_w, w, sizeof(w)));
-  // 6-point rule on the 16 congruent sub-triangles of the 4-fold uniform refinement
-  double sb[NSUB][3], sw[NSUB];
-  int k = 0;
-  const int m = 4;
-  for (int i = 0; i < m; ++i)
-    for (int j = 0; j < m - i; ++j) {
-      int cnt = (i + j < m - 1) ? 2 : 1;
-      for (int up = 0; up < cnt; ++up) {
-        int li[3][2];
-        if (up == 0) {
-          li[0][0] = i; li[0][1] = j; li[1][0] = i + 1; li[1][1] = j; li[2][0] = i; li[2][1] = j + 1;
-        } else {
-          li[0][0] = i + 1; li[0][1] = j; li[1][0] = i + 1; li[1][1] = j + 1; li[2][0] = i; li[2][1] = j + 1;
-        }
-        double cb[3][3];
-        for (int c = 0; c < 3; ++c) {
-          cb[c][0] = 1.0 - (li[c][0] + li[c][1]) / (double)m;
-          cb[c][1] = li[c][0] / (double)m;
-          cb[c][2] = li[c][1] / (double)m;
-        }
-        for (int q = 0; q < QS; ++q) {
-          for (int d = 0; d < 3; ++d)
-            sb[k][d] = h_tri_b[q][0] * cb[0][d] + h_tri_b[q][1] * cb[1][d] + h_tri_b[q][2] * cb[2][d];
-          sw[k] = h_tri_w[q] / (m * m);
-          ++k;
-        }
-      }
-    }
-  PB_CUDA(cudaMemcpyToSymbol(c_sub_b, sb, sizeof(sb)));
-  PB_CUDA(cudaMemcpyToSymbol(c_sub_w, sw, sizeof(sw)));
+  PB_TRY(init_correction_rules());
   // float-float exp tables: exp(-k0 / 256), k0 < 16 (constant memory)
   float2 lo[16];
   for (int k = 0; k < 16; ++k) {
@@ -1144,23 +873,6 @@ int launch_surface_geometry(Mesh* m, Surface* s) {
       m->xyz.p, m->nv, s->tri.p, s->vmap.p, s->nt, s->ctr[0], s->ctr[1], s->ctr[2], s->qx.p, s->qw.p, s->nrm.p,
       s->area.p, s->qpf.p);
   PB_LAUNCHED(m);
-  return PBFB_OK;
-}
-
-int launch_pair_corrections(Mesh* m, Surface* s, double kappa) {
-  if (s->npair == 0) return PBFB_OK;
-  int threads = 128;
-  int blocks = blocks_for((int64_t)s->npair * 32, threads);
-  k_pair_corrections<<<blocks, threads, 0, m->stream>>>(
-      s->npair, s->pair_t.p, s->pair_s.p, s->pair_cls.p, s->pair_perm.p, s->tri.p, s->vmap.p, m->xyz.p, m->nv,
-      s->nrm.p, s->area.p, s->qx.p, s->qw.p, s->nt, kappa, s->pairV.p, s->pairK.p, s->pairVfull.p,
-      m->red2.p);
-  PB_LAUNCHED(m);
-  // per-slot sums (fixed order): corrections, mass, V diagonal
-  PB_TRY(launch_gather(m, s->cnnz, s->cg_ptr.p, s->cg_idx.p, s->pairV.p, nullptr, 1.0, s->corrV.p));
-  PB_TRY(launch_gather(m, s->cnnz, s->cg_ptr.p, s->cg_idx.p, s->pairK.p, nullptr, 1.0, s->corrK.p));
-  PB_TRY(launch_gather(m, s->cnnz, s->cg_ptr.p, s->cg_idx.p, m->red2.p, nullptr, 1.0, s->mass.p));
-  PB_TRY(launch_gather(m, s->nv, s->dg_ptr.p, s->dg_idx.p, s->pairVfull.p, nullptr, 1.0, s->diagV.p));
   return PBFB_OK;
 }
 

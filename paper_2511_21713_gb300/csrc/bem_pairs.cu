@@ -35,6 +35,7 @@
 #include <vector>
 
 #include "f32x2.cuh"
+#include "fp64_math.cuh"
 #include "pbfb_internal.cuh"
 #include "quad_tables.cuh"
 
@@ -50,7 +51,6 @@ constexpr int D_GEO = 21;            // float64 rows: 18 coordinates, 3 normals
 constexpr int D_SRC = 12;            // s, mu
 constexpr int FF_HI = 657;           // exp(-k / 16): arguments are cut at 41, entries from 640 (x = 40) are 0
 constexpr int FF_LO = 64;            // exp(-k / 1024)
-constexpr int D_TAB = 2048;          // 2^(-k / 2048)
 
 // ---- float-float on pairs of float32 (per component the scalar operations' rounding)
 __device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
@@ -370,35 +370,6 @@ __global__ void __launch_bounds__(32 * PW, NP == 3 ? 3 : 4)
 
 // ---- float64
 
-// 1/sqrt(r2): the hardware's estimate y0 (about 2^-20), e = 1 - r2 y0^2, y0 (1 + e/2 + 3 e^2/8); the
-// next term of the series, 5 e^3/16, is below 2^-60
-__device__ __forceinline__ double rsqrt64(double r2) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
-  const double e = fma(-(r2 * y), y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
-// 2^-x for 0 <= x: 2^-x = 2^-m T[j] 2^-f, x = m + j / 2048 + f with |f| <= 2^-12 (k = 2048 m + j from the
-// float32 value of x, the float64 remainder exact), 2^-f = 1 + f (-L + f (L^2/2 - f L^3/6)), L = ln 2
-// (truncation 2^-54).  0 once 2^-m leaves the normal numbers.
-__device__ __forceinline__ double exp2_neg(double x, const double* __restrict__ tab) {
-  // float32 bits of x cut to [2^-60, 1100] (exponent bias 1023 -> 127 modulo 2^32)
-  const int xhi = min(max(__double2hiint(x), 0x3C300000), 0x40913000);
-  const unsigned xb = __funnelshift_l(__double2loint(x), xhi, 3) - 0xC0000000u;
-  const float m = __fmaf_rn(__uint_as_float(xb), 2048.f, 12582912.f);
-  const int k = __float_as_int(m) - 0x4B400000;
-  const float kf = __fmul_rn(__fsub_rn(m, 12582912.f), 1.f / 2048.f);
-  const int kb = __float_as_int(kf);
-  // kf as a float64 number (0 becomes 2^-127: far below any rounding here)
-  double f = x - __hiloint2double((kb >> 3) + (896 << 20), kb << 29);
-  double T = tab[k & (D_TAB - 1)];
-  const int e = k / D_TAB;
-  T = __hiloint2double(__double2hiint(T) - (e << 20), __double2loint(T));
-  if (e > 1020) T = f = 0.0;
-  constexpr double L = 0.69314718055994530942;
-  return fma(T * f, fma(f, fma(f, -L * L * L / 6.0, 0.5 * L * L), -L), T);
-}
-
 template <bool YUK>
 __global__ void __launch_bounds__(32 * PW, 2)
     k_pairs_f64(int nt, int ntask, int nT, int tpg, int G, int K, const double* __restrict__ geo,
@@ -406,9 +377,9 @@ __global__ void __launch_bounds__(32 * PW, 2)
                 double* PI, double* PJ) {
   extern __shared__ double smem[];
   double* s_tab = smem;  // 2^(-k / 2048) (Yukawa)
-  double* s_warp = smem + (YUK ? D_TAB : 0);
+  double* s_warp = smem + (YUK ? EXP2_TAB : 0);
   if (YUK) {
-    for (int k = threadIdx.x; k < D_TAB; k += 32 * PW) s_tab[k] = tab[k];
+    for (int k = threadIdx.x; k < EXP2_TAB; k += 32 * PW) s_tab[k] = tab[k];
     __syncthreads();
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -613,12 +584,14 @@ __global__ void k_pairs_src(int nt, int nT, const int* __restrict__ tri, const i
 
 inline int blocks_for(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
+}  // namespace
+
 // exp(-k / 16) and exp(-k / 1024) as float-float pairs, 2^(-k / 2048) in float64 (host-computed, once per mesh)
 int pair_tables(Mesh* m, bool f64) {
   if (f64) {
     if (m->pair_tab64.n) return PBFB_OK;
-    std::vector<double> t(D_TAB);
-    for (int k = 0; k < D_TAB; ++k) t[k] = std::exp2(-k / (double)D_TAB);
+    std::vector<double> t(EXP2_TAB);
+    for (int k = 0; k < EXP2_TAB; ++k) t[k] = std::exp2(-k / (double)EXP2_TAB);
     return m->pair_tab64.upload(t.data(), t.size(), m->stream);
   }
   if (m->pair_tab.n) return PBFB_OK;
@@ -630,8 +603,6 @@ int pair_tables(Mesh* m, bool f64) {
   }
   return m->pair_tab.upload(t.data(), t.size(), m->stream);
 }
-
-}  // namespace
 
 // Split of a surface's tile pairs into tasks: G groups of tpg tiles, K parts of the 32 steps, and nsub
 // shares of a triangle's points (3: a packed pair per lane; 1: all six).  One tile per group while that
@@ -716,7 +687,7 @@ int launch_pairs(Mesh* m, Surface* s, const double* x, const double* lam, double
   KernelClassTimer& tm = f64 ? m->t_nbody64 : m->t_nbodyff;
   timer_begin(m, tm, &ev);
   if (f64) {
-    const int smem = ((yuk ? D_TAB : 0) + PW * (D_GEO + D_SRC + QS) * PT) * (int)sizeof(double);
+    const int smem = ((yuk ? EXP2_TAB : 0) + PW * (D_GEO + D_SRC + QS) * PT) * (int)sizeof(double);
     const void* fn = yuk ? (const void*)k_pairs_f64<true> : (const void*)k_pairs_f64<false>;
     int a_nt = nt, a_task = S.ntask, a_nT = nT, a_tpg = S.tpg, a_G = S.G, a_K = S.K;
     double a_kap = kappa;
@@ -740,7 +711,7 @@ int launch_pairs(Mesh* m, Surface* s, const double* x, const double* lam, double
 
 // Shared-memory limits of the float64 form, once per device (called by mesh creation, before any launch)
 int init_pair_attributes() {
-  const int smem = (D_TAB + PW * (D_GEO + D_SRC + QS) * PT) * (int)sizeof(double);
+  const int smem = (EXP2_TAB + PW * (D_GEO + D_SRC + QS) * PT) * (int)sizeof(double);
   for (const void* f : {(const void*)k_pairs_f64<true>, (const void*)k_pairs_f64<false>})
     PB_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   return PBFB_OK;

@@ -333,7 +333,6 @@ int launch_csr_spmv(Mesh* m, int nrows, const int* ptr, const int* col, const do
 int launch_surface_geometry(Mesh* m, Surface* s);
 // test reduction of far-field partials (sums the source splits in place, then reduces per vertex)
 int test_reduce(Mesh* m, Surface* s, double* val, int nsplit, double* y, bool accumulate);
-int launch_pair_corrections(Mesh* m, Surface* s, double kappa);
 int launch_bem_far(Mesh* m, Surface* s, const double* x, const double* lam, double cs, double cd,
                    double kappa, int precision, double* y, bool accumulate);
 int launch_bem_far_ff(Mesh* m, Surface* s, const double* x, const double* lam, double cs, double cd,
@@ -362,6 +361,11 @@ size_t pair_work(int64_t nt);
 int launch_pairs(Mesh* m, Surface* s, const double* x, const double* lam, double cs, double cd, double kappa, bool f64,
                  double** val);
 int init_pair_attributes();
+int pair_tables(Mesh* m, bool f64);  // exponential tables, once per mesh
+
+// ---- bem_corrections.cu
+int init_correction_rules();
+int launch_pair_corrections(Mesh* m, Surface* s, double kappa);
 
 // ---- treecode.cu: hierarchical float32 far field
 constexpr int TREE_MIN_POINTS = 65536;  // built-in: treecode for surfaces of at least this many points

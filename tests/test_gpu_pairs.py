@@ -67,3 +67,23 @@ def test_yukawa_range(kappa):
         assert np.isfinite(a).all() and np.isfinite(b).all()
         assert np.abs(a - b).max() <= TOL * np.abs(b).max(), (kappa, op)
     m.close()
+
+
+# the near-field rules (every pair class) with a kernel of almost no decay, of ordinary decay, and one that
+# decays within a triangle (kappa h = 20); the float64 parity bound of the boundary operators, 1e-11
+@pytest.mark.parametrize("kappa", [1e-9, 0.2, 8.0])
+def test_corrections_over_kappa(kappa):
+    import torch
+    from oracle import bem
+    from paper_2511_21713_gb300 import inputs, pbfb
+    case = inputs.sphere_case(nu=3, a=4.0, R=6.0, layers=1, kappa=kappa)
+    V, K = bem.assemble(bem.Surface(case.xyz, case.gs_tris), kappa)
+    m = pbfb.Mesh.from_case(case)
+    m.set_params(case.eps_in, case.eps_out, kappa, case.T, pbfb.FP64)
+    x = np.random.default_rng(5).standard_normal(m.n_s)
+    for op, A in ((0, V), (1, K)):
+        y = torch.zeros(m.n_s, dtype=torch.float64, device="cuda")
+        m.bem_apply(pbfb.GAMMA_S, op, torch.as_tensor(x, device="cuda"), y)
+        ref = A @ x
+        assert np.abs(y.cpu().numpy() - ref).max() <= 1e-11 * np.abs(ref).max(), (kappa, op)
+    m.close()
