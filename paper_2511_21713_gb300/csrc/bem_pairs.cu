@@ -23,7 +23,7 @@
 //
 // Measured on GB300 (one operator product, Laplace and Yukawa surface): float-float, 8000 triangles a
 // surface, 7.58 + 11.12 ms for mutual pairs of points with a dipole vector each (97.7 and 145.7 float32 lane
-// operations per ordered pair) to 4.4 + 6.3 ms (58 and 82 counted in the source; three quarters of the float32
+// operations per ordered pair) to 3.9 + 5.7 ms (58 and 82 counted in the source; 82 to 86 % of the float32
 // pipes' rate); float64, 3380 triangles, 14.9 + 33.6 ms one-directionally with the library's root and
 // exponential to 7.0 + 11.6 ms (9.3 and 13.3 float64 operations per ordered pair, four fifths of the
 // float64 pipe's rate).  Errors of V and K against 64 bits: float64 unchanged (7e-16 to 1.7e-15), float-float
@@ -201,7 +201,7 @@ __device__ __forceinline__ PairTask pair_task(int task, int nT, int tpg, int G, 
 }
 
 template <bool YUK, int NP>
-__global__ void __launch_bounds__(32 * PW, NP == 3 ? 3 : 4)
+__global__ void __launch_bounds__(32 * PW, NP == 3 ? 2 : 3)
     k_pairs_ff(int nt, int ntask, int nT, int tpg, int G, int K, const float* __restrict__ geo,
                const float* __restrict__ src, const float2* __restrict__ tab, double* PI,
                double* PJ) {
@@ -274,8 +274,11 @@ __global__ void __launch_bounds__(32 * PW, NP == 3 ? 3 : 4)
         const float* tb = tile + b;
         const bool own = dg && k == 0;  // the lane's own triangle
         Ff<float2> S[NP], H[NP], Db[NP];
-        // not unrolled: 6 copies of the pair arithmetic would not fit the instruction cache
-#pragma unroll 1
+        // Unrolled as far as the instruction cache allows (the Yukawa pair is half as long again), with registers
+        // for two blocks an SM: the longer run of independent pairs fills the float32 pipes better than a
+        // third block.  8000 triangles, Laplace / Yukawa: not unrolled, three blocks 4.60 / 6.40 ms; 2, three
+        // 4.36 / 6.06; 2, two 4.25 / 5.86; 3, two 4.14 / 5.78; 6, two 3.99 / 6.98.
+#pragma unroll (YUK ? 3 : 6)
         for (int q = 0; q < QS; ++q) {
           float bh[3], bl[3];
 #pragma unroll
