@@ -24,6 +24,7 @@
 #include <cstdint>
 #include <mutex>
 
+#include "f32x2.cuh"
 #include "pbfb_internal.cuh"
 #include "quad_tables.cuh"
 
@@ -31,79 +32,135 @@ namespace pbfb {
 
 namespace {
 
-constexpr double INV4PI = 0.079577471545947667884;
-constexpr int DW_T = 128;          // source vertices (threads) per block of the W kernel
-constexpr int DW_A = 8;            // target points per block of the W kernel
+constexpr int DW_T = 2;            // test triangles per block of the row kernel
+constexpr int DW_S = 1536;         // trial triangles at a time
+constexpr int DW_NT = 384;         // its threads
+constexpr int DW_SMEM = 9 * DW_T * DW_S * (int)sizeof(float);
 constexpr int SW_B = 64;           // sweep pivot block
 constexpr int SW_TILE = 128;       // update tile (and ld granularity)
 constexpr size_t DENSE_W_BYTES = size_t(256) << 20;  // float32 work matrix W, per chunk
 
-// W[a - a0][j] = sum over points b of the triangles around vertex j (b != a) of
-//   w_b psi_j(y_b) g(x_a, y_b)
-// for targets a in [a0, a0 + na).  Threads run over j; each block holds DW_A targets.
+// Rows (tau, a) of W = Pt^T G P for the triangles tau in [t0, t0 + gridDim.x DW_T): row 3 (tau - t0) + a, column j
+// receives sum over (sigma, b) around vertex j with sigma >= tau of L_ab(tau, sigma), the pair tau = sigma halved
+// (the other half of the symmetric G comes from the transpose in k_dense_sym), with
+//   L_ab = sum_{q, p} w_q psi_a(x_q) g(x_q, y_p) psi_b(y_p) w_p / (4 pi)
+// over the 6 x 6 points of the pair (coincident points left out).  A block takes DW_T test triangles and DW_S
+// trial triangles at a time: thread sigma evaluates the 36 kernel values once (they serve three vertices on
+// either side), contracts them to 3 x 3 and leaves those in shared memory; then a thread per vertex adds the
+// entries of its triangles in incidence order.  The kernel's root (and exponential) on the special-function
+// unit bounds it: 1 or 2 per point pair, about 8 float32 operations' time each.
+// GB300, 3920 triangles (1962 vertices), Yukawa: 1279 us for G P evaluated once per (point, vertex), its weights
+// multiplied in float64 each time, and 515 us for the second product; 287 us and 44 us so.
 template <bool YUK>
-__global__ void __launch_bounds__(DW_T) k_dense_w(int nv, int a0, int na, const float4* __restrict__ qpf,
-                                                  const double* __restrict__ qw, const int* __restrict__ inc_ptr,
-                                                  const int* __restrict__ inc_idx, float kappa,
-                                                  float* __restrict__ W) {
-  const int j = blockIdx.x * DW_T + threadIdx.x;
-  const int ab = blockIdx.y * DW_A;
-  float tx[DW_A], ty[DW_A], tz[DW_A], acc[DW_A];
+__global__ void __launch_bounds__(DW_NT, 2) k_dense_rows(int nv, int nt, int t0, int t1, const float4* __restrict__ qpf,
+                                                      const double* __restrict__ qw, const float* __restrict__ wq,
+                                                      const int* __restrict__ inc_ptr,
+                                                      const int* __restrict__ inc_idx, float nk,
+                                                      float* __restrict__ W) {
+  extern __shared__ float4 sm4[];
+  float* L = reinterpret_cast<float*>(sm4);  // [DW_T][3 a][3 b][DW_S]
+  __shared__ float4 tp[DW_T][QS];            // test points
+  __shared__ float tw[DW_T][QS][3];          // w_q psi_a(x_q) / 4 pi
+  const int tau0 = t0 + blockIdx.x * DW_T;
+  if (threadIdx.x < DW_T * QS) {
+    const int u = threadIdx.x / QS, q = threadIdx.x % QS;
+    const int j = QS * min(tau0 + u, nt - 1) + q;
+    tp[u][q] = qpf[j];
 #pragma unroll
-  for (int u = 0; u < DW_A; ++u) {
-    const float4 p = qpf[a0 + min(ab + u, na - 1)];
-    tx[u] = p.x;
-    ty[u] = p.y;
-    tz[u] = p.z;
-    acc[u] = 0.f;
+    for (int a = 0; a < 3; ++a) tw[u][q][a] = (float)(qw[j] * c_tri_b[q][a] * 0.079577471545947667884);
   }
-  if (j < nv) {
-    for (int e = inc_ptr[j]; e < inc_ptr[j + 1]; ++e) {
-      const int ent = inc_idx[e];
-      const int t = ent / 3, k = ent - 3 * t;
-      for (int q = 0; q < QS; ++q) {
-        const int b = QS * t + q;
-        const float4 p = qpf[b];
-        const float wb = (float)(qw[b] * c_tri_b[q][k] * INV4PI);
+  __syncthreads();
+  for (int s0 = tau0; s0 < nt; s0 += DW_S) {
+    const int s1 = min(nt, s0 + DW_S);
+    for (int s = s0 + threadIdx.x; s < s1; s += DW_NT) {
+      float y[QS][3], wb[QS][3];
 #pragma unroll
-        for (int u = 0; u < DW_A; ++u) {
-          const float dx = tx[u] - p.x, dy = ty[u] - p.y, dz = tz[u] - p.z;
-          // the coincident point gets r2 = 1e-30 (finite terms) and weight 0
-          const float r2 = fmaxf(dx * dx + dy * dy + dz * dz, 1e-30f);
-          const float ir = rsqrtf(r2);
-          float g = (a0 + ab + u != b) ? ir : 0.f;
-          if (YUK) g *= __expf(-kappa * r2 * ir);
-          acc[u] += wb * g;
+      for (int p = 0; p < QS; ++p) {
+        const float4 f = qpf[QS * s + p];
+        y[p][0] = f.x;
+        y[p][1] = f.y;
+        y[p][2] = f.z;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) wb[p][b] = wq[(size_t)b * QS * nt + QS * s + p];
+      }
+#pragma unroll 1
+      for (int u = 0; u < DW_T; ++u) {
+        const bool own = s == tau0 + u;
+        float acc[3][3] = {};
+#pragma unroll
+        for (int q = 0; q < QS; ++q) {
+          const float4 x = tp[u][q];
+          float h[3] = {};
+#pragma unroll
+          for (int p = 0; p < QS; ++p) {
+            const float dx = x.x - y[p][0], dy = x.y - y[p][1], dz = x.z - y[p][2];
+            // the coincident point gets r2 = 1e-30 (finite terms) and weight 0
+            const float r2 = fmaxf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)), 1e-30f);
+            const float ir = rsqrt_approx(r2);
+            float g = ir;
+            if (YUK) g *= ex2_approx(nk * (r2 * ir));
+            if (p == q && own) g = 0.f;
+#pragma unroll
+            for (int b = 0; b < 3; ++b) h[b] = fmaf(g, wb[p][b], h[b]);
+          }
+#pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            const float wa = tw[u][q][a];
+#pragma unroll
+            for (int b = 0; b < 3; ++b) acc[a][b] = fmaf(wa, h[b], acc[a][b]);
+          }
         }
+        const float f = own ? 0.5f : (s < tau0 + u ? 0.f : 1.f);
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+          for (int b = 0; b < 3; ++b) L[((3 * u + a) * 3 + b) * DW_S + s - s0] = f * acc[a][b];
       }
     }
-  }
+    __syncthreads();
+    for (int j = threadIdx.x; j < nv; j += DW_NT) {
+      float v[3 * DW_T];
 #pragma unroll
-  for (int u = 0; u < DW_A; ++u)
-    if (j < nv && ab + u < na) W[(size_t)(ab + u) * nv + j] = acc[u];
+      for (int r = 0; r < 3 * DW_T; ++r) v[r] = 0.f;
+      for (int e = inc_ptr[j]; e < inc_ptr[j + 1]; ++e) {
+        const int ent = inc_idx[e], s = ent / 3, b = ent - 3 * s;
+        if (s < s0 || s >= s1) continue;
+#pragma unroll
+        for (int r = 0; r < 3 * DW_T; ++r) v[r] += L[(3 * r + b) * DW_S + s - s0];
+      }
+#pragma unroll
+      for (int r = 0; r < 3 * DW_T; ++r)
+        if (tau0 + r / 3 < t1) {
+          float* w = W + (size_t)(3 * (tau0 - t0) + r) * nv + j;
+          *w = s0 > tau0 ? *w + v[r] : v[r];
+        }
+    }
+    __syncthreads();
+  }
 }
 
-// A[i][j] += sum over (tau, a) around vertex i with tau in [t0, t1) of
-//   sum_q w_q psi_i(x_q) W[q-point of tau][j]
-__global__ void k_dense_v(int nv, int ld, int t0, int t1, const float* __restrict__ W,
-                          const double* __restrict__ qw, const int* __restrict__ inc_ptr,
-                          const int* __restrict__ inc_idx, float* __restrict__ A) {
+// A[i][j] += sum over (tau, a) around vertex i with tau in [t0, t1) of W's row (tau, a)
+__global__ void k_dense_fold(int nv, int ld, int t0, int t1, const float* __restrict__ W,
+                             const int* __restrict__ inc_ptr, const int* __restrict__ inc_idx, float* __restrict__ A) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = blockIdx.y;
   if (j >= nv) return;
   float acc = 0.f;
   bool any = false;
   for (int e = inc_ptr[i]; e < inc_ptr[i + 1]; ++e) {
-    const int ent = inc_idx[e];
-    const int t = ent / 3, k = ent - 3 * t;
+    const int ent = inc_idx[e], t = ent / 3, a = ent - 3 * t;
     if (t < t0 || t >= t1) continue;
     any = true;
-    for (int q = 0; q < QS; ++q) {
-      const int a = QS * t + q;
-      acc += (float)(qw[a] * c_tri_b[q][k]) * W[(size_t)(a - QS * t0) * nv + j];
-    }
+    acc += W[(size_t)(3 * (t - t0) + a) * nv + j];
   }
   if (any) A[(size_t)i * ld + j] += acc;
+}
+
+// wq[b][j] = w_j psi_b(y_j)
+__global__ void k_dense_weights(int nq, const double* __restrict__ qw, float* __restrict__ wq) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= nq) return;
+  for (int b = 0; b < 3; ++b) wq[(size_t)b * nq + j] = (float)(qw[j] * c_tri_b[j % QS][b]);
 }
 
 // zero, with the identity on the padding diagonal
@@ -115,96 +172,116 @@ __global__ void k_dense_init(int n, int ld, float* __restrict__ A) {
   }
 }
 
-// sparse exact-minus-regular corrections, one thread per row
+// half of the sparse exact-minus-regular corrections, one thread per row
 __global__ void k_dense_corr(int nv, int ld, const int* __restrict__ ptr, const int* __restrict__ col,
                              const double* __restrict__ corr, float* __restrict__ A) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nv) return;
-  for (int s = ptr[i]; s < ptr[i + 1]; ++s) A[(size_t)i * ld + col[s]] += (float)corr[s];
+  for (int s = ptr[i]; s < ptr[i + 1]; ++s) A[(size_t)i * ld + col[s]] += 0.5f * (float)corr[s];
 }
 
-// A <- (A + A^T) / 2; the thread of (i, j > i) writes both entries
+// A <- A + A^T by 32 x 32 tiles on and above the diagonal; a block writes a tile and its mirror image
 __global__ void k_dense_sym(int n, int ld, float* __restrict__ A) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  const int i = blockIdx.y;
-  if (j <= i || j >= n) return;
-  const float v = 0.5f * (A[(size_t)i * ld + j] + A[(size_t)j * ld + i]);
-  A[(size_t)i * ld + j] = v;
-  A[(size_t)j * ld + i] = v;
-}
-
-// Sweep of the SW_B x SW_B pivot block at (k0, k0), scalar pivots in order, in shared memory.
-// Writes the swept block S (= -D, D the inverse of the block) and flags a pivot that is not
-// positive and finite.
-__global__ void __launch_bounds__(256) k_sweep_pivot(int ld, int k0, const float* __restrict__ A,
-                                                     float* __restrict__ S, int* __restrict__ flag) {
-  __shared__ float sS[SW_B][SW_B + 1];
-  __shared__ float rowp[SW_B], colp[SW_B];
-  const int tid = threadIdx.x;
-  for (int e = tid; e < SW_B * SW_B; e += 256) {
-    const int r = e / SW_B, c = e % SW_B;
-    sS[r][c] = A[(size_t)(k0 + r) * ld + k0 + c];
+  __shared__ float t[32][33], r[32][33];
+  const int I = blockIdx.y, J = blockIdx.x;
+  if (J < I) return;
+  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
+    const int i = 32 * I + k, j = 32 * J + threadIdx.x;  // ld is a multiple of 128: the padding tiles exist
+    t[k][threadIdx.x] = A[(size_t)i * ld + j];
+    r[k][threadIdx.x] = A[(size_t)(32 * J + k) * ld + 32 * I + threadIdx.x];
   }
   __syncthreads();
-  bool bad = false;
-  for (int p = 0; p < SW_B; ++p) {
-    if (tid < SW_B) {
-      rowp[tid] = sS[p][tid];
-      colp[tid] = sS[tid][p];
-    }
-    __syncthreads();
-    const float d = rowp[p];
-    bad = bad || !(d > 0.f) || !isfinite(d);
-    const float inv = 1.f / d;
-    for (int e = tid; e < SW_B * SW_B; e += 256) {
-      const int r = e / SW_B, c = e % SW_B;
-      sS[r][c] -= colp[r] * rowp[c] * inv;
-    }
-    __syncthreads();
-    if (tid < SW_B) {
-      sS[p][tid] = rowp[tid] * inv;
-      sS[tid][p] = colp[tid] * inv;
-    }
-    __syncthreads();
-    if (tid == 0) sS[p][p] = -inv;
-    __syncthreads();
-  }
-  if (tid == 0 && bad) atomicExch(flag, 1);
-  for (int e = tid; e < SW_B * SW_B; e += 256) {
-    const int r = e / SW_B, c = e % SW_B;
-    S[e] = sS[r][c];
+  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
+    const int i = 32 * I + k, j = 32 * J + threadIdx.x;
+    if (i < n && j < n) A[(size_t)i * ld + j] = t[k][threadIdx.x] + r[threadIdx.x][k];
+    if (I != J && 32 * J + k < n && 32 * I + threadIdx.x < n)
+      A[(size_t)(32 * J + k) * ld + 32 * I + threadIdx.x] = r[k][threadIdx.x] + t[threadIdx.x][k];
   }
 }
 
-// Row panel of the pivot: P = A[K, :] (old values) and U = D P with D = -S; one column per thread.
-// Only the tiles on and below the diagonal are kept current during the sweep (the matrix stays
-// symmetric), so row K beyond its diagonal tile is read from column K: A[K][j] = A[j][K].
-__global__ void __launch_bounds__(128) k_sweep_panel(int ld, int k0, const float* __restrict__ A,
-                                                     const float* __restrict__ S, float* __restrict__ P,
-                                                     float* __restrict__ U) {
+// Sweep of the SW_B x SW_B pivot block at (k0, k0), scalar pivots in order, and the row panel of the pivot:
+// P = A[K, :] (old values) and U = D P, D = -S the inverse of the block; the swept block S is written and a pivot
+// that is not positive and finite flagged.  Only the tiles on and below the diagonal are kept current during the
+// sweep (the matrix stays symmetric), so row K beyond its diagonal tile is read from column K: A[K][j] = A[j][K].
+// The 64 dependent pivot steps bound it: every block sweeps the pivot block itself (no launch between the two
+// halves), a thread keeping a 4 x 4 piece in registers and a step passing the pivot's row and column through
+// one of two shared buffers, so that it needs one barrier; the panel's columns are loaded before.  A block takes
+// 128 columns and nr of U's rows (blockIdx.y): fewer rows for more blocks on small matrices.
+// GB300, ld = 2048, per step: 37.5 us for one block with four barriers a pivot and 15 us for the panel; 20.5 us
+// together, and one launch gap less.
+__global__ void __launch_bounds__(256) k_sweep_pivot_panel(int ld, int k0, int nr, const float* __restrict__ A,
+                                                           float* __restrict__ S, float* __restrict__ P,
+                                                           float* __restrict__ U, int* __restrict__ flag) {
+  __shared__ float rowp[2][SW_B], colp[2][SW_B];
   __shared__ float sD[SW_B][SW_B];
-  for (int e = threadIdx.x; e < SW_B * SW_B; e += 128) sD[e / SW_B][e % SW_B] = -S[e];
-  __syncthreads();
-  const int j = blockIdx.x * 128 + threadIdx.x;  // ld is a multiple of 128
+  const int col = threadIdx.x & 127, half = threadIdx.x >> 7;
+  const int j = blockIdx.x * 128 + col;  // ld is a multiple of 128
   const int kend = (k0 / SW_TILE + 1) * SW_TILE;  // end of the pivot's diagonal tile
   float pv[SW_B];
   if (j < kend) {
 #pragma unroll
     for (int p = 0; p < SW_B; ++p) pv[p] = A[(size_t)(k0 + p) * ld + j];
   } else {
-    const float4* col = reinterpret_cast<const float4*>(A + (size_t)j * ld + k0);
+    const float4* c = reinterpret_cast<const float4*>(A + (size_t)j * ld + k0);
 #pragma unroll
     for (int q = 0; q < SW_B / 4; ++q) {
-      const float4 v = col[q];
+      const float4 v = c[q];
       pv[4 * q] = v.x;
       pv[4 * q + 1] = v.y;
       pv[4 * q + 2] = v.z;
       pv[4 * q + 3] = v.w;
     }
   }
+  const int tr = threadIdx.x / 16, tc = threadIdx.x % 16;  // rows tr + 16 i, columns tc + 16 j
+  float v[4][4];
 #pragma unroll
-  for (int p = 0; p < SW_B; ++p) P[(size_t)p * ld + j] = pv[p];
-  for (int p = 0; p < SW_B; ++p) {
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[i][c] = A[(size_t)(k0 + tr + 16 * i) * ld + k0 + tc + 16 * c];
+  bool bad = false;
+#pragma unroll
+  for (int pi = 0; pi < 4; ++pi)
+#pragma unroll 1
+    for (int pk = 0; pk < 16; ++pk) {
+      const int p = 16 * pi + pk, buf = pk & 1;
+      if (tr == pk)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) rowp[buf][tc + 16 * c] = v[pi][c];
+      if (tc == pk)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) colp[buf][tr + 16 * i] = v[i][pi];
+      __syncthreads();
+      const float d = rowp[buf][p];
+      bad = bad || !(d > 0.f) || !isfinite(d);
+      const float inv = 1.f / d;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float x = colp[buf][tr + 16 * i];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[i][c] -= x * rowp[buf][tc + 16 * c] * inv;
+      }
+      if (tr == pk)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[pi][c] = rowp[buf][tc + 16 * c] * inv;
+      if (tc == pk)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i][pi] = colp[buf][tr + 16 * i] * inv;
+      if (tr == pk && tc == pk) v[pi][pi] = -inv;
+    }
+  const bool first = blockIdx.x == 0 && blockIdx.y == 0;
+  if (first && threadIdx.x == 0 && bad) atomicExch(flag, 1);
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      sD[tr + 16 * i][tc + 16 * c] = -v[i][c];
+      if (first) S[(tr + 16 * i) * SW_B + tc + 16 * c] = v[i][c];
+    }
+  __syncthreads();
+  if (blockIdx.y == 0 && half == 0)
+#pragma unroll
+    for (int p = 0; p < SW_B; ++p) P[(size_t)p * ld + j] = pv[p];
+  for (int p = blockIdx.y * nr + half; p < (int)(blockIdx.y + 1) * nr; p += 2) {
     float acc = 0.f;
 #pragma unroll
     for (int q = 0; q < SW_B; ++q) acc += sD[p][q] * pv[q];
@@ -246,7 +323,13 @@ __global__ void __launch_bounds__(256) k_sweep_update(int ld, int k0, float* __r
   for (int p = 0; p < SW_B; ++p) {
     float a[8];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) a[r] = Ps[p * SW_TILE + ty + 16 * r];
+    for (int r = 0; r < 2; ++r) {
+      const float4 v = *reinterpret_cast<const float4*>(Ps + p * SW_TILE + 8 * ty + 4 * r);
+      a[4 * r] = v.x;
+      a[4 * r + 1] = v.y;
+      a[4 * r + 2] = v.z;
+      a[4 * r + 3] = v.w;
+    }
     const float4 b0 = *reinterpret_cast<const float4*>(Us + p * SW_TILE + 4 * tx);
     const float4 b1 = *reinterpret_cast<const float4*>(Us + p * SW_TILE + 64 + 4 * tx);
     const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
@@ -258,7 +341,7 @@ __global__ void __launch_bounds__(256) k_sweep_update(int ld, int k0, float* __r
   const bool slow = (k0 >= i0 && k0 < i0 + SW_TILE) || (k0 >= j0 && k0 < j0 + SW_TILE);
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
-    const int i = i0 + ty + 16 * r;
+    const int i = i0 + 8 * ty + r;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int j = j0 + 64 * h + 4 * tx;
@@ -344,7 +427,7 @@ size_t dense_bytes(int n) {
 
 size_t dense_work_bytes(int n, int nt) {
   const size_t ld = (size_t)dense_ld(n);
-  return std::min(DENSE_W_BYTES, (size_t)QS * nt * n * 4) + (2 * SW_B * ld + SW_B * SW_B + 64) * 4;
+  return std::min(DENSE_W_BYTES, (size_t)3 * nt * n * 4) + (2 * SW_B * ld + SW_B * SW_B + 64 + (size_t)3 * QS * nt) * 4;
 }
 
 int build_dense_single_layer(Mesh* m, Surface* s, double kappa, bool invert) {
@@ -362,57 +445,52 @@ int build_dense_single_layer(Mesh* m, Surface* s, double kappa, bool invert) {
   PB_TRY(ensure_f(s->vinv, (size_t)ld * ld));
   s->vinv_ld = ld;
   // triangles per chunk of W (at most DENSE_W_BYTES of float32, released after the build)
-  const int ct = (int)std::max<size_t>(1, std::min<size_t>(nt, DENSE_W_BYTES / ((size_t)QS * n * 4)));
-  const size_t wlen = ((size_t)ct * QS * n + 63) / 64 * 64;  // keeps the panels 256-byte aligned
-  PB_TRY(ensure_f(m->dwork, wlen + 2 * (size_t)SW_B * ld + SW_B * SW_B));
+  const int ct = (int)std::max<size_t>(1, std::min<size_t>(nt, DENSE_W_BYTES / ((size_t)3 * n * 4)));
+  const size_t wlen = ((size_t)ct * 3 * n + 63) / 64 * 64;  // keeps the panels 256-byte aligned
+  PB_TRY(ensure_f(m->dwork, wlen + 2 * (size_t)SW_B * ld + SW_B * SW_B + 3 * (size_t)s->nq));
   if (m->dflag.n < 1) PB_TRY(m->dflag.alloc(1));
   float* W = m->dwork.p;
   float* P = W + wlen;
   float* U = P + (size_t)SW_B * ld;
   float* S = U + (size_t)SW_B * ld;
+  float* wq = S + SW_B * SW_B;
   float* A = s->vinv.p;
   cudaEvent_t ev;
   timer_begin(m, m->t_dense, &ev);
   k_dense_init<<<4 * 152, 256, 0, m->stream>>>(n, ld, A);
   PB_LAUNCHED(m);
-  const dim3 gw((n + DW_T - 1) / DW_T, 1);
-  if ((QS * ct + DW_A - 1) / DW_A > 65535) {
-    set_error("dense single layer: work chunk too large");
-    return PBFB_ERR_INVALID;
-  }
+  k_dense_weights<<<(s->nq + 255) / 256, 256, 0, m->stream>>>(s->nq, s->qw.p, wq);
+  PB_LAUNCHED(m);
+  const int gj = (n + 127) / 128;
+  const float nk = (float)(-kappa * 1.44269504088896340736);
   for (int t0 = 0; t0 < nt; t0 += ct) {
     const int t1 = std::min(nt, t0 + ct);
-    const int na = QS * (t1 - t0);
-    dim3 g(gw.x, (na + DW_A - 1) / DW_A);
-    if (kappa != 0.0)
-      k_dense_w<true><<<g, DW_T, 0, m->stream>>>(n, QS * t0, na, s->qpf.p, s->qw.p, s->inc_ptr.p, s->inc_idx.p,
-                                                (float)kappa, W);
-    else
-      k_dense_w<false><<<g, DW_T, 0, m->stream>>>(n, QS * t0, na, s->qpf.p, s->qw.p, s->inc_ptr.p, s->inc_idx.p,
-                                                 0.f, W);
+    const auto fn = kappa != 0.0 ? k_dense_rows<true> : k_dense_rows<false>;
+    fn<<<(t1 - t0 + DW_T - 1) / DW_T, DW_NT, DW_SMEM, m->stream>>>(n, nt, t0, t1, s->qpf.p, s->qw.p, wq, s->inc_ptr.p,
+                                                                   s->inc_idx.p, nk, W);
     PB_LAUNCHED(m);
-    k_dense_v<<<dim3(gw.x, n), DW_T, 0, m->stream>>>(n, ld, t0, t1, W, s->qw.p, s->inc_ptr.p, s->inc_idx.p, A);
+    k_dense_fold<<<dim3(gj, n), 128, 0, m->stream>>>(n, ld, t0, t1, W, s->inc_ptr.p, s->inc_idx.p, A);
     PB_LAUNCHED(m);
   }
   k_dense_corr<<<(n + 127) / 128, 128, 0, m->stream>>>(n, ld, s->c_ptr.p, s->c_col.p, s->corrV.p, A);
   PB_LAUNCHED(m);
-  k_dense_sym<<<dim3(gw.x, n), DW_T, 0, m->stream>>>(n, ld, A);
+  const int n32 = (n + 31) / 32;
+  k_dense_sym<<<dim3(n32, n32), dim3(32, 8), 0, m->stream>>>(n, ld, A);
   PB_LAUNCHED(m);
   if (invert) {
     PB_CUDA(cudaMemsetAsync(m->dflag.p, 0, sizeof(int), m->stream));
     const int smem = 2 * SW_B * SW_TILE * (int)sizeof(float);  // attribute set by init_dense_attributes
     const int ntile = ld / SW_TILE;
     const int gu = ntile * (ntile + 1) / 2;  // tiles on and below the diagonal
+    const int nr = ld <= 2432 ? 8 : (ld <= 4864 ? 16 : (ld <= 9728 ? 32 : SW_B));  // about a block an SM
     for (int k0 = 0; k0 < ld; k0 += SW_B) {
-      k_sweep_pivot<<<1, 256, 0, m->stream>>>(ld, k0, A, S, m->dflag.p);
-      PB_LAUNCHED(m);
-      k_sweep_panel<<<ld / 128, 128, 0, m->stream>>>(ld, k0, A, S, P, U);
+      k_sweep_pivot_panel<<<dim3(ld / 128, SW_B / nr), 256, 0, m->stream>>>(ld, k0, nr, A, S, P, U, m->dflag.p);
       PB_LAUNCHED(m);
       k_sweep_update<<<gu, 256, smem, m->stream>>>(ld, k0, A, P, U, S);
       PB_LAUNCHED(m);
     }
-    const int n32 = ld / 32;
-    k_sweep_mirror<<<n32 * (n32 - 1) / 2, dim3(32, 8), 0, m->stream>>>(ld, A);
+    const int l32 = ld / 32;
+    k_sweep_mirror<<<l32 * (l32 - 1) / 2, dim3(32, 8), 0, m->stream>>>(ld, A);
     PB_LAUNCHED(m);
     PB_CUDA(cudaMemcpyAsync(m->pinned, m->dflag.p, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
   }
@@ -442,6 +520,8 @@ int init_dense_attributes() {
   if (dev < 64 && ((done >> dev) & 1)) return PBFB_OK;
   PB_CUDA(cudaFuncSetAttribute(k_sweep_update, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                2 * SW_B * SW_TILE * (int)sizeof(float)));
+  for (const void* f : {(const void*)k_dense_rows<true>, (const void*)k_dense_rows<false>})
+    PB_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, DW_SMEM));
   PB_CUDA(cudaFuncSetAttribute(k_dense_apply, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                dense_ld(DENSE_V_MAX) * (int)sizeof(float)));
   if (dev < 64) done |= 1ull << dev;
