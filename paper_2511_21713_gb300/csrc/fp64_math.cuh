@@ -37,5 +37,31 @@ __device__ __forceinline__ double exp2_neg(double x, const double* __restrict__ 
   return fma(T * f, fma(f, fma(f, -L * L * L / 6.0, 0.5 * L * L), -L), T);
 }
 
+// e^a and e^-a for a >= 0: a = (k / 2048) ln 2 + f, |f| <= 1.7e-4 (ln 2 / 2048 in two parts, the first with 30
+// bits so that its product with k is exact), e^+-f = 1 + (f^2/2 + f^4/24) +- (f + f^3/6) (truncation 2^-62),
+// 2^-+k/2048 from the table.  From 700 on (and for a NaN) the library's exponentials.
+__device__ __forceinline__ void exp_pm(double a, const double* __restrict__ tab, double& ep, double& em) {
+  if (!(a < 700.0)) {
+    ep = exp(a);
+    em = exp(-a);
+    return;
+  }
+  const int ahi = max(__double2hiint(a), 0x3C300000);
+  const unsigned ab = __funnelshift_l(__double2loint(a), ahi, 3) - 0xC0000000u;  // float32 bits of max(a, 2^-60)
+  const float m = __fmaf_rn(__uint_as_float(ab), 2954.6394f, 12582912.f);  // 2048 / ln 2
+  const int k = __float_as_int(m) - 0x4B400000;
+  const int kb = __float_as_int(__fsub_rn(m, 12582912.f));
+  const double kd = __hiloint2double((kb >> 3) + (896 << 20), kb << 29);  // k (0 becomes 2^-127)
+  constexpr double C1 = 0x1.62e42fe8p-12, C2 = 4.3423507025813853e-13;  // ln 2 / 2048 = C1 + C2
+  const double f = fma(-kd, C2, fma(-kd, C1, a)), s = f * f;
+  const double even = s * fma(s, 1.0 / 24.0, 0.5), odd = f * fma(s, 1.0 / 6.0, 1.0);
+  const int e = k / EXP2_TAB, j = k & (EXP2_TAB - 1);
+  const double tm = tab[j], tp = tab[(EXP2_TAB - j) & (EXP2_TAB - 1)];  // 2^-j/2048; 2^(j/2048 - 1), or 1 for j = 0
+  const double Tm = __hiloint2double(__double2hiint(tm) - (e << 20), __double2loint(tm));
+  const double Tp = __hiloint2double(__double2hiint(tp) + ((e + (j != 0)) << 20), __double2loint(tp));
+  ep = fma(Tp, even + odd, Tp);
+  em = fma(Tm, even - odd, Tm);
+}
+
 }  // namespace
 }  // namespace pbfb

@@ -184,6 +184,7 @@ struct Mesh {
   int nq = 0;
   DBuf<double> qxyz, qz;    // 3*nq SoA, nq
   DBuf<double> coul;        // nm: <sum z/|x-x_k|, psi_i> (no l_B/eps_m)
+  DBuf<double> coul_ce;     // 2*nq of Gamma_m: the charges' potential and normal field sums (k_coulomb)
   bool charges = false;
   // parameters
   double eps_m = 0, eps_s = 0, kappa = 0, T = 0, lB = 0, kT = 0, coef = 0;
@@ -218,7 +219,6 @@ struct Mesh {
   DBuf<double> pval, pdinv;
   DBuf<float> pvalf, pdinvf;        // float32 copies for the mixed precision's cooperative PCG
   DBuf<float> pcgf;                 // its vectors x, r, z, p, q, w (n each; z stays 0 past nv)
-  DBuf<double> reac_rec, reac_part; // reaction potentials: Gamma_m point records, chunk partials
   bool pcg_f32 = false;             // the cooperative PCG runs in float32
   int tune_pcg_prec = 0;            // its arithmetic: 0 built-in (float32 in MIXED), 1 float64, 2 float32
   double gs_radius = 1.0;           // sqrt(|Gamma_s| / 4 pi)
@@ -246,8 +246,7 @@ struct Mesh {
   DBuf<float> dwork;                // dense single-layer build: W chunk, sweep panels
   DBuf<int> dflag;                  // sweep pivot status
   // Newton workspace
-  DBuf<double> xL, xNL, phi, cvec, dvec, du, pvec, tmp, Nvec, bvec, xout, urb;
-  std::vector<double> qz_h;  // charges (host copy)
+  DBuf<double> xL, xNL, phi, cvec, dvec, du, pvec, tmp, Nvec, bvec, xout;
   // statistics
   double launches = 0;
   bool timing = false;
@@ -324,7 +323,10 @@ int launch_omega_elements(Mesh* m, int scheme, const double* u, const double* du
                           const double* omegas_dev, int nomega, double coef, double* loc, bool* ff);
 int launch_omega_dots(Mesh* m, int nomega, const double* loc, const double* c, const double* p,
                       double* dots_dev, bool ff);
-int launch_ion_energy(Mesh* m, const double* u, double* out_dev);
+// the ion integral of u1 + u2
+int launch_ion_energy(Mesh* m, const double* u1, const double* u2, double* out_dev);
+// out_dev[k] = sum of the nb rows of width w in m->red, fixed order
+int launch_sum_partials(Mesh* m, int nb, int w, double* out_dev);
 int launch_fill_operator(Mesh* m);
 int launch_csr_spmv(Mesh* m, int nrows, const int* ptr, const int* col, const double* val, const double* x,
                     double* y, bool accumulate);
@@ -338,8 +340,7 @@ int launch_bem_far(Mesh* m, Surface* s, const double* x, const double* lam, doub
 int launch_bem_far_ff(Mesh* m, Surface* s, const double* x, const double* lam, double cs, double cd,
                       double kappa, double* y, bool accumulate);
 int launch_coulomb(Mesh* m);
-// reaction potentials of x_L and x_NL at the charges: ur_dev[0, nq) and ur_dev[nq, 2 nq)
-int launch_reaction_potentials(Mesh* m, const double* xL, const double* xNL, double* ur_dev);
+int launch_reaction_energy(Mesh* m, const double* xL, const double* xNL, double* out_dev);
 int bem_apply_noalloc(Mesh* m, int which, int op, const double* x, double* y);
 
 // Grid of the float-float coordinates' high parts for lengths scaled by `scale` (a power of 2): differences

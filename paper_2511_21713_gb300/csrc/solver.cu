@@ -1738,25 +1738,15 @@ static int gamma_m_flux(Mesh* m, const double* x, bool coulomb, double* lam) {
 }
 
 static int energy(Mesh* m, const double* xL, const double* xNL, double* out4) {
-  PB_TRY(ensure(m->tmp, m->n));
-  PB_TRY(ensure(m->urb, 2 * (size_t)m->nq));
-  PB_TRY(launch_reaction_potentials(m, xL, xNL, m->urb.p));
-  std::vector<double> urh(2 * (size_t)m->nq);
-  PB_CUDA(cudaMemcpyAsync(urh.data(), m->urb.p, urh.size() * sizeof(double), cudaMemcpyDeviceToHost, m->stream));
-  // ion term on u = (x_L + x_NL) restricted to the shell
-  PB_TRY(launch_axpby(m, m->nv, 1.0, xL, 1.0, xNL, m->tmp.p));
-  PB_TRY(launch_ion_energy(m, m->tmp.p, m->scal.p + 1000));
-  PB_CUDA(cudaMemcpyAsync(m->pinned, m->scal.p + 1000, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
+  // reaction energies, then the ion term on u = x_L + x_NL restricted to the shell
+  double* e3 = m->scal.p + 1000;
+  PB_TRY(launch_reaction_energy(m, xL, xNL, e3));
+  PB_TRY(launch_ion_energy(m, xL, xNL, e3 + 2));
+  PB_CUDA(cudaMemcpyAsync(m->pinned, e3, 3 * sizeof(double), cudaMemcpyDeviceToHost, m->stream));
   PB_CUDA(cudaStreamSynchronize(m->stream));
-  double LC = 0.0, NC = 0.0;
-  for (int k = 0; k < m->nq; ++k) {
-    LC += m->qz_h[k] * urh[k];
-    NC += m->qz_h[k] * urh[m->nq + k];
-  }
-  LC *= 0.5 * m->kT;
-  NC *= 0.5 * m->kT;
+  const double LC = m->pinned[0] * (0.5 * m->kT / (4.0 * M_PI)), NC = m->pinned[1] * (0.5 * m->kT / (4.0 * M_PI));
   const double c0 = m->coef / (8.0 * M_PI * m->lB);
-  const double dG = m->kT * c0 * m->pinned[0];
+  const double dG = m->kT * c0 * m->pinned[2];
   out4[0] = LC + NC + dG;
   out4[1] = LC;
   out4[2] = NC;
@@ -2035,11 +2025,12 @@ int charges_set(Mesh* m, const double* xyz, const double* z, int n_q) {
     PB_TRY(point_load(m, xyz, z, n_q, rho));
     PB_TRY(m->rho.upload(rho.data(), rho.size(), m->stream));
   }
-  PB_TRY(m->qxyz.upload(soa.data(), soa.size(), m->stream));
-  PB_TRY(m->qz.upload(z, n_q, m->stream));
-  m->qz_h.assign(z, z + n_q);
+  PB_TRY(ensure(m->qxyz, soa.size()));
+  PB_TRY(ensure(m->qz, n_q));
+  PB_CUDA(cudaMemcpyAsync(m->qxyz.p, soa.data(), soa.size() * sizeof(double), cudaMemcpyHostToDevice, m->stream));
+  PB_CUDA(cudaMemcpyAsync(m->qz.p, z, n_q * sizeof(double), cudaMemcpyHostToDevice, m->stream));
   m->nq = n_q;
-  PB_TRY(m->coul.alloc(m->sm.nv));
+  PB_TRY(ensure(m->coul, m->sm.nv));
   PB_TRY(launch_coulomb(m));
   if (cudaStreamSynchronize(m->stream) != cudaSuccess) {
     set_error("charges_set: %s", cudaGetErrorString(cudaGetLastError()));
