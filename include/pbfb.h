@@ -409,10 +409,12 @@ typedef struct pbfb_tuning {
                                         pbfb_newton_opts.residual_far. */
   int32_t pcg_precision;             /* arithmetic of the cooperative inner PCG (CSR forms):
                                         1 float64, 2 float32 (float32 matrix and vectors, float64
-                                        block and grid sums; meshes of at most 480 FEM rows per SM
+                                        block and grid sums; meshes of at most 992 FEM rows per SM
                                         run the pipelined form with each row and its vectors held
                                         in registers, one grid barrier per step, for
-                                        pcg_lanes 2, 4 or 8 alike); 0 built-in: float32 in the PBFB_MIXED
+                                        pcg_lanes 2, 4 or 8 alike); meshes of at most 15,872
+                                        (float64: 11,776) FEM rows run on one cluster of 16 blocks
+                                        instead, also for pcg_lanes 2, 4 or 8 alike; 0 built-in: float32 in the PBFB_MIXED
                                         precision, float64 otherwise.  The sliced-ELL form
                                         (pcg_lanes 1) is float64 only. */
 } pbfb_tuning;

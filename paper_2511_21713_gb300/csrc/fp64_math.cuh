@@ -16,6 +16,15 @@ __device__ __forceinline__ double rsqrt64(double r2) {
   return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
+// 1/d: the hardware's estimate (about 2^-20) and two Newton steps, y (2 - d y); a d of 0 or below the normal
+// numbers gives a non-finite value
+__device__ __forceinline__ double rcp64(double d) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+  y = fma(y, fma(-d, y, 1.0), y);
+  return fma(y, fma(-d, y, 1.0), y);
+}
+
 // 2^-x for 0 <= x: 2^-x = 2^-m T[j] 2^-f, x = m + j / 2048 + f with |f| <= 2^-12 (k = 2048 m + j from the
 // float32 value of x, the float64 remainder exact), 2^-f = 1 + f (-L + f (L^2/2 - f L^3/6)), L = ln 2
 // (truncation 2^-54).  0 once 2^-m leaves the normal numbers.

@@ -688,6 +688,7 @@ int mesh_create(const double* xyz, int nv, const int* tets, int64_t nt, const in
   PB_TRY(init_quadrature());
   PB_TRY(init_dense_attributes());
   PB_TRY(init_pair_attributes());
+  PB_TRY(init_pcg_attributes());
   Mesh* m = new Mesh();
   int st = PBFB_OK;
   auto fail = [&](int s) {

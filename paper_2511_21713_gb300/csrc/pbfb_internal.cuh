@@ -225,6 +225,7 @@ struct Mesh {
   int coop_blocks = 0;              // grid of the cooperative inner PCG (-1: not available)
   int coop_blocks_f32 = 0;          // grid of its float32 form (one block per SM; -1: not available)
   int coop_blocks_pipe = 0;         // blocks of its register-resident pipelined form (one per SM)
+  bool pcg_cluster = false;         // small meshes: the PCG on one thread-block cluster is available
   bool no_coop = false;             // never use the grid-barrier PCG (meshes solved concurrently)
   int tune_tpt = 0;                 // float32 far field: targets per thread (0 = heuristic)
   int tune_bps = 0;                 // float32 far field: target blocks per SM for the source split
@@ -387,6 +388,9 @@ int launch_dense_apply(Mesh* m, Surface* s, double scale, const double* v, doubl
 int dense_copy_out(Mesh* m, Surface* s, float scale, float* out, int ld_out);
 // launch attributes of the dense kernels, once per device (called by mesh creation)
 int init_dense_attributes();
+
+// ---- launch attributes of the cluster PCG, once per device (solver.cu)
+int init_pcg_attributes();
 
 // ---- one application of the block preconditioner (solver.cu), for the autotuner: prepares it at
 // the current Jacobian (dense surface blocks if requested) and applies it to v

@@ -17,8 +17,10 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
+#include "fp64_math.cuh"
 #include "pbfb_internal.cuh"
 #include "warp_sum.cuh"
 
@@ -276,23 +278,25 @@ __global__ void k_diag_inv(int nv, const int* __restrict__ ptr, const int* __res
 // the recurrence state st = {gamma_old, alpha_old, gamma_0} (st[3], st[4] receive alpha and beta).
 // f32_rules adds the float32 forms' stops: r.z at 1e-12 of its first value, or a non-positive or
 // huge alpha.  A zero r.z (e.g. a right-hand side that vanishes on the FEM rows) gives
-// alpha = beta = 0: nothing left to do.  Returns 1 to stop before this step's update.
+// alpha = beta = 0: nothing left to do.  Returns 1 to stop before this step's update.  The float64 latencies of
+// this chain are on every step's critical path, so it has one reciprocal; the two of the next step's state (st[5],
+// st[6]) are taken by cg_inverses_lane0 while the others use alpha and beta.
+__device__ __forceinline__ bool cg_rcp_range(double d) { return fabs(d) > 1e-290 && fabs(d) < 1e290; }
+
 __device__ __forceinline__ int cg_scalars_lane0(double gamma, double delta, int it, bool f32_rules, double* st) {
   if (it == 0) {
-    st[0] = 1.0;
-    st[1] = 1.0;
+    st[0] = 0.0;
     st[2] = gamma;
   }
   const double gamma_old = st[0], alpha_old = st[1];
   double beta = 0.0, alpha = 0.0;
   if (gamma != 0.0) {
-    if (it == 0 || gamma_old == 0.0 || alpha_old == 0.0) {
-      alpha = delta != 0.0 ? gamma / delta : 0.0;
-    } else {
-      beta = gamma / gamma_old;
-      const double den = delta - beta * gamma / alpha_old;
-      alpha = den != 0.0 ? gamma / den : 0.0;
+    double den = delta;
+    if (gamma_old != 0.0 && alpha_old != 0.0) {
+      beta = cg_rcp_range(gamma_old) ? gamma * st[5] : gamma / gamma_old;
+      den = delta - (cg_rcp_range(alpha_old) ? beta * gamma * st[6] : beta * gamma / alpha_old);
     }
+    if (den != 0.0) alpha = cg_rcp_range(den) ? gamma * rcp64(den) : gamma / den;
   }
   int s = 0;
   if (f32_rules && (!(gamma > 1e-12 * st[2]) || !(alpha > 0.0 && alpha < 3e38 && fabs(beta) < 3e38))) s = 1;
@@ -301,6 +305,12 @@ __device__ __forceinline__ int cg_scalars_lane0(double gamma, double delta, int 
   st[3] = alpha;
   st[4] = beta;
   return s;
+}
+
+// the reciprocals of the state for the next step (used where cg_rcp_range holds)
+__device__ __forceinline__ void cg_inverses_lane0(double* st) {
+  st[5] = rcp64(st[0]);
+  st[6] = rcp64(st[1]);
 }
 
 // The scalars of a Chronopoulos-Gear step from the two grid sums: warp 0 of every block reads the
@@ -312,7 +322,7 @@ __device__ __forceinline__ int cg_scalars_lane0(double gamma, double delta, int 
 // Returns true when the iteration is to stop before this step's update.
 __device__ __forceinline__ bool cg_step_scalars(const double* pa, const double* pb, int nb, int it, bool f32_rules,
                                                 double* alpha_out, double* beta_out) {
-  __shared__ double st[5];  // gamma_old, alpha_old, gamma_0, alpha, beta
+  __shared__ double st[7];  // gamma_old, alpha_old, gamma_0, alpha, beta, 1 / gamma_old, 1 / alpha_old
   __shared__ int stop;
   if (threadIdx.x < 32) {
     // lane l adds entries l, l + 32, ... in that order, loaded 8 at a time (independent loads)
@@ -343,6 +353,7 @@ __device__ __forceinline__ bool cg_step_scalars(const double* pa, const double* 
   *alpha_out = st[3];
   *beta_out = st[4];
   const bool s = stop != 0;
+  if (threadIdx.x == 0) cg_inverses_lane0(st);
   __syncthreads();
   return s;
 }
@@ -521,7 +532,7 @@ __global__ void __launch_bounds__(PCG_F32_T, 1)
   for (int i = tid; i < nv; i += stride) x_out[i] = (double)x[i];
 }
 
-// The float32 form with its state resident in registers, for meshes of at most PCG_RES_ROWS rows
+// The float32 form with its state resident in registers, for meshes of at most 992 rows
 // per SM, in the pipelined form of Ghysels and Vanroose (2014): with u = M r, w = A u, m = M w and
 // n = A m, every vector is updated by its own recurrence (z = n + beta z, q = m + beta q,
 // s = w + beta s, p = u + beta p; x += alpha p, r -= alpha s, u -= alpha q, w -= alpha z), so that
@@ -532,9 +543,11 @@ __global__ void __launch_bounds__(PCG_F32_T, 1)
 // the scalars (cg_step_scalars' arithmetic), so the float64 sums and divisions stay off the
 // critical path.  A thread owns one row for the whole solve: its row of the FEM block (at most
 // PCG_RES_CAP entries in registers; longer rows read the rest each step; the coupling columns past
-// nv are dropped) and its x, r, u, w, m, z, q, s, p and diagonal.  Blocks of 1 + 15 warps, one
-// per SM (4 warps per SM sub-partition: up to 128 registers a thread).  m and the block partials are double-buffered by step parity: a step reads one buffer
-// while it writes the other, and the barrier separates the two uses.
+// nv are dropped) and its x, r, u, w, m, z, q, s, p and diagonal.  One block per SM with the rows
+// spread evenly: 1 + 15 warps (up to 128 registers a thread) to 480 rows a block, 1 + 31 warps (64)
+// to 992.  m and the block partials are double-buffered by step parity: a step reads one buffer while
+// it writes the other, and the barrier separates the two uses.  GB300, 30 steps on 97,954 rows: 513 us
+// in the form above, 179 us here; 72,036 rows (480 a block) 154 us.
 // one row's product with a vector in global memory: the register-held entries, then the rest
 __device__ __forceinline__ float pipe_row_product(const int (&cidx)[16], const float (&cval)[16], int k_more,
                                                   int k_end, const int* __restrict__ col,
@@ -554,23 +567,24 @@ __device__ __forceinline__ float pipe_row_product(const int (&cidx)[16], const f
 }
 
 constexpr int PCG_RES_CAP = 16;  // (pipe_row_product's register entries)
-constexpr int PCG_RES_ROWS = 480;
-constexpr int PCG_PIPE_T = 32 + PCG_RES_ROWS;
+// threads of a block: 480 rows with up to 128 registers a thread, or 992 with 64 (larger meshes)
+constexpr int PCG_PIPE_T = 32 + 480, PCG_PIPE_T2 = 32 + 992;
 
-__global__ void __launch_bounds__(PCG_PIPE_T, 1)
-    k_pcg_pipe_f32(int nv, int iters, const int* __restrict__ ptr, const int* __restrict__ col,
+template <int NT>
+__global__ void __launch_bounds__(NT, 1)
+    k_pcg_pipe_f32(int nv, int rows, int iters, const int* __restrict__ ptr, const int* __restrict__ col,
                    const float* __restrict__ val, const double* __restrict__ b, const float* __restrict__ dinv,
                    double* __restrict__ x_out, float* __restrict__ mbuf, float* __restrict__ ubuf,
                    double* __restrict__ part) {
   namespace cg = cooperative_groups;
   cg::grid_group grid = cg::this_grid();
-  __shared__ float red[2][PCG_PIPE_T / 32];
-  __shared__ double st[5];
+  __shared__ float red[2][NT / 32];
+  __shared__ double st[7];
   __shared__ int stop;
-  const int nb = gridDim.x;
+  const int nb = gridDim.x, nw = blockDim.x >> 5;
   const int warp = threadIdx.x >> 5;
-  const int row = blockIdx.x * PCG_RES_ROWS + (int)threadIdx.x - 32;
-  const bool valid = warp > 0 && row < nv;
+  const int row = blockIdx.x * rows + (int)threadIdx.x - 32;  // rows a block: blockDim.x - 32 or fewer
+  const bool valid = warp > 0 && (int)threadIdx.x - 32 < rows && row < nv;
   const bool owner = valid;
   int cidx[PCG_RES_CAP];
   float cval[PCG_RES_CAP];
@@ -609,7 +623,7 @@ __global__ void __launch_bounds__(PCG_PIPE_T, 1)
     }
     __syncthreads();
     if (warp == 0) {
-      const bool in = threadIdx.x < PCG_PIPE_T / 32;
+      const bool in = (int)threadIdx.x < nw;
       double sg = in ? red[0][threadIdx.x] : 0.0, sd = in ? red[1][threadIdx.x] : 0.0;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
@@ -676,6 +690,7 @@ __global__ void __launch_bounds__(PCG_PIPE_T, 1)
       n = valid ? pipe_row_product(cidx, cval, k_more, k_end, col, val, nv, mbuf + (size_t)cur * nv) : 0.f;
     __syncthreads();
     if (stop) break;  // identical sums in every block: the same decision everywhere
+    if (threadIdx.x == 0) cg_inverses_lane0(st);
     if (owner) {
       const float a = (float)st[3], bt = (float)st[4];
       z = fmaf(bt, z, n);
@@ -695,6 +710,176 @@ __global__ void __launch_bounds__(PCG_PIPE_T, 1)
     }
   }
   if (owner) x_out[row] = (double)x;
+}
+
+// Small meshes: the whole inner PCG on one thread-block cluster of PCG_CL blocks.  What bounds a step there is the
+// chain of latencies -- gathers, block sums, barriers -- and a cluster's hardware barrier takes a fraction of a
+// grid barrier's 1.5 us; the block sums travel by writes into every block's shared memory before it.  A
+// thread owns a row, as in k_pcg_pipe_f32 (the columns as 16-bit pairs: rows are below 65,536), warp 0 takes the
+// sums and scalars.  float32: the pipelined form, one barrier a step, gathers of m.  float64: the
+// Chronopoulos-Gear form of k_pcg_coop, two barriers a step (its residual follows the recurrence of standard CG
+// to float64 rounding), gathers of z.  The vectors that other blocks read are stored to L2 (st.cg) and loaded after
+// a barrier, whose acquire drops stale L1 lines.
+// GB300, 30 steps, against the grid-wide forms: float64 552 rows 258 -> 154 us, 3528 rows 268 -> 180, 11,022 rows
+// 396 -> 302; float32 552 rows 157 -> 95 us, 3528 rows 159 -> 98, 15,862 rows 163 -> 135.
+constexpr int PCG_CL = 16;             // blocks of the cluster (non-portable size)
+constexpr int PCG_CL_T32 = 1024, PCG_CL_T64 = 768;  // most threads a block: 64 and 80 registers each
+
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT, 1)
+    k_pcg_cluster(int nv, int rows, int iters, const int* __restrict__ ptr, const int* __restrict__ col,
+                  const T* __restrict__ val, const double* __restrict__ b, const T* __restrict__ dinv,
+                  double* __restrict__ x_out, T* __restrict__ buf) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  constexpr bool F32 = sizeof(T) == 4;
+  __shared__ double red[2][NT / 32];
+  __shared__ double part[2][2][PCG_CL];  // [parity][dot][block]
+  __shared__ double st[7];
+  __shared__ int stop;
+  const int rank = (int)cl.block_rank(), nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int row = rank * rows + (int)threadIdx.x - 32;
+  const bool valid = warp > 0 && (int)threadIdx.x - 32 < rows && row < nv;
+  unsigned cidx[PCG_RES_CAP / 2];
+  T cval[PCG_RES_CAP];
+  int k_more = 0, k_end = 0;
+#pragma unroll
+  for (int t = 0; t < PCG_RES_CAP / 2; ++t) cidx[t] = 0;
+#pragma unroll
+  for (int t = 0; t < PCG_RES_CAP; ++t) cval[t] = (T)0;
+  if (valid) {
+    const int k0 = ptr[row], e = ptr[row + 1];
+#pragma unroll
+    for (int t = 0; t < PCG_RES_CAP; ++t) {
+      const int k = k0 + t;
+      const int c = k < e ? col[k] : nv;
+      cidx[t / 2] |= (unsigned)(c < nv ? c : row) << (16 * (t & 1));
+      if (c < nv) cval[t] = val[k];
+    }
+    k_more = k0 + PCG_RES_CAP;
+    k_end = e;
+  }
+  auto product = [&](const T* v) {
+    T g[PCG_RES_CAP];
+#pragma unroll
+    for (int t = 0; t < PCG_RES_CAP; ++t) g[t] = v[(cidx[t / 2] >> (16 * (t & 1))) & 0xffffu];
+    T acc = (T)0;
+#pragma unroll
+    for (int t = 0; t < PCG_RES_CAP; ++t) acc = fma(cval[t], g[t], acc);
+    for (int k = k_more; k < k_end; ++k) {
+      const int c = col[k];
+      if (c < nv) acc = fma(val[k], v[c], acc);
+    }
+    return acc;
+  };
+  // block sums of a and b (warp sums in T, the warps' values added in float64 in warp order) into every block's
+  // slot of parity par; the caller's next cluster barrier makes them visible
+  auto block_dots = [&](T a, T bb, int par) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      a += __shfl_down_sync(0xffffffffu, a, o);
+      bb += __shfl_down_sync(0xffffffffu, bb, o);
+    }
+    if (lane == 0) {
+      red[0][warp] = a;
+      red[1][warp] = bb;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      double sa = lane < nw ? red[0][lane] : 0.0, sb = lane < nw ? red[1][lane] : 0.0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        sa += __shfl_xor_sync(0xffffffffu, sa, o);
+        sb += __shfl_xor_sync(0xffffffffu, sb, o);
+      }
+      if (lane < PCG_CL) {
+        double* p = cl.map_shared_rank(&part[par][0][0], lane);
+        p[rank] = sa;
+        p[PCG_CL + rank] = sb;
+      }
+    }
+  };
+  // warp 0: the cluster's sums of parity par and the scalars of step it into st[3], st[4]
+  auto scalars = [&](int par, int it) {
+    double sa = lane < PCG_CL ? part[par][0][lane] : 0.0, sb = lane < PCG_CL ? part[par][1][lane] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      sa += __shfl_xor_sync(0xffffffffu, sa, o);
+      sb += __shfl_xor_sync(0xffffffffu, sb, o);
+    }
+    if (lane == 0) stop = cg_scalars_lane0(sa, sb, it, F32, st);
+  };
+  T x = (T)0, r = (T)0, di = (T)0;
+  if (valid) {
+    di = dinv[row];
+    r = (T)b[row];
+  }
+  if constexpr (F32) {
+    T* mbuf = buf;
+    T* ubuf = buf + 2 * (size_t)nv;
+    T u = di * r, w = (T)0, m = (T)0, z = (T)0, q = (T)0, sv = (T)0, p = (T)0;
+    if (valid) __stcg(ubuf + row, u);
+    cl.sync();
+    if (valid) {
+      w = product(ubuf);
+      m = di * w;
+      __stcg(mbuf + row, m);
+    }
+    block_dots(r * u, w * u, 0);
+    cl.sync();
+    for (int it = 0; it < iters; ++it) {
+      const int cur = it & 1, nxt = cur ^ 1;
+      T n = (T)0;
+      if (warp == 0)
+        scalars(cur, it);
+      else if (valid)
+        n = product(mbuf + (size_t)cur * nv);
+      __syncthreads();
+      if (stop) break;  // identical sums in every block: the same decision everywhere
+      if (threadIdx.x == 0) cg_inverses_lane0(st);
+      if (valid) {
+        const T a = (T)st[3], bt = (T)st[4];
+        z = fma(bt, z, n);
+        q = fma(bt, q, m);
+        sv = fma(bt, sv, w);
+        p = fma(bt, p, u);
+        x = fma(a, p, x);
+        r = fma(-a, sv, r);
+        u = fma(-a, q, u);
+        w = fma(-a, z, w);
+        m = di * w;
+        __stcg(mbuf + (size_t)nxt * nv + row, m);
+      }
+      if (it + 1 < iters) {
+        block_dots(r * u, w * u, nxt);
+        cl.sync();
+      }
+    }
+  } else {
+    T* zbuf = buf;
+    T z = di * r, p = (T)0, q = (T)0;
+    if (valid) __stcg(zbuf + row, z);
+    cl.sync();
+    for (int it = 0; it < iters; ++it) {
+      const T w = valid ? product(zbuf) : (T)0;
+      block_dots(r * z, z * w, it & 1);
+      cl.sync();  // every gather of z is done
+      if (warp == 0) scalars(it & 1, it);
+      __syncthreads();
+      if (threadIdx.x == 0) cg_inverses_lane0(st);
+      if (valid) {
+        const T a = st[3], bt = st[4];
+        p = fma(bt, p, z);
+        q = fma(bt, q, w);
+        x = fma(a, p, x);
+        r = fma(-a, q, r);
+        z = di * r;
+        __stcg(zbuf + row, z);
+      }
+      cl.sync();
+    }
+  }
+  if (valid) x_out[row] = (double)x;
 }
 
 // The same iteration with the FEM block in sliced ELL form (slices of 32 consecutive rows, each
@@ -1001,6 +1186,52 @@ static int build_sell(Mesh* m) {
   return PBFB_OK;
 }
 
+// launch configuration of one cluster of PCG_CL blocks of nt threads
+struct ClusterLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  ClusterLaunch(int nt, cudaStream_t stream) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = PCG_CL;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(PCG_CL);
+    cfg.blockDim = dim3(nt);
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+  }
+};
+
+// whether the device can hold such a cluster at the kernel's largest block
+template <class K>
+static bool cluster_fits(K kernel, int nt) {
+  int n = 0;
+  const bool ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+  ClusterLaunch L(nt, 0);
+  if (!ok || cudaOccupancyMaxActiveClusters(&n, kernel, &L.cfg) != cudaSuccess) n = 0;
+  cudaGetLastError();
+  return n >= 1;
+}
+
+// The cluster PCG's attributes, once per device (called by mesh creation, before any launch); whether it can run
+static std::mutex g_cluster_mu;
+static signed char g_cluster[64] = {};  // 0 not asked, 1 available, -1 not
+int init_pcg_attributes() {
+  int dev = 0;
+  PB_CUDA(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lk(g_cluster_mu);
+  if (dev < 64 && g_cluster[dev] == 0)
+    g_cluster[dev] = cluster_fits(k_pcg_cluster<float, PCG_CL_T32>, PCG_CL_T32) &&
+                             cluster_fits(k_pcg_cluster<double, PCG_CL_T64>, PCG_CL_T64)
+                         ? 1
+                         : -1;
+  return PBFB_OK;
+}
+static bool pcg_cluster_available(int dev) {
+  std::lock_guard<std::mutex> lk(g_cluster_mu);
+  return dev < 64 && g_cluster[dev] == 1;
+}
+
 static int prepare_block_precond(Mesh* m, bool dense) {
   m->dense_m = dense && !m->full && m->sm.nv <= DENSE_V_MAX;
   m->dense_s = dense && m->ss.nv <= DENSE_V_MAX;
@@ -1024,9 +1255,11 @@ static int prepare_block_precond(Mesh* m, bool dense) {
     PB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perf4, k_pcg_coop_f32<4>, PCG_F32_T, 0));
     PB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perf2, k_pcg_coop_f32<2>, PCG_F32_T, 0));
     m->coop_blocks_f32 = (coop && std::min({perf8, perf4, perf2}) >= 1) ? nsm : -1;
-    int perr = 0;
-    PB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perr, k_pcg_pipe_f32, PCG_PIPE_T, 0));
-    m->coop_blocks_pipe = (coop && perr >= 1) ? nsm : 0;
+    int perr = 0, perr2 = 0;
+    PB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perr, k_pcg_pipe_f32<PCG_PIPE_T>, PCG_PIPE_T, 0));
+    PB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perr2, k_pcg_pipe_f32<PCG_PIPE_T2>, PCG_PIPE_T2, 0));
+    m->coop_blocks_pipe = (coop && perr >= 1 && perr2 >= 1) ? nsm : 0;
+    m->pcg_cluster = pcg_cluster_available(m->dev);
     // all resident blocks (memory-level parallelism for the SpMV phases), but no more than
     // one pass of 8 lanes per row needs
     int want = (m->tune_pcg_bps > 0 ? std::min(per, m->tune_pcg_bps) : per) * nsm;
@@ -1157,6 +1390,22 @@ static int block_precond(Mesh* m, const double* v, double* z, int inner_iters) {
       PB_LAUNCHED(m);
       return PBFB_OK;
     }
+    // Rows a block of the cluster, in whole warps: the cluster form wherever its blocks' registers hold the rows
+    // (float64 11,776, float32 15,872), as its barrier is the cheaper one at every such size: 154 against 258 us at
+    // 552 rows, 302 against 396 us at 11,022 (float64); 95 against 157 and 135 against 163 us at 552 and 15,862.
+    const int crow = ((nv + PCG_CL - 1) / PCG_CL + 31) / 32 * 32;
+    if (m->pcg_cluster && crow <= (m->pcg_f32 ? PCG_CL_T32 : PCG_CL_T64) - 32) {
+      ClusterLaunch L(32 + crow, m->stream);
+      if (m->pcg_f32)
+        PB_CUDA(cudaLaunchKernelEx(&L.cfg, k_pcg_cluster<float, PCG_CL_T32>, nv, crow, inner_iters, sp, sc2,
+                                   (const float*)m->pvalf.p, (const double*)vu, (const float*)m->pdinvf.p, z,
+                                   m->pcgf.p));
+      else
+        PB_CUDA(cudaLaunchKernelEx(&L.cfg, k_pcg_cluster<double, PCG_CL_T64>, nv, crow, inner_iters, sp, sc2, pv,
+                                   (const double*)vu, dinv, z, pz));
+      PB_LAUNCHED(m);
+      return PBFB_OK;
+    }
     if (m->pcg_f32) {
       // float32 vectors, n each: the FEM rows' coupling columns (>= nv) read z there, which stays 0
       float* fx = m->pcgf.p;
@@ -1168,13 +1417,16 @@ static int block_precond(Mesh* m, const double* v, double* z, int inner_iters) {
       const float* fv = m->pvalf.p;
       const float* fd = m->pdinvf.p;
       void* argsf[] = {&nvv, &iters, &sp, &sc2, &fv, (void*)&vu, &fd, &z, &fx, &fr, &fz, &fp, &fq, &fw, &part};
-      if (nv <= PCG_RES_ROWS * m->coop_blocks_pipe) {
-        int nbr = (nv + PCG_RES_ROWS - 1) / PCG_RES_ROWS;
+      if (nv <= (PCG_PIPE_T2 - 32) * m->coop_blocks_pipe) {
+        // a block an SM where that leaves each at least 480 rows, the rows spread evenly in whole warps
+        int rows = std::max(PCG_PIPE_T - 32, ((nv + m->coop_blocks_pipe - 1) / m->coop_blocks_pipe + 31) / 32 * 32);
+        const int nbr = (nv + rows - 1) / rows;
         float* mb = fx;  // m, two buffers of nv (the x and r vectors of the form below)
         float* ub = fq;
-        void* argsr[] = {&nvv, &iters, &sp, &sc2, &fv, (void*)&vu, &fd, &z, &mb, &ub, &part};
-        PB_CUDA(cudaLaunchCooperativeKernel((const void*)k_pcg_pipe_f32, dim3(nbr), dim3(PCG_PIPE_T), argsr, 0,
-                                            m->stream));
+        void* argsr[] = {&nvv, &rows, &iters, &sp, &sc2, &fv, (void*)&vu, &fd, &z, &mb, &ub, &part};
+        const void* kr = rows + 32 <= PCG_PIPE_T ? (const void*)k_pcg_pipe_f32<PCG_PIPE_T>
+                                                 : (const void*)k_pcg_pipe_f32<PCG_PIPE_T2>;
+        PB_CUDA(cudaLaunchCooperativeKernel(kr, dim3(nbr), dim3(rows + 32), argsr, 0, m->stream));
         PB_LAUNCHED(m);
         return PBFB_OK;
       }

@@ -1,0 +1,90 @@
+"""The inner PCG's forms, the Coulomb sums and the dense single layer at the sizes where
+their blocks, chunks and forms change."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def dev(a):
+    import torch
+    return torch.as_tensor(np.ascontiguousarray(a, np.float64), device="cuda")
+
+
+# FEM rows: 24, 36 (most blocks of the cluster idle), 552 (a ragged warp), 11,772 / 11,808 (the float64 cluster
+# form's last size, and past it), 15,862 / 16,240 (float32's), 72,036 / 80,212 (both block sizes of the
+# grid-wide form), 149,812 / 155,574 (its last size, and past it; on 152 SMs).
+# One GMRES step gives the preconditioned vector up to a factor; a few PCG steps before convergence, so every
+# form gives the same iterate up to rounding: rows of at most about 30 terms, 7 steps, a tenfold growth per form
+# and unit roundoff u: 2000 u, times 5 for the dot products' part = 1e4 u.
+@pytest.mark.parametrize("nu,layers", [(1, 1), (1, 2), (3, 5), (14, 5), (7, 23), (12, 10), (9, 19), (20, 17), (27, 10),
+                                       (24, 25), (24, 26)])
+def test_inner_pcg_forms_agree(nu, layers):
+    from paper_2511_21713_gb300 import inputs, pbfb
+    case = inputs.sphere_case(nu=nu, a=4.0, R=8.0, layers=layers)
+    m = pbfb.Mesh.from_case(case)
+    assert m.n_v == (10 * nu * nu + 2) * (layers + 1)
+    m.set_params(case.eps_in, case.eps_out, case.kappa, case.T)
+    m.clear_jacobian()
+    b = dev(np.random.default_rng(nu).standard_normal(m.n))
+    for steps in (1, 7):
+        z = {}
+        for key, tuning in dict(sell=dict(pcg_lanes=1), f64=dict(pcg_precision=1), f32=dict(pcg_precision=2)).items():
+            m.apply_tuning(tuning)
+            x = dev(np.zeros(m.n))
+            with pytest.raises(pbfb.PbfbError) as e:
+                m.gmres(b, x, 1e-14, maxit=1, precond=pbfb.BLOCK, inner_iters=steps)
+            assert e.value.code == 3
+            y = x.cpu().numpy()[:m.n_v]
+            z[key] = y / np.linalg.norm(y)
+        assert np.linalg.norm(z["f64"] - z["sell"]) <= 1e4 * 2.0 ** -53, steps
+        assert np.linalg.norm(z["f32"] - z["sell"]) <= 1e4 * 2.0 ** -24, steps
+    m.close()
+
+
+# the sums over the charges run in chunks (1300 of them: several per block); they are linear in the charges, so
+# parts of the set add up to the whole: regrouped sums of float64 numbers, 1e-12 of the parts' magnitudes
+@pytest.mark.parametrize("nu", [1, 5, 14])
+def test_reaction_energies_add_up(nu):
+    from paper_2511_21713_gb300 import inputs, pbfb
+    case = inputs.sphere_case(nu=nu, a=4.0, R=6.0, layers=1)
+    m = pbfb.Mesh.from_case(case)
+    m.set_params(case.eps_in, case.eps_out, case.kappa, case.T)
+    rng = np.random.default_rng(nu)
+    q, z = 2.0 * (rng.random((1300, 3)) - 0.5), rng.standard_normal(1300)
+    xL, xNL = (dev(0.1 * rng.standard_normal(m.n)) for _ in range(2))
+
+    def energy(k):
+        m.charges_set(q[k], z[k])
+        return m.energy(xL, xNL)[1:3]
+    parts = [energy(k) for k in (slice(0, 1), slice(1, 4), slice(4, 300), slice(300, 1300))]
+    assert (np.abs(energy(slice(None)) - sum(parts)) <= 1e-12 * (1.0 + sum(map(np.abs, parts)))).all()
+    m.close()
+
+
+# triangles: 20, 1280 (one chunk), 1620, 3920 (several); columns of the float64 operator, symmetrised, against the
+# float32 matrix: float32 weights and kernel values, sums of at most 36 * 36 of them in a few pieces: 16 * 2^-24
+@pytest.mark.parametrize("nu", [1, 8, 9, 14])
+def test_dense_single_layer_columns(nu):
+    import torch
+    from paper_2511_21713_gb300 import inputs, pbfb
+    case = inputs.sphere_case(nu=nu, a=4.0, R=6.0, layers=1)
+    m = pbfb.Mesh.from_case(case)
+    m.set_params(case.eps_in, case.eps_out, case.kappa, case.T)
+    for which, n in ((pbfb.GAMMA_M, m.n_m), (pbfb.GAMMA_S, m.n_s)):
+        D = torch.zeros((n, n), dtype=torch.float32, device="cuda")
+        m.single_layer_dense(which, 0, D)
+        assert torch.equal(D, D.T)
+        D = D.cpu().numpy().astype(np.float64)
+        k = np.unique(np.r_[0, n // 3, n - 1])
+        V = np.empty((n, k.size))
+        for j, kj in enumerate(k):
+            x, y = dev(np.zeros(n)), dev(np.zeros(n))
+            x[kj] = 1.0
+            m.bem_apply(which, 0, x, y)
+            V[:, j] = y.cpu().numpy()
+        S = 0.5 * (V[k] + V[k].T)
+        assert np.abs(D[np.ix_(k, k)] - S).max() <= 2.0 ** -20 * np.abs(V).max()
+        # V itself is symmetric up to the quadrature of near pairs
+        assert np.abs(D[:, k] - V).max() <= 1e-3 * np.abs(V).max()
+    m.close()
