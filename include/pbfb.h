@@ -227,8 +227,8 @@ int pbfb_surface_vertices(const pbfb_mesh* mesh, int which, int32_t* out);
  * units of e) and computes <sum_k z_k / |x - x_k|, psi_i> on Gamma_m
  * (the Coulomb data of Sec. 2.3.1).  Charges must be finite; n_q >= 1.  On a
  * shell mesh every charge must lie strictly inside Gamma_m (in Omega_m, as the
- * three-region model of Sec. 2.1 places them), checked on the host by the
- * winding number of pbfb_check_charges before any GPU work; PBFB_ERR_INVALID
+ * three-region model of Sec. 2.1 places them), checked by the winding number of
+ * pbfb_check_charges before the charges are taken; PBFB_ERR_INVALID
  * otherwise, the mesh keeping its previous charges. */
 int pbfb_charges_set(pbfb_mesh* mesh, const double* xyz, const double* z, int32_t n_q);
 

@@ -885,14 +885,6 @@ int mesh_create(const double* xyz, int nv, const int* tets, int64_t nt, const in
     }
     m->gs_radius = std::sqrt(area / (4.0 * M_PI));
   }
-  if (!m->full) {
-    // Gamma_m's triangles (as stored: normal out of the solute) for the charges' winding numbers
-    m->gm_tri_xyz.resize(9 * (size_t)sm.nt);
-    for (int t = 0; t < sm.nt; ++t)
-      for (int a = 0; a < 3; ++a)
-        for (int d = 0; d < 3; ++d)
-          m->gm_tri_xyz[9 * (size_t)t + 3 * a + d] = xyz_h[3 * (size_t)sm.vmap_h[sm.tri_h[3 * t + a]] + d];
-  }
   for (int si = 0; si < 2; ++si) {
     const Surface& s = si == 0 ? sm : ss;
     if (m->full && si == 0) {
@@ -1014,18 +1006,13 @@ int check_charges_inside(const double* tri9, size_t nt, const double* q, int nq,
   winding_numbers(tri9, nt, q, nq, w.data());
   if (w_out) std::copy(w.begin(), w.end(), w_out);
   for (int k = 0; k < nq; ++k)
-    if (!(w[k] > 0.75)) {
-      set_error("charge %d at (%g, %g, %g) is not strictly inside Gamma_m (winding number %.3f)", k, q[3 * k],
-                q[3 * k + 1], q[3 * k + 2], w[k]);
-      return PBFB_ERR_INVALID;
-    }
+    if (!(w[k] > 0.75)) return charge_outside(k, q + 3 * (size_t)k, w[k]);
   return PBFB_OK;
 }
 
-int charges_inside_gamma_m(const Mesh* m, const double* q, int nq) {
-  const size_t nt = m->gm_tri_xyz.size() / 9;
-  if (nt == 0) return PBFB_OK;
-  return check_charges_inside(m->gm_tri_xyz.data(), nt, q, nq, nullptr);
+int charge_outside(int k, const double* q, double w) {
+  set_error("charge %d at (%g, %g, %g) is not strictly inside Gamma_m (winding number %.3f)", k, q[0], q[1], q[2], w);
+  return PBFB_ERR_INVALID;
 }
 
 }  // namespace pbfb

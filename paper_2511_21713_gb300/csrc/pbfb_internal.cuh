@@ -185,6 +185,7 @@ struct Mesh {
   DBuf<double> qxyz, qz;    // 3*nq SoA, nq
   DBuf<double> coul;        // nm: <sum z/|x-x_k|, psi_i> (no l_B/eps_m)
   DBuf<double> coul_ce;     // 2*nq of Gamma_m: the charges' potential and normal field sums (k_coulomb)
+  DBuf<double> wind;        // the inside check's points and chunk sums
   bool charges = false;
   // parameters
   double eps_m = 0, eps_s = 0, kappa = 0, T = 0, lB = 0, kT = 0, coef = 0;
@@ -266,7 +267,6 @@ struct Mesh {
   int64_t nt_m = 0;
   DBuf<int> tets_m;                 // 4*nt_m SoA
   DBuf<double> vol_m, a1m;          // Omega_m volumes; per slot: its stiffness (eps_m applied at fill)
-  std::vector<double> gm_tri_xyz;   // shell meshes: 9 per Gamma_m triangle (host), for the winding number
   std::vector<double> grid_xyz;     // 3*nv AoS (host), for locating the charges
   std::vector<int> tets_m_h;        // 4*nt_m AoS (host)
   std::vector<int> cell_ptr, cell_tet;  // uniform grid over the Omega_m tets' bounding boxes
@@ -302,8 +302,8 @@ size_t estimate_bytes(int64_t nv, int64_t nt, int64_t ngm, int64_t ngs, int rest
 // sum_k z_k v_i(x_k) over the Omega_m tets (a mesh with Omega_m); PBFB_ERR_INVALID for a charge
 // in none of them
 int point_load(Mesh* m, const double* q_xyz, const double* z, int nq, std::vector<double>& rho);
-int charges_inside_gamma_m(const Mesh* m, const double* q_xyz, int nq);
 int check_charges_inside(const double* tri9, size_t nt, const double* q, int nq, double* w_out);
+int charge_outside(int k, const double* q, double w);  // sets the error text, returns PBFB_ERR_INVALID
 }  // namespace pbfb
 pbfb::Mesh* pbfb_mesh_internal(pbfb_mesh* h);
 namespace pbfb {
@@ -341,6 +341,8 @@ int launch_bem_far(Mesh* m, Surface* s, const double* x, const double* lam, doub
 int launch_bem_far_ff(Mesh* m, Surface* s, const double* x, const double* lam, double cs, double cd,
                       double kappa, double* y, bool accumulate);
 int launch_coulomb(Mesh* m);
+// winding numbers of Gamma_m at nq host points (SoA), on the device (pbfb_check_charges' formula)
+int launch_winding_numbers(Mesh* m, const double* soa, int nq, double* w);
 int launch_reaction_energy(Mesh* m, const double* xL, const double* xNL, double* out_dev);
 int bem_apply_noalloc(Mesh* m, int which, int op, const double* x, double* y);
 

@@ -2270,13 +2270,18 @@ int charges_set(Mesh* m, const double* xyz, const double* z, int n_q) {
       return PBFB_ERR_INVALID;
     }
   }
-  if (!m->full) PB_TRY(charges_inside_gamma_m(m, xyz, n_q));
+  std::vector<double> rho;
   if (m->full) {
     // point loads of the charges on the Omega_m tets (Eq. fembem_matrix's right-hand side)
-    std::vector<double> rho;
     PB_TRY(point_load(m, xyz, z, n_q, rho));
-    PB_TRY(m->rho.upload(rho.data(), rho.size(), m->stream));
+  } else {
+    // inside Gamma_m by its winding numbers, from buffers of the check's own: a refusal leaves the charges as they were
+    std::vector<double> w(n_q);
+    PB_TRY(launch_winding_numbers(m, soa.data(), n_q, w.data()));
+    for (int k = 0; k < n_q; ++k)
+      if (!(w[k] > 0.75)) return charge_outside(k, xyz + 3 * (size_t)k, w[k]);
   }
+  if (m->full) PB_TRY(m->rho.upload(rho.data(), rho.size(), m->stream));
   PB_TRY(ensure(m->qxyz, soa.size()));
   PB_TRY(ensure(m->qz, n_q));
   PB_CUDA(cudaMemcpyAsync(m->qxyz.p, soa.data(), soa.size() * sizeof(double), cudaMemcpyHostToDevice, m->stream));

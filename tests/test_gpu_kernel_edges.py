@@ -1,4 +1,4 @@
-"""The inner PCG's forms, the Coulomb sums and the dense single layer at the sizes where
+"""The inner PCG's forms, the winding numbers, the Coulomb sums and the dense single layer at the sizes where
 their blocks, chunks and forms change."""
 import numpy as np
 import pytest
@@ -39,6 +39,34 @@ def test_inner_pcg_forms_agree(nu, layers):
             z[key] = y / np.linalg.norm(y)
         assert np.linalg.norm(z["f64"] - z["sell"]) <= 1e4 * 2.0 ** -53, steps
         assert np.linalg.norm(z["f32"] - z["sell"]) <= 1e4 * 2.0 ** -24, steps
+    m.close()
+
+
+# a block takes 64 charges and a chunk of the triangles; the refused charge is the last one
+@pytest.mark.parametrize("nq", [1, 64, 65, 1300])
+@pytest.mark.parametrize("nu", [1, 7])
+def test_charges_inside_check(nq, nu):
+    from paper_2511_21713_gb300 import inputs, pbfb
+    case = inputs.sphere_case(nu=nu, a=4.0, R=6.0, layers=1)
+    m = pbfb.Mesh.from_case(case)
+    rng = np.random.default_rng(nq)
+    q = rng.standard_normal((nq, 3))
+    q *= 3.0 / np.linalg.norm(q, axis=1)[:, None] * rng.random((nq, 1))
+    m.charges_set(q, rng.standard_normal(nq))
+    P = np.asarray(case.xyz)[np.asarray(case.gm_tris)[5]]
+    # the face's plane test: 1e-12 of the product of the distances; a point off it by more belongs to a side
+    n = np.cross(P[1] - P[0], P[2] - P[0])
+    n /= np.linalg.norm(n) * np.sign(n @ P[0])
+    c = P.mean(axis=0)
+    for p, w in ((c, 0.5), (P[1], 0.5), (c + 1e-6 * n, 0.0), (2.0 * c, 0.0), (100.0 * c, 0.0)):
+        bad = q.copy()
+        bad[-1] = p
+        with pytest.raises(pbfb.PbfbError) as e:
+            m.charges_set(bad, np.ones(nq))
+        assert e.value.code == 1
+        assert f"charge {nq - 1} " in str(e.value) and f"winding number {w:.3f}" in str(e.value).replace("-0.000", "0.000")
+    q[-1] = c - 1e-6 * n
+    m.charges_set(q, np.ones(nq))
     m.close()
 
 
