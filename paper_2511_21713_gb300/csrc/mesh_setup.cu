@@ -916,7 +916,7 @@ int mesh_create(const double* xyz, int nv, const int* tets, int64_t nt, const in
   if ((st = m->a1.alloc(m->snnz))) return fail(st);
   if ((st = m->vol.alloc(nti))) return fail(st);
   if ((st = m->tloc.alloc(14 * (size_t)nti))) return fail(st);
-  if ((st = m->red.alloc((size_t)152 * 7 * 64 + 1024))) return fail(st);
+  if ((st = m->red.alloc((size_t)152 * 7 * (OMEGA_MAX + 1) + 1024))) return fail(st);
   if ((st = m->scal.alloc(8192))) return fail(st);
   if ((st = m->red2.alloc(9 * (size_t)std::max(sm.npair, ss.npair)))) return fail(st);
   if (cudaMallocHost((void**)&m->pinned, 4096 * sizeof(double)) != cudaSuccess) {

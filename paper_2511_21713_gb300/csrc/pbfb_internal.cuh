@@ -43,6 +43,12 @@ const char* last_error();
 constexpr int QS = 6;
 constexpr int QT = 14;
 
+// Relaxation factors of one batch, passed to the kernels by value.
+constexpr int OMEGA_MAX = 64;
+struct OmegaSet {
+  double v[OMEGA_MAX];
+};
+
 // Owned device allocation.
 template <class T>
 struct DBuf {
@@ -314,14 +320,16 @@ int init_quadrature();
 // ---- fem_kernels.cu
 int launch_tet_volumes(Mesh* m, const int* tets, int64_t nt, double* vol);
 int launch_stiffness_local(Mesh* m, const int* tets, int64_t nt, const double* vol, double* loc10);
-// ff: the tet-local entries are float-float pairs (the mixed precision's sinh-scheme kernels)
 int launch_gather(Mesh* m, int nslots, const int* ptr, const int* idx, const double* local,
-                  const double* base, double scale, double* out, bool ff = false);
+                  const double* base, double scale, double* out);
+// the element loop's tet-local entries (m->tloc; ff: float-float pairs) into the operator values and N_out (or null)
+int launch_assemble_gather(Mesh* m, bool ff, double* N_out);
 // *ff tells whether loc was written as float-float pairs
 int launch_element_nl(Mesh* m, int scheme, const double* u, double coef, double* loc, bool* ff);
 int launch_spmv(Mesh* m, const double* x, double* y);
 int launch_omega_elements(Mesh* m, int scheme, const double* u, const double* du,
-                          const double* omegas_dev, int nomega, double coef, double* loc, bool* ff);
+                          const double* omegas, int nomega, double coef, double* loc, bool* ff);
+// dots_dev: 7 per omega, then the surface rows' p.c and c.c, and p.p
 int launch_omega_dots(Mesh* m, int nomega, const double* loc, const double* c, const double* p,
                       double* dots_dev, bool ff);
 // the ion integral of u1 + u2

@@ -1086,9 +1086,7 @@ static int set_params(Mesh* m, double eps_in, double eps_out, double kappa, doub
 static int assemble(Mesh* m, int scheme, const double* u, double* N_out) {
   bool ff = false;
   PB_TRY(launch_element_nl(m, scheme, u, m->coef, m->tloc.p, &ff));
-  PB_TRY(launch_gather(m, m->snnz, m->jg_ptr.p, m->jg_idx.p, m->tloc.p, m->s_base.p, 1.0, m->s_val.p, ff));
-  if (N_out)
-    PB_TRY(launch_gather(m, m->nv, m->ng_ptr.p, m->ng_idx.p, m->tloc.p + 10 * m->nt, nullptr, 1.0, N_out, ff));
+  PB_TRY(launch_assemble_gather(m, ff, N_out));
   return PBFB_OK;
 }
 
@@ -1701,25 +1699,19 @@ static int gmres(Mesh* m, const double* b, double* x, double tol, int restart, i
 // Batched a7: dots (host, nomega x 8) = (p+r').r, (p+r').p, (p+r').r', r.r'', p.r'', r.r, p.r, p.p
 static int omega_eval(Mesh* m, int scheme, const double* u, const double* du, const double* c, const double* p,
                       const double* omegas, int nomega, double* dots) {
-  if (nomega < 1 || nomega > 64) {
+  if (nomega < 1 || nomega > OMEGA_MAX) {
     set_error("n_omega must be in [1, 64]");
     return PBFB_ERR_INVALID;
   }
   PB_TRY(ensure(m->wloc, (size_t)nomega * 12 * m->nt));
-  // constant (omega-independent) parts over the surface rows, and p.p
-  const int nv = m->nv, n = m->n, nb = n - nv;
-  double* dv = m->scal.p;  // [0, 64) omegas, [64, ...) results
-  std::memcpy(m->pinned, omegas, nomega * sizeof(double));
-  PB_CUDA(cudaMemcpyAsync(dv, m->pinned, nomega * sizeof(double), cudaMemcpyHostToDevice, m->stream));
+  double* dv = m->scal.p;  // 7 per omega, then the surface rows' p.c and c.c, and p.p
   bool ff = false;
-  PB_TRY(launch_omega_elements(m, scheme, u, du, dv, nomega, m->coef, m->wloc.p, &ff));
-  PB_TRY(launch_omega_dots(m, nomega, m->wloc.p, c, p, dv + 64, ff));
-  PB_TRY(dot_dev(m, p + nv, c + nv, nb, dv + 64 + 7 * 64));
-  PB_TRY(dot_dev(m, c + nv, c + nv, nb, dv + 64 + 7 * 64 + 1));
-  PB_TRY(dot_dev(m, p, p, n, dv + 64 + 7 * 64 + 2));
-  PB_CUDA(cudaMemcpyAsync(m->pinned, dv + 64, (7 * 64 + 3) * sizeof(double), cudaMemcpyDeviceToHost, m->stream));
+  PB_TRY(launch_omega_elements(m, scheme, u, du, omegas, nomega, m->coef, m->wloc.p, &ff));
+  PB_TRY(launch_omega_dots(m, nomega, m->wloc.p, c, p, dv, ff));
+  PB_CUDA(cudaMemcpyAsync(m->pinned, dv, (7 * nomega + 3) * sizeof(double), cudaMemcpyDeviceToHost, m->stream));
   PB_CUDA(cudaStreamSynchronize(m->stream));
-  const double pcb = m->pinned[7 * 64], ccb = m->pinned[7 * 64 + 1], pp = m->pinned[7 * 64 + 2];
+  const double* k3 = m->pinned + 7 * nomega;
+  const double pcb = k3[0], ccb = k3[1], pp = k3[2];
   for (int o = 0; o < nomega; ++o) {
     const double* f = m->pinned + 7 * o;  // p.r, r'.r, r'.p, r'.r', r.r'', p.r'', r.r (FEM rows)
     double pr = f[0] + pcb;

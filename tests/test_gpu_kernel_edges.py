@@ -116,3 +116,40 @@ def test_dense_single_layer_columns(nu):
         # V itself is symmetric up to the quadrature of near pairs
         assert np.abs(D[:, k] - V).max() <= 1e-3 * np.abs(V).max()
     m.close()
+
+
+# float-float element kernels against the float64 ones, over the table's range: u near 0, at and between table
+# points, past the first 512 of them (|u| > ln 2), up to the end of the float-float range (60) and past it, zeros,
+# tiny and huge values; vertices on both sides of the two-lanes-a-vertex rule (19,456 unknowns), one and several
+# omegas.  Each sum has 24 tets of 14 points, a product of a few roundings of 2^-47 each: 1e-12 of the sum of
+# magnitudes, which is at most the largest entry where all terms have a sign.
+@pytest.mark.parametrize("nu,layers", [(2, 1), (9, 20), (14, 10)])
+@pytest.mark.parametrize("scheme", ["HS", "T3", "T7"])
+def test_float_float_elements(nu, layers, scheme):
+    from paper_2511_21713_gb300 import inputs, pbfb
+    case = inputs.sphere_case(nu=nu, a=4.0, R=8.0, layers=layers)
+    m = pbfb.Mesh.from_case(case)
+    rng = np.random.default_rng(nu)
+    for scale in (0.0, 1e-20, 1e-4, np.log(2.0) / 512, 0.7, 5.0, 59.0, 70.0):
+        u = scale * rng.random(m.n_v)
+        u[::7] = scale
+        du = 0.01 * (scale + 1e-3) * rng.random(m.n_v)
+        c, p = rng.standard_normal(m.n), rng.standard_normal(m.n)
+        out = {}
+        for prec in (pbfb.FP64, pbfb.MIXED):
+            # float64's sinh is exact to 1e-16 absolutely: for the small fields its reference is T7 (u^9 / 9! away)
+            sch = pbfb.T7 if prec == pbfb.FP64 and scheme == "HS" and scale < 0.01 else getattr(pbfb, scheme)
+            m.set_params(case.eps_in, case.eps_out, case.kappa, case.T, prec)
+            N = dev(np.zeros(m.n_v))
+            m.assemble(sch, dev(u), N)
+            om = [m.omega_eval(sch, dev(u), dev(du), dev(c), dev(p), o) for o in ([0.5], [0.0, 0.25, 0.5, 1.0, 2.0])]
+            out[prec] = N.cpu().numpy(), m.fem_rows()[2], om
+        (N0, J0, o0), (N1, J1, o1) = out[pbfb.FP64], out[pbfb.MIXED]
+        assert np.abs(N1 - N0).max() <= 1e-12 * np.abs(N0).max() + 1e-300
+        assert np.abs(J1 - J0).max() <= 1e-12 * np.abs(J0).max()
+        for a, b in zip(o0, o1):
+            # every dot is at most |p + r'| or |r| times another: bounded by the batch's largest squares
+            assert np.isfinite(a).all()
+            assert np.abs(a - b).max() <= 1e-12 * np.abs(a).max() * np.sqrt(m.n)
+        assert np.allclose(o1[0][0], o1[1][2], rtol=1e-13, atol=1e-13 * np.abs(o1[1]).max())
+    m.close()
