@@ -11,8 +11,9 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
-#include <map>
+#include <exception>
 #include <string>
+#include <system_error>
 #include <thread>
 #include <unordered_map>
 #include <vector>
@@ -26,21 +27,65 @@ namespace {
 
 thread_local std::string g_err;
 
-// counting sort of (key, value) pairs by key in [0, nkeys): returns ptr (nkeys+1) and values
-void bucket(const std::vector<int>& keys, const std::vector<int>& vals, int nkeys, std::vector<int>& ptr,
-            std::vector<int>& out) {
+// f(k, i0, i1) for a partition of [0, n) into ranges k = 0, 1, ... on up to 16 host threads, each with `grain` items
+// or more; the same n and grain give the same partition.  An exception of a range is rethrown here.
+constexpr int HOST_THREADS = 16;
+template <class F>
+void parallel_ranges(int64_t n, int64_t grain, F f) {
+  const int64_t hw = std::max(1u, std::min((unsigned)HOST_THREADS, std::thread::hardware_concurrency()));
+  const int nth = (int)std::max<int64_t>(1, std::min(hw, n / grain));
+  std::exception_ptr err[HOST_THREADS];
+  auto run = [&](int k) {
+    try {
+      f(k, n * k / nth, n * (k + 1) / nth);
+    } catch (...) {
+      err[k] = std::current_exception();
+    }
+  };
+  std::thread th[HOST_THREADS];
+  int k = 1;
+  try {
+    for (; k < nth; ++k) th[k] = std::thread(run, k);
+  } catch (const std::system_error&) {  // no more threads: the rest runs here
+  }
+  const int started = k;
+  run(0);
+  for (; k < nth; ++k) run(k);
+  for (int q = 1; q < started; ++q) th[q].join();
+  for (int q = 0; q < nth; ++q)
+    if (err[q]) std::rethrow_exception(err[q]);
+}
+
+// counting sort of the values val(e), e = 0..n-1, by keys[e] in [0, nkeys): ptr (nkeys + 1) and the values, in
+// ascending e within a key.  A thread takes a range of the keys and reads all of them (sequentially: a fraction of
+// the scattered writes).
+template <class V>
+void bucket(const int* keys, int64_t n, int nkeys, V val, std::vector<int>& ptr, std::vector<int>& out) {
   ptr.assign(nkeys + 1, 0);
-  for (int k : keys) ptr[k + 1]++;
+  out.resize(n);
+  auto ranges = [&](auto f) { parallel_ranges(n < 40000 ? 1 : nkeys, n < 40000 ? 1 : std::max(1, nkeys / 16), f); };
+  auto clip = [&](int64_t& k0, int64_t& k1) {
+    if (n < 40000) k0 = 0, k1 = nkeys;
+  };
+  ranges([&](int, int64_t k0, int64_t k1) {
+    clip(k0, k1);
+    for (int64_t e = 0; e < n; ++e)
+      if (keys[e] >= k0 && keys[e] < k1) ptr[keys[e] + 1]++;
+  });
   for (int i = 0; i < nkeys; ++i) ptr[i + 1] += ptr[i];
-  out.resize(keys.size());
   std::vector<int> pos(ptr.begin(), ptr.end() - 1);
-  for (size_t e = 0; e < keys.size(); ++e) out[pos[keys[e]]++] = vals[e];
+  ranges([&](int, int64_t k0, int64_t k1) {
+    clip(k0, k1);
+    for (int64_t e = 0; e < n; ++e)
+      if (keys[e] >= k0 && keys[e] < k1) out[pos[keys[e]]++] = val(e);
+  });
 }
 
 struct HostSurface {
   std::vector<int> tri;    // local ids
   std::vector<int> verts;  // shell ids
   std::vector<double> P;   // nt*9 corner coordinates
+  std::vector<int> iptr, inc;  // per vertex: its triangles' entries 3 t + a, ascending
 };
 
 // Triangle-pair classification (ordered pairs: test t, trial s): touching pairs (identical, common
@@ -50,19 +95,12 @@ struct HostSurface {
 // smaller index), within radius 2 h of that triangle, so every pair is found once whatever the
 // spread of triangle sizes; host threads over the triangles.  Each row (test t) lists its trial
 // triangles in ascending order.
-void classify_pairs(const HostSurface& hs, std::vector<int>& pt, std::vector<int>& ps, std::vector<int>& cls,
-                    std::vector<int>& perm) {
+// pptr: the pairs of test t are pptr[t] .. pptr[t + 1] - 1.
+void classify_pairs(const HostSurface& hs, std::vector<int>& pptr, std::vector<int>& pt, std::vector<int>& ps,
+                    std::vector<int>& cls, std::vector<int>& perm) {
   const int nt = (int)hs.tri.size() / 3;
-  const int nv = (int)hs.verts.size();
-  std::vector<int> iptr(nv + 1, 0), inc(3 * (size_t)nt);
-  for (int t = 0; t < nt; ++t)
-    for (int a = 0; a < 3; ++a) ++iptr[hs.tri[3 * t + a] + 1];
-  for (int v = 0; v < nv; ++v) iptr[v + 1] += iptr[v];
-  {
-    std::vector<int> fill(iptr.begin(), iptr.end() - 1);
-    for (int t = 0; t < nt; ++t)
-      for (int a = 0; a < 3; ++a) inc[fill[hs.tri[3 * t + a]]++] = t;
-  }
+  const std::vector<int>& iptr = hs.iptr;
+  const std::vector<int>& inc = hs.inc;
   std::vector<double> cen(3 * (size_t)nt), h(nt);
   double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
   for (int t = 0; t < nt; ++t) {
@@ -109,16 +147,14 @@ void classify_pairs(const HostSurface& hs, std::vector<int>& pt, std::vector<int
     for (int t = 0; t < nt; ++t) ctri[fill[cof[t]]++] = t;
   }
   // near pairs, both orientations, from per-thread buffers merged in thread (= triangle) order
-  const int nth = (int)std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
-  std::vector<std::vector<int>> found(nth);
-  auto search = [&](int k) {
+  std::vector<int> found[HOST_THREADS];
+  parallel_ranges(nt, 32, [&](int k, int64_t t0, int64_t t1) {
     std::vector<int> stamp(nt, -1);
     std::vector<int>& out = found[k];
-    const int t0 = (int)((int64_t)nt * k / nth), t1 = (int)((int64_t)nt * (k + 1) / nth);
-    for (int t = t0; t < t1; ++t) {
+    for (int t = (int)t0; t < (int)t1; ++t) {
       for (int a = 0; a < 3; ++a) {
         const int v = hs.tri[3 * t + a];
-        for (int q = iptr[v]; q < iptr[v + 1]; ++q) stamp[inc[q]] = t;
+        for (int q = iptr[v]; q < iptr[v + 1]; ++q) stamp[inc[q] / 3] = t;
       }
       const double* c = &cen[3 * (size_t)t];
       const double r = 2.0 * h[t];
@@ -144,13 +180,7 @@ void classify_pairs(const HostSurface& hs, std::vector<int>& pt, std::vector<int
             }
           }
     }
-  };
-  {
-    std::vector<std::thread> th;
-    for (int k = 1; k < nth; ++k) th.emplace_back(search, k);
-    search(0);
-    for (auto& x : th) x.join();
-  }
+  });
   // rows: near partners of every triangle (both orientations), counting sort by row
   std::vector<int> nptr(nt + 1, 0);
   for (const auto& f : found)
@@ -168,60 +198,81 @@ void classify_pairs(const HostSurface& hs, std::vector<int>& pt, std::vector<int
         near[fill[f[q + 1]]++] = f[q];
       }
   }
-  std::vector<int> cnt(nt, 0), touched;
-  std::vector<std::array<int, 2>> row;  // (s, class)
-  for (int t = 0; t < nt; ++t) {
-    touched.clear();
-    row.clear();
-    for (int a = 0; a < 3; ++a) {
-      const int v = hs.tri[3 * t + a];
-      for (int q = iptr[v]; q < iptr[v + 1]; ++q) {
-        const int u = inc[q];
-        if (cnt[u] == 0) touched.push_back(u);
-        cnt[u]++;
-      }
-    }
-    for (int u : touched) {
-      const int c = cnt[u];
-      row.push_back({u, c == 3 ? PAIR_IDENTICAL : (c == 2 ? PAIR_EDGE : PAIR_VERTEX)});
-    }
-    for (int q = nptr[t]; q < nptr[t + 1]; ++q) row.push_back({near[q], PAIR_NEAR});
-    std::sort(row.begin(), row.end());
-    for (auto& e : row) {
-      int u = e[0], c = e[1];
-      int p[6] = {0, 1, 2, 0, 1, 2};
-      const int* T = &hs.tri[3 * t];
-      const int* S = &hs.tri[3 * u];
-      if (c == PAIR_EDGE) {
-        // shared vertices in the test triangle's order go to reference vertices 0 and 1
-        int sh[2], ns = 0;
-        for (int a = 0; a < 3; ++a)
-          for (int b = 0; b < 3; ++b)
-            if (T[a] == S[b]) sh[ns++] = a;
-        int sb[2];
-        for (int k = 0; k < 2; ++k)
-          for (int b = 0; b < 3; ++b)
-            if (S[b] == T[sh[k]]) sb[k] = b;
-        p[0] = sh[0]; p[1] = sh[1]; p[2] = 3 - sh[0] - sh[1];
-        p[3] = sb[0]; p[4] = sb[1]; p[5] = 3 - sb[0] - sb[1];
-      } else if (c == PAIR_VERTEX) {
-        int ia = 0, ib = 0;
-        for (int a = 0; a < 3; ++a)
-          for (int b = 0; b < 3; ++b)
-            if (T[a] == S[b]) { ia = a; ib = b; }
-        for (int k = 0; k < 3; ++k) {
-          p[k] = (ia + k) % 3;
-          p[3 + k] = (ib + k) % 3;
+  struct Rows {
+    std::vector<int> s, cls, perm;
+  } rows[HOST_THREADS];
+  pptr.assign(nt + 1, 0);
+  parallel_ranges(nt, 64, [&](int k, int64_t t0, int64_t t1) {
+    std::vector<int> cnt(nt, 0), touched;
+    std::vector<std::array<int, 2>> row;  // (s, class)
+    Rows& out = rows[k];
+    for (int t = (int)t0; t < (int)t1; ++t) {
+      touched.clear();
+      row.clear();
+      for (int a = 0; a < 3; ++a) {
+        const int v = hs.tri[3 * t + a];
+        for (int q = iptr[v]; q < iptr[v + 1]; ++q) {
+          const int u = inc[q] / 3;
+          if (cnt[u] == 0) touched.push_back(u);
+          cnt[u]++;
         }
       }
-      pt.push_back(t);
-      ps.push_back(u);
-      cls.push_back(c);
-      for (int k = 0; k < 6; ++k) perm.push_back(p[k]);
+      for (int u : touched) {
+        const int c = cnt[u];
+        row.push_back({u, c == 3 ? PAIR_IDENTICAL : (c == 2 ? PAIR_EDGE : PAIR_VERTEX)});
+      }
+      for (int q = nptr[t]; q < nptr[t + 1]; ++q) row.push_back({near[q], PAIR_NEAR});
+      std::sort(row.begin(), row.end());
+      for (auto& e : row) {
+        int u = e[0], c = e[1];
+        int p[6] = {0, 1, 2, 0, 1, 2};
+        const int* T = &hs.tri[3 * t];
+        const int* S = &hs.tri[3 * u];
+        if (c == PAIR_EDGE) {
+          // shared vertices in the test triangle's order go to reference vertices 0 and 1
+          int sh[2], ns = 0;
+          for (int a = 0; a < 3; ++a)
+            for (int b = 0; b < 3; ++b)
+              if (T[a] == S[b]) sh[ns++] = a;
+          int sb[2];
+          for (int k = 0; k < 2; ++k)
+            for (int b = 0; b < 3; ++b)
+              if (S[b] == T[sh[k]]) sb[k] = b;
+          p[0] = sh[0]; p[1] = sh[1]; p[2] = 3 - sh[0] - sh[1];
+          p[3] = sb[0]; p[4] = sb[1]; p[5] = 3 - sb[0] - sb[1];
+        } else if (c == PAIR_VERTEX) {
+          int ia = 0, ib = 0;
+          for (int a = 0; a < 3; ++a)
+            for (int b = 0; b < 3; ++b)
+              if (T[a] == S[b]) { ia = a; ib = b; }
+          for (int k = 0; k < 3; ++k) {
+            p[k] = (ia + k) % 3;
+            p[3 + k] = (ib + k) % 3;
+          }
+        }
+        out.s.push_back(u);
+        out.cls.push_back(c);
+        out.perm.insert(out.perm.end(), p, p + 6);
+      }
+      pptr[t + 1] = (int)row.size();
+      for (int u : touched) cnt[u] = 0;
     }
-    for (int u : touched) cnt[u] = 0;
-  }
+  });
+  for (int t = 0; t < nt; ++t) pptr[t + 1] += pptr[t];
+  const int np = pptr[nt];
+  pt.resize(np);
+  ps.resize(np);
+  cls.resize(np);
+  perm.resize(6 * (size_t)np);
+  parallel_ranges(nt, 64, [&](int k, int64_t t0, int64_t t1) {
+    const int p0 = pptr[t0];
+    std::copy(rows[k].s.begin(), rows[k].s.end(), ps.begin() + p0);
+    std::copy(rows[k].cls.begin(), rows[k].cls.end(), cls.begin() + p0);
+    std::copy(rows[k].perm.begin(), rows[k].perm.end(), perm.begin() + 6 * (size_t)p0);
+    for (int64_t t = t0; t < t1; ++t) std::fill(pt.begin() + pptr[t], pt.begin() + pptr[t + 1], (int)t);
+  });
 }
+
 
 int build_surface(Mesh* m, Surface* s, const std::vector<int>& gtri, const std::vector<double>& xyz_h) {
   const int nt = (int)gtri.size() / 3;
@@ -266,21 +317,12 @@ int build_surface(Mesh* m, Surface* s, const std::vector<int>& gtri, const std::
   PB_TRY(s->tri.upload(hs.tri.data(), hs.tri.size(), m->stream));
   PB_TRY(s->vmap.upload(verts.data(), verts.size(), m->stream));
   // test-reduction incidence: per vertex (t*3 + a)
-  {
-    std::vector<int> keys, vals;
-    for (int t = 0; t < nt; ++t)
-      for (int a = 0; a < 3; ++a) {
-        keys.push_back(hs.tri[3 * t + a]);
-        vals.push_back(3 * t + a);
-      }
-    std::vector<int> ptr, out;
-    bucket(keys, vals, s->nv, ptr, out);
-    PB_TRY(s->inc_ptr.upload(ptr.data(), ptr.size(), m->stream));
-    PB_TRY(s->inc_idx.upload(out.data(), out.size(), m->stream));
-  }
+  bucket(hs.tri.data(), 3 * (int64_t)nt, s->nv, [](int64_t e) { return (int)e; }, hs.iptr, hs.inc);
+  PB_TRY(s->inc_ptr.upload(hs.iptr.data(), hs.iptr.size(), m->stream));
+  PB_TRY(s->inc_idx.upload(hs.inc.data(), hs.inc.size(), m->stream));
   // special pairs and the correction pattern
-  std::vector<int> pt, ps, cls, perm;
-  classify_pairs(hs, pt, ps, cls, perm);
+  std::vector<int> pptr, pt, ps, cls, perm;
+  classify_pairs(hs, pptr, pt, ps, cls, perm);
   s->npair = (int)pt.size();
   PB_TRY(s->pair_t.upload(pt.data(), pt.size(), m->stream));
   PB_TRY(s->pair_s.upload(ps.data(), ps.size(), m->stream));
@@ -288,54 +330,66 @@ int build_surface(Mesh* m, Surface* s, const std::vector<int>& gtri, const std::
   PB_TRY(s->pair_perm.upload(perm.data(), perm.size(), m->stream));
   {
     // entry e = 9 p + 3 a + b of pair p couples test vertex tri[pt[p]][a] and trial vertex
-    // tri[ps[p]][b]; rows by counting sort, then columns sorted within each row
-    const size_t ne = 9 * (size_t)s->npair;
-    std::vector<int> rows(ne), vals(ne), slot_of(ne), dk, dv;
-    for (size_t e = 0; e < ne; ++e) {
-      const int p = (int)(e / 9), a = (int)(e / 3) % 3, b = (int)(e % 3);
-      rows[e] = hs.tri[3 * pt[p] + a];
-      vals[e] = (int)e;
-      if (rows[e] == hs.tri[3 * ps[p] + b]) {
-        dk.push_back(rows[e]);
-        dv.push_back((int)e);
+    // tri[ps[p]][b]: row i's entries are those of its triangles' pairs, in ascending order
+    auto entries = [&](int i, auto f) {  // f(entry, trial vertex)
+      for (int q = hs.iptr[i]; q < hs.iptr[i + 1]; ++q) {
+        const int t = hs.inc[q] / 3, a = hs.inc[q] % 3;
+        for (int p = pptr[t]; p < pptr[t + 1]; ++p)
+          for (int b = 0; b < 3; ++b) f(9 * p + 3 * a + b, hs.tri[3 * (size_t)ps[p] + b]);
       }
-    }
-    std::vector<int> colv(ne);
-    for (size_t e = 0; e < ne; ++e) colv[e] = hs.tri[3 * ps[e / 9] + e % 3];
-    std::vector<int> rptr, rent;
-    bucket(rows, vals, s->nv, rptr, rent);
+    };
+    // sizes, and the distinct columns (a marker per column), sorted
+    std::vector<int> dptr(s->nv + 1, 0), eptr(s->nv + 1, 0), cols[HOST_THREADS];
     s->c_ptr_h.assign(s->nv + 1, 0);
-    s->c_col_h.clear();
-    // per row: the distinct columns in first-seen order (a marker per column), sorted, then every
-    // entry's slot is its column's rank in the row
-    std::vector<int> mark(s->nv, -1), distinct;
+    parallel_ranges(s->nv, 32, [&](int k, int64_t i0, int64_t i1) {
+      std::vector<int> mark(s->nv, -1);
+      for (int i = (int)i0; i < (int)i1; ++i) {
+        const size_t w0 = cols[k].size();
+        entries(i, [&](int, int c) {
+          eptr[i + 1]++;
+          if (c == i) dptr[i + 1]++;
+          if (mark[c] != i) {
+            mark[c] = i;
+            cols[k].push_back(c);
+          }
+        });
+        std::sort(cols[k].begin() + w0, cols[k].end());
+        s->c_ptr_h[i + 1] = (int)(cols[k].size() - w0);
+      }
+    });
     for (int i = 0; i < s->nv; ++i) {
-      distinct.clear();
-      for (int q = rptr[i]; q < rptr[i + 1]; ++q) {
-        const int c = colv[rent[q]];
-        if (mark[c] < 0) {
-          mark[c] = 0;
-          distinct.push_back(c);
-        }
-      }
-      std::sort(distinct.begin(), distinct.end());
-      const int base = (int)s->c_col_h.size();
-      for (size_t r = 0; r < distinct.size(); ++r) {
-        mark[distinct[r]] = base + (int)r;
-        s->c_col_h.push_back(distinct[r]);
-      }
-      for (int q = rptr[i]; q < rptr[i + 1]; ++q) slot_of[rent[q]] = mark[colv[rent[q]]];
-      for (int c : distinct) mark[c] = -1;
-      s->c_ptr_h[i + 1] = (int)s->c_col_h.size();
+      s->c_ptr_h[i + 1] += s->c_ptr_h[i];
+      dptr[i + 1] += dptr[i];
+      eptr[i + 1] += eptr[i];
     }
-    s->cnnz = (int)s->c_col_h.size();
-    std::vector<int> ptr, out;
-    bucket(slot_of, vals, s->cnnz, ptr, out);
-    PB_TRY(s->cg_ptr.upload(ptr.data(), ptr.size(), m->stream));
-    PB_TRY(s->cg_idx.upload(out.data(), out.size(), m->stream));
-    bucket(dk, dv, s->nv, ptr, out);
-    PB_TRY(s->dg_ptr.upload(ptr.data(), ptr.size(), m->stream));
-    PB_TRY(s->dg_idx.upload(out.data(), out.size(), m->stream));
+    s->cnnz = s->c_ptr_h[s->nv];
+    s->c_col_h.resize(s->cnnz);
+    std::vector<int> cgp(s->cnnz + 1), cgi(eptr[s->nv]), dgi(dptr[s->nv]);
+    cgp[s->cnnz] = eptr[s->nv];
+    parallel_ranges(s->nv, 32, [&](int k, int64_t i0, int64_t i1) {
+      std::copy(cols[k].begin(), cols[k].end(), s->c_col_h.begin() + s->c_ptr_h[i0]);
+      std::vector<int> rank(s->nv), pos;
+      for (int i = (int)i0; i < (int)i1; ++i) {
+        const int c0 = s->c_ptr_h[i], n = s->c_ptr_h[i + 1] - c0;
+        pos.assign(n + 1, 0);
+        for (int r = 0; r < n; ++r) rank[s->c_col_h[c0 + r]] = r;
+        entries(i, [&](int, int c) { pos[rank[c] + 1]++; });
+        pos[0] = eptr[i];
+        for (int r = 0; r < n; ++r) {
+          cgp[c0 + r] = pos[r];
+          pos[r + 1] += pos[r];
+        }
+        int d = dptr[i];
+        entries(i, [&](int e, int c) {
+          cgi[pos[rank[c]]++] = e;
+          if (c == i) dgi[d++] = e;
+        });
+      }
+    });
+    PB_TRY(s->cg_ptr.upload(cgp.data(), cgp.size(), m->stream));
+    PB_TRY(s->cg_idx.upload(cgi.data(), cgi.size(), m->stream));
+    PB_TRY(s->dg_ptr.upload(dptr.data(), dptr.size(), m->stream));
+    PB_TRY(s->dg_idx.upload(dgi.data(), dgi.size(), m->stream));
     PB_TRY(s->c_ptr.upload(s->c_ptr_h.data(), s->c_ptr_h.size(), m->stream));
     PB_TRY(s->c_col.upload(s->c_col_h.data(), s->c_col_h.size(), m->stream));
   }
@@ -358,7 +412,7 @@ int build_surface(Mesh* m, Surface* s, const std::vector<int>& gtri, const std::
   return PBFB_OK;
 }
 
-int64_t key2(int r, int c) { return ((int64_t)r << 32) | (uint32_t)c; }
+uint64_t key2(int r, int c) { return ((uint64_t)(uint32_t)r << 32) | (uint32_t)c; }
 
 }  // namespace
 
@@ -421,51 +475,77 @@ static int validate(const double* xyz, int nv, const int* tets, int64_t nt, cons
       return PBFB_ERR_INVALID;
     }
   // boundary faces of the tets: faces used once, with the opposite vertex for orientation.
-  // Faces are bucketed by their smallest vertex and sorted by the other two within a bucket.
-  std::vector<std::array<int, 3>> fv(4 * (size_t)nt);  // sorted vertex triple of face 4 t + k
-  std::vector<int> fkey(4 * (size_t)nt), fidx(4 * (size_t)nt);
-  for (int64_t t = 0; t < nt; ++t) {
-    const int* T = tets + 4 * t;
-    double e[3][3];
-    for (int k = 0; k < 3; ++k)
-      for (int d = 0; d < 3; ++d) e[k][d] = xyz[3 * T[k + 1] + d] - xyz[3 * T[0] + d];
-    double det = e[0][0] * (e[1][1] * e[2][2] - e[1][2] * e[2][1]) - e[0][1] * (e[1][0] * e[2][2] - e[1][2] * e[2][0]) +
-                 e[0][2] * (e[1][0] * e[2][1] - e[1][1] * e[2][0]);
-    double L2 = 0.0;
-    for (int k = 0; k < 3; ++k) L2 = std::max(L2, e[k][0] * e[k][0] + e[k][1] * e[k][1] + e[k][2] * e[k][2]);
-    if (!(std::fabs(det) > 1e-12 * L2 * std::sqrt(L2))) {
-      set_error("mesh_create: degenerate tetrahedron %lld", (long long)t);
-      return PBFB_ERR_INVALID;
+  // Face 4 t + k by its smallest vertex, then sorted by the other two (one number) within a bucket.
+  struct Face {
+    uint64_t key;
+    int id;
+    bool operator<(const Face& o) const { return key != o.key ? key < o.key : id < o.id; }
+  };
+  std::vector<int> fkey(4 * (size_t)nt);
+  std::vector<uint64_t> fother(4 * (size_t)nt);
+  int64_t degenerate[HOST_THREADS];
+  std::fill(degenerate, degenerate + HOST_THREADS, nt);
+  parallel_ranges(nt, 4096, [&](int th, int64_t t0, int64_t t1) {
+    for (int64_t t = t0; t < t1; ++t) {
+      const int* T = tets + 4 * t;
+      double e[3][3];
+      for (int k = 0; k < 3; ++k)
+        for (int d = 0; d < 3; ++d) e[k][d] = xyz[3 * T[k + 1] + d] - xyz[3 * T[0] + d];
+      double det = e[0][0] * (e[1][1] * e[2][2] - e[1][2] * e[2][1]) -
+                   e[0][1] * (e[1][0] * e[2][2] - e[1][2] * e[2][0]) +
+                   e[0][2] * (e[1][0] * e[2][1] - e[1][1] * e[2][0]);
+      double L2 = 0.0;
+      for (int k = 0; k < 3; ++k) L2 = std::max(L2, e[k][0] * e[k][0] + e[k][1] * e[k][1] + e[k][2] * e[k][2]);
+      if (!(std::fabs(det) > 1e-12 * L2 * std::sqrt(L2))) {
+        degenerate[th] = t;
+        return;
+      }
+      for (int k = 0; k < 4; ++k) {
+        std::array<int, 3> f;
+        int q = 0;
+        for (int a = 0; a < 4; ++a)
+          if (a != k) f[q++] = T[a];
+        std::sort(f.begin(), f.end());
+        fkey[4 * t + k] = f[0];
+        fother[4 * t + k] = key2(f[1], f[2]);
+      }
     }
-    for (int k = 0; k < 4; ++k) {
-      std::array<int, 3> f;
-      int q = 0;
-      for (int a = 0; a < 4; ++a)
-        if (a != k) f[q++] = T[a];
-      std::sort(f.begin(), f.end());
-      fv[4 * t + k] = f;
-      fkey[4 * t + k] = f[0];
-      fidx[4 * t + k] = (int)(4 * t + k);
-    }
+  });
+  const int64_t bad = *std::min_element(degenerate, degenerate + HOST_THREADS);
+  if (bad < nt) {
+    set_error("mesh_create: degenerate tetrahedron %lld", (long long)bad);
+    return PBFB_ERR_INVALID;
   }
   std::vector<int> fptr, ford;
-  bucket(fkey, fidx, nv, fptr, ford);
-  auto face_less = [&](int x, int y) { return fv[x] < fv[y]; };
-  for (int v = 0; v < nv; ++v) std::sort(ford.begin() + fptr[v], ford.begin() + fptr[v + 1], face_less);
+  bucket(fkey.data(), 4 * nt, nv, [](int64_t e) { return (int)e; }, fptr, ford);
+  std::vector<Face> face(ford.size());
   // per sorted face position: multiplicity of its triple (1 boundary, 2 interior)
-  std::vector<int> fcount(ford.size(), 0);
+  std::vector<char> fcount(ford.size(), 0);
+  size_t nbs[HOST_THREADS] = {}, nifs[HOST_THREADS] = {};
+  bool more[HOST_THREADS] = {};
+  parallel_ranges(nv, 512, [&](int th, int64_t v0, int64_t v1) {
+    for (size_t q = fptr[v0]; q < (size_t)fptr[v1]; ++q) face[q] = {fother[ford[q]], ford[q]};
+    for (int64_t v = v0; v < v1; ++v) {
+      std::sort(face.begin() + fptr[v], face.begin() + fptr[v + 1]);
+      for (size_t a = fptr[v]; a < (size_t)fptr[v + 1];) {
+        size_t b = a + 1;
+        while (b < (size_t)fptr[v + 1] && face[b].key == face[a].key) ++b;
+        if (b - a > 2) more[th] = true;
+        if (b - a == 1) nbs[th]++;
+        if (b - a == 2 && region && region[face[a].id / 4] != region[face[a + 1].id / 4]) nifs[th]++;
+        for (size_t c = a; c < b; ++c) fcount[c] = (char)std::min<size_t>(b - a, 3);
+        a = b;
+      }
+    }
+  });
   size_t nb = 0, nif = 0;
-  for (size_t a = 0; a < ford.size();) {
-    size_t b = a + 1;
-    while (b < ford.size() && fv[ford[b]] == fv[ford[a]]) ++b;
-    if (b - a > 2) {
+  for (int th = 0; th < HOST_THREADS; ++th) {
+    if (more[th]) {
       set_error("mesh_create: a face is shared by more than two tets");
       return PBFB_ERR_INVALID;
     }
-    if (b - a == 1) nb++;
-    if (b - a == 2 && region && region[ford[a] / 4] != region[ford[a + 1] / 4]) nif++;
-    for (size_t c = a; c < b; ++c) fcount[c] = (int)(b - a);
-    a = b;
+    nb += nbs[th];
+    nif += nifs[th];
   }
   if (!region && nb != (size_t)ngm + (size_t)ngs) {
     set_error("mesh_create: %zu boundary faces but %d + %d surface triangles", nb, ngm, ngs);
@@ -476,18 +556,27 @@ static int validate(const double* xyz, int nv, const int* tets, int64_t nt, cons
               "triangles", nb, nif, ngs, ngm);
     return PBFB_ERR_INVALID;
   }
-  // position in ford of the boundary face with this sorted triple, or -1
+  // position of the face with this sorted triple, or -1
   auto find_face = [&](const std::array<int, 3>& f) -> long long {
-    auto b = ford.begin() + fptr[f[0]], e = ford.begin() + fptr[f[0] + 1];
-    auto it = std::lower_bound(b, e, f, [&](int x, const std::array<int, 3>& y) { return fv[x] < y; });
-    if (it == e || fv[*it] != f) return -1;
-    return (long long)(it - ford.begin());
+    auto b = face.begin() + fptr[f[0]], e = face.begin() + fptr[f[0] + 1];
+    auto it = std::lower_bound(b, e, Face{key2(f[1], f[2]), -1});
+    if (it == e || it->key != key2(f[1], f[2])) return -1;
+    return (long long)(it - face.begin());
   };
   std::vector<char> onm(nv, 0), ons(nv, 0);
   for (int surf = 0; surf < 2; ++surf) {
     const int* tri = surf == 0 ? gm : gs;
     int ntri = surf == 0 ? ngm : ngs;
-    std::map<std::pair<int, int>, int> dedges;
+    // directed edges (vertex pairs) in an open table of at most a quarter's load; 0 is no pair of distinct ids + 1
+    size_t slots = 64;
+    while (slots < 12 * (size_t)ntri) slots *= 2;
+    std::vector<uint64_t> edges(slots, 0);
+    auto edge = [&](int a, int b) -> uint64_t& {  // the pair's entry or the free one for it
+      const uint64_t key = key2(a + 1, b + 1);
+      size_t q = (key * 0x9E3779B97F4A7C15ull) >> 20 & (slots - 1);
+      while (edges[q] != 0 && edges[q] != key) q = (q + 1) & (slots - 1);
+      return edges[q];
+    };
     for (int t = 0; t < ntri; ++t) {
       const int* F = tri + 3 * t;
       if (F[0] == F[1] || F[1] == F[2] || F[0] == F[2]) {
@@ -499,7 +588,7 @@ static int validate(const double* xyz, int nv, const int* tets, int64_t nt, cons
       const long long pos = find_face(f);
       const bool interface = region && surf == 0;  // Gamma_m between the regions
       if (interface) {
-        if (pos < 0 || fcount[pos] != 2 || region[ford[pos] / 4] == region[ford[pos + 1] / 4]) {
+        if (pos < 0 || fcount[pos] != 2 || region[face[pos].id / 4] == region[face[pos + 1].id / 4]) {
           set_error("mesh_create: Gamma_m triangle %d is not a face between Omega_m and Omega_i tets", t);
           return PBFB_ERR_INVALID;
         }
@@ -511,7 +600,7 @@ static int validate(const double* xyz, int nv, const int* tets, int64_t nt, cons
       fcount[pos] = 3;  // claimed
       // orientation: the opposite tet vertex lies on the positive side for Gamma_m (of the
       // Omega_i tet for an interface), on the negative side for Gamma_s
-      const int fid = interface && region[ford[pos] / 4] != 1 ? ford[pos + 1] : ford[pos];
+      const int fid = face[interface && region[face[pos].id / 4] != 1 ? pos + 1 : pos].id;
       int o = tets[fid];
       double a[3], b[3], c[3];
       for (int d = 0; d < 3; ++d) {
@@ -526,19 +615,21 @@ static int validate(const double* xyz, int nv, const int* tets, int64_t nt, cons
         return PBFB_ERR_INVALID;
       }
       for (int k = 0; k < 3; ++k) {
-        auto key = std::make_pair(F[k], F[(k + 1) % 3]);
-        if (++dedges[key] > 1) {
+        uint64_t& e = edge(F[k], F[(k + 1) % 3]);
+        if (e != 0) {
           set_error("mesh_create: surface is not consistently oriented / manifold");
           return PBFB_ERR_INVALID;
         }
+        e = key2(F[k] + 1, F[(k + 1) % 3] + 1);
         (surf == 0 ? onm : ons)[F[k]] = 1;
       }
     }
-    for (auto& kv : dedges)
-      if (!dedges.count(std::make_pair(kv.first.second, kv.first.first))) {
-        set_error("mesh_create: %s is not closed", surf == 0 ? "Gamma_m" : "Gamma_s");
-        return PBFB_ERR_INVALID;
-      }
+    for (int t = 0; t < ntri; ++t)
+      for (int k = 0; k < 3; ++k)
+        if (edge(tri[3 * t + (k + 1) % 3], tri[3 * t + k]) == 0) {
+          set_error("mesh_create: %s is not closed", surf == 0 ? "Gamma_m" : "Gamma_s");
+          return PBFB_ERR_INVALID;
+        }
   }
   for (int v = 0; v < nv; ++v)
     if (onm[v] && ons[v]) {
@@ -742,133 +833,164 @@ int mesh_create(const double* xyz, int nv, const int* tets, int64_t nt, const in
   sm.col0 = nv;
   ss.col0 = nv + sm.nv;
   m->n = nv + sm.nv + ss.nv;
-  // ---- sparse-part pattern of the coupled operator
-  std::vector<int64_t> keys;
-  keys.reserve(16 * (size_t)nt + 4 * (size_t)(sm.cnnz + ss.cnnz));
-  for (int r = 0; r < 2; ++r) {
-    const int* tt = r == 0 ? ti : tm_h.data();
-    const int64_t cnt = r == 0 ? nti : ntm;
-    for (int64_t t = 0; t < cnt; ++t)
-      for (int a = 0; a < 4; ++a)
-        for (int b = 0; b < 4; ++b) keys.push_back(key2(tt[4 * t + a], tt[4 * t + b]));
-  }
-  // mass pattern (vertices sharing a triangle) for the FEM coupling entries
-  auto mass_pairs = [](const Surface& s, std::vector<std::pair<int, int>>& mp) {
-    for (int t = 0; t < s.nt; ++t)
-      for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) mp.push_back({s.tri_h[3 * t + a], s.tri_h[3 * t + b]});
-    std::sort(mp.begin(), mp.end());
-    mp.erase(std::unique(mp.begin(), mp.end()), mp.end());
-  };
-  // (an interior Gamma_m couples nothing: its lam_m rows are the identity)
-  std::vector<std::pair<int, int>> mpm, mps;
-  if (!m->full) mass_pairs(sm, mpm);
-  mass_pairs(ss, mps);
-  for (auto& e : mpm) keys.push_back(key2(sm.vmap_h[e.first], sm.col0 + e.second));
-  for (auto& e : mps) keys.push_back(key2(ss.vmap_h[e.first], ss.col0 + e.second));
-  for (const Surface* s : {&sm, &ss}) {
-    if (m->full && s == &sm) {
-      for (int i = 0; i < s->nv; ++i) keys.push_back(key2(s->col0 + i, s->col0 + i));
-      continue;
+  // ---- sparse-part pattern of the coupled operator, row by row: a FEM row has the vertices of its tets, then the
+  // surface unknowns of the vertices it shares a triangle with (mass coupling; an interior Gamma_m couples nothing:
+  // its lam_m rows are the identity)
+  const int* tt[2] = {ti, tm_h.data()};
+  const int64_t tn[2] = {nti, ntm};
+  std::vector<int> vptr[2], vtet[2];  // per vertex and region: its tets' entries 4 t + a, ascending
+  for (int r = 0; r < 2; ++r) bucket(tt[r], 4 * tn[r], nv, [](int64_t e) { return (int)e; }, vptr[r], vtet[r]);
+  // per surface: the mass pattern's rows (vertices sharing a triangle), and the surface's vertex at a mesh vertex
+  std::vector<int> mptr[2], mcol[2];
+  std::vector<int> at[2] = {std::vector<int>(nv, -1), std::vector<int>(nv, -1)};
+  for (int si = 0; si < 2; ++si) {
+    const Surface& s = si == 0 ? sm : ss;
+    mptr[si].assign(s.nv + 1, 0);
+    if (si == 0 && m->full) continue;
+    std::vector<int> ip, ie;
+    bucket(s.tri_h.data(), 3 * (int64_t)s.nt, s.nv, [](int64_t e) { return (int)e; }, ip, ie);
+    std::vector<int> row;
+    for (int i = 0; i < s.nv; ++i) {
+      at[si][s.vmap_h[i]] = i;
+      row.clear();
+      for (int q = ip[i]; q < ip[i + 1]; ++q)
+        for (int b = 0; b < 3; ++b) row.push_back(s.tri_h[3 * (size_t)(ie[q] / 3) + b]);
+      std::sort(row.begin(), row.end());
+      row.erase(std::unique(row.begin(), row.end()), row.end());
+      mcol[si].insert(mcol[si].end(), row.begin(), row.end());
+      mptr[si][i + 1] = (int)mcol[si].size();
     }
-    for (int i = 0; i < s->nv; ++i)
-      for (int k = s->c_ptr_h[i]; k < s->c_ptr_h[i + 1]; ++k) {
-        int j = s->c_col_h[k];
-        keys.push_back(key2(s->col0 + i, s->vmap_h[j]));
-        keys.push_back(key2(s->col0 + i, s->col0 + j));
-      }
   }
-  {
-    // rows by counting sort, then sorted unique columns within each row
-    std::vector<int> rk(keys.size()), ck(keys.size());
-    for (size_t k = 0; k < keys.size(); ++k) {
-      rk[k] = (int)(keys[k] >> 32);
-      ck[k] = (int)(keys[k] & 0xffffffff);
-    }
-    std::vector<int>().swap(m->s_col_h);
-    std::vector<int64_t>().swap(keys);
-    std::vector<int> rptr, cols;
-    bucket(rk, ck, m->n, rptr, cols);
-    m->s_ptr_h.assign(m->n + 1, 0);
-    size_t w = 0;
-    std::vector<char> seen(m->n, 0);
-    for (int r = 0; r < m->n; ++r) {
-      // distinct columns of the row (a marker per column), then sorted in place
-      const size_t w0 = w;
-      for (int q = rptr[r]; q < rptr[r + 1]; ++q) {
-        const int c = cols[q];
-        if (!seen[c]) {
-          seen[c] = 1;
-          cols[w++] = c;
+  // row sizes; the FEM columns, distinct (a marker per column) and sorted
+  std::vector<int> cols[HOST_THREADS];
+  m->s_ptr_h.assign(m->n + 1, 0);
+  parallel_ranges(nv, 256, [&](int k, int64_t v0, int64_t v1) {
+    std::vector<int> mark(nv, -1);
+    std::vector<int>& out = cols[k];
+    for (int v = (int)v0; v < (int)v1; ++v) {
+      const size_t w0 = out.size();
+      for (int r = 0; r < 2; ++r)
+        for (int q = vptr[r][v]; q < vptr[r][v + 1]; ++q) {
+          const int* T = tt[r] + 4 * (int64_t)(vtet[r][q] / 4);
+          for (int b = 0; b < 4; ++b)
+            if (mark[T[b]] != v) {
+              mark[T[b]] = v;
+              out.push_back(T[b]);
+            }
         }
-      }
-      std::sort(cols.begin() + w0, cols.begin() + w);
-      for (size_t q = w0; q < w; ++q) seen[cols[q]] = 0;
-      m->s_ptr_h[r + 1] = (int)w;
+      std::sort(out.begin() + w0, out.end());
+      int len = (int)(out.size() - w0);
+      for (int si = 0; si < 2; ++si)
+        if (const int i = at[si][v]; i >= 0) len += mptr[si][i + 1] - mptr[si][i];
+      m->s_ptr_h[v + 1] = len;
     }
-    cols.resize(w);
-    m->s_col_h.swap(cols);
-    m->snnz = (int)w;
+  });
+  for (int si = 0; si < 2; ++si) {
+    const Surface& s = si == 0 ? sm : ss;
+    for (int i = 0; i < s.nv; ++i)
+      m->s_ptr_h[s.col0 + i + 1] = si == 0 && m->full ? 1 : 2 * (s.c_ptr_h[i + 1] - s.c_ptr_h[i]);
   }
+  for (int i = 0; i < m->n; ++i) m->s_ptr_h[i + 1] += m->s_ptr_h[i];
+  m->snnz = m->s_ptr_h[m->n];
   m->fem_nnz = m->s_ptr_h[nv];
+  m->s_col_h.resize(m->snnz);
   auto slot = [&](int r, int c) -> int {
     auto b = m->s_col_h.begin() + m->s_ptr_h[r], e = m->s_col_h.begin() + m->s_ptr_h[r + 1];
     return (int)(std::lower_bound(b, e, c) - m->s_col_h.begin());
   };
-  std::vector<int> kind(m->snnz, -1), ref(m->snnz, 0);
-  DBuf<int> jm_ptr, jm_idx;  // Omega_m stiffness gather (set-up only)
-  {
-    // per slot: tet-local entries (k * cnt + t) of the Omega_i tets, and of the Omega_m tets
-    std::vector<int> ptr, outv;
-    for (int r = 0; r < (ntm ? 2 : 1); ++r) {
-      const int* tt = r == 0 ? ti : tm_h.data();
-      const int64_t cnt = r == 0 ? nti : ntm;
-      std::vector<int> jk, jv;
-      jk.reserve(16 * (size_t)cnt);
-      jv.reserve(16 * (size_t)cnt);
-      for (int64_t t = 0; t < cnt; ++t)
-        for (int a = 0; a < 4; ++a)
-          for (int b = 0; b < 4; ++b) {
-            int sl = slot(tt[4 * t + a], tt[4 * t + b]);
-            kind[sl] = 0;
-            jk.push_back(sl);
-            jv.push_back((int)(sym10(a, b) * cnt + t));
-          }
-      bucket(jk, jv, m->snnz, ptr, outv);
-      if ((st = (r == 0 ? m->jg_ptr : jm_ptr).upload(ptr.data(), ptr.size(), stream))) return fail(st);
-      if ((st = (r == 0 ? m->jg_idx : jm_idx).upload(outv.data(), outv.size(), stream))) return fail(st);
-    }
-    std::vector<int> nk, nvv;
-    for (int64_t t = 0; t < nti; ++t)
-      for (int a = 0; a < 4; ++a) {
-        nk.push_back(ti[4 * t + a]);
-        nvv.push_back((int)(a * nti + t));
-      }
-    bucket(nk, nvv, nv, ptr, outv);
-    if ((st = m->ng_ptr.upload(ptr.data(), ptr.size(), stream))) return fail(st);
-    if ((st = m->ng_idx.upload(outv.data(), outv.size(), stream))) return fail(st);
-  }
   auto cslot = [](const Surface& s, int i, int j) -> int {
     auto b = s.c_col_h.begin() + s.c_ptr_h[i], e = s.c_col_h.begin() + s.c_ptr_h[i + 1];
     return (int)(std::lower_bound(b, e, j) - s.c_col_h.begin());
   };
-  for (auto& e : mpm) {
-    int sl = slot(sm.vmap_h[e.first], sm.col0 + e.second);
-    kind[sl] = 1;
-    ref[sl] = cslot(sm, e.first, e.second);
+  std::vector<int> kind(m->snnz, 0), ref(m->snnz, 0);
+  DBuf<int> jm_ptr, jm_idx;  // Omega_m stiffness gather (set-up only)
+  {
+    // per slot: tet-local entries (k * cnt + t) of the Omega_i tets, and of the Omega_m tets; a row's lie together
+    // (four for every entry of vtet), the slots past the FEM columns have none
+    std::vector<int> jp[2], ji[2];
+    for (int r = 0; r < (ntm ? 2 : 1); ++r) {
+      jp[r].assign(m->snnz + 1, (int)(16 * tn[r]));
+      ji[r].resize(16 * tn[r]);
+    }
+    parallel_ranges(nv, 256, [&](int k, int64_t v0, int64_t v1) {
+      std::vector<int> rank(nv), pos;
+      const int* src = cols[k].data();
+      for (int v = (int)v0; v < (int)v1; ++v) {
+        int* row = m->s_col_h.data() + m->s_ptr_h[v];
+        const int s0 = m->s_ptr_h[v], len = m->s_ptr_h[v + 1] - s0;
+        int nf = len, mass = 0;
+        for (int si = 0; si < 2; ++si)
+          if (const int i = at[si][v]; i >= 0) mass += mptr[si][i + 1] - mptr[si][i];
+        nf -= mass;
+        for (int q = 0; q < nf; ++q) {
+          row[q] = src[q];
+          rank[src[q]] = q;
+        }
+        src += nf;
+        for (int si = 0, q = nf; si < 2; ++si)
+          if (const int i = at[si][v]; i >= 0) {
+            const Surface& s = si == 0 ? sm : ss;
+            for (int e = mptr[si][i]; e < mptr[si][i + 1]; ++e, ++q) {
+              row[q] = s.col0 + mcol[si][e];
+              kind[s0 + q] = 1 + si;
+              ref[s0 + q] = cslot(s, i, mcol[si][e]);
+            }
+          }
+        for (int r = 0; r < (ntm ? 2 : 1); ++r) {
+          pos.assign(nf + 1, 0);
+          auto entries = [&](auto f) {  // f(column's rank, tet-local entry)
+            for (int q = vptr[r][v]; q < vptr[r][v + 1]; ++q) {
+              const int64_t t = vtet[r][q] / 4;
+              const int a = vtet[r][q] % 4;
+              for (int b = 0; b < 4; ++b) f(rank[tt[r][4 * t + b]], (int)(sym10(a, b) * tn[r] + t));
+            }
+          };
+          entries([&](int c, int) { pos[c + 1]++; });
+          pos[0] = 4 * vptr[r][v];
+          for (int q = 0; q < nf; ++q) {
+            jp[r][s0 + q] = pos[q];
+            pos[q + 1] += pos[q];
+          }
+          for (int q = nf; q < len; ++q) jp[r][s0 + q] = pos[nf];
+          entries([&](int c, int e) { ji[r][pos[c]++] = e; });
+        }
+      }
+    });
+    for (int r = 0; r < (ntm ? 2 : 1); ++r) {
+      if ((st = (r == 0 ? m->jg_ptr : jm_ptr).upload(jp[r].data(), jp[r].size(), stream))) return fail(st);
+      if ((st = (r == 0 ? m->jg_idx : jm_idx).upload(ji[r].data(), ji[r].size(), stream))) return fail(st);
+    }
+    for (int& e : vtet[0]) e = (int)((e % 4) * nti + e / 4);
+    if ((st = m->ng_ptr.upload(vptr[0].data(), vptr[0].size(), stream))) return fail(st);
+    if ((st = m->ng_idx.upload(vtet[0].data(), vtet[0].size(), stream))) return fail(st);
   }
-  for (auto& e : mps) {
-    int sl = slot(ss.vmap_h[e.first], ss.col0 + e.second);
-    kind[sl] = 2;
-    ref[sl] = cslot(ss, e.first, e.second);
+  for (int si = 0; si < 2; ++si) {
+    const Surface& s = si == 0 ? sm : ss;
+    for (int i = 0; i < s.nv; ++i) {
+      const int s0 = m->s_ptr_h[s.col0 + i], c0 = s.c_ptr_h[i], n = s.c_ptr_h[i + 1] - c0;
+      if (m->full && si == 0) {
+        m->s_col_h[s0] = s.col0 + i;
+        kind[s0] = 7;
+        continue;
+      }
+      for (int q = 0; q < n; ++q) {
+        const int j = s.c_col_h[c0 + q];
+        m->s_col_h[s0 + q] = s.vmap_h[j];
+        m->s_col_h[s0 + n + q] = s.col0 + j;
+        kind[s0 + q] = si == 0 ? 3 : 5;
+        kind[s0 + n + q] = si == 0 ? 4 : 6;
+        ref[s0 + q] = ref[s0 + n + q] = c0 + q;
+      }
+    }
   }
   {
     // Robin term of the block preconditioner: u-u slots of Gamma_s vertex pairs sharing a triangle
     std::vector<int> rs, rr;
-    for (auto& e : mps) {
-      rs.push_back(slot(ss.vmap_h[e.first], ss.vmap_h[e.second]));
-      rr.push_back(cslot(ss, e.first, e.second));
-    }
+    for (int i = 0; i < ss.nv; ++i)
+      for (int e = mptr[1][i]; e < mptr[1][i + 1]; ++e) {
+        rs.push_back(slot(ss.vmap_h[i], ss.vmap_h[mcol[1][e]]));
+        rr.push_back(cslot(ss, i, mcol[1][e]));
+      }
     m->nrobin = (int)rs.size();
     if ((st = m->robin_slot.upload(rs.data(), rs.size(), stream))) return fail(st);
     if ((st = m->robin_ref.upload(rr.data(), rr.size(), stream))) return fail(st);
@@ -885,28 +1007,6 @@ int mesh_create(const double* xyz, int nv, const int* tets, int64_t nt, const in
     }
     m->gs_radius = std::sqrt(area / (4.0 * M_PI));
   }
-  for (int si = 0; si < 2; ++si) {
-    const Surface& s = si == 0 ? sm : ss;
-    if (m->full && si == 0) {
-      for (int i = 0; i < s.nv; ++i) kind[slot(s.col0 + i, s.col0 + i)] = 7;
-      continue;
-    }
-    for (int i = 0; i < s.nv; ++i)
-      for (int k = s.c_ptr_h[i]; k < s.c_ptr_h[i + 1]; ++k) {
-        int j = s.c_col_h[k];
-        int a = slot(s.col0 + i, s.vmap_h[j]);
-        int b = slot(s.col0 + i, s.col0 + j);
-        kind[a] = si == 0 ? 3 : 5;
-        ref[a] = k;
-        kind[b] = si == 0 ? 4 : 6;
-        ref[b] = k;
-      }
-  }
-  for (int k = 0; k < m->snnz; ++k)
-    if (kind[k] < 0) {
-      set_error("internal: unassigned operator slot");
-      return fail(PBFB_ERR_STATE);
-    }
   if ((st = m->s_ptr.upload(m->s_ptr_h.data(), m->s_ptr_h.size(), stream))) return fail(st);
   if ((st = m->s_col.upload(m->s_col_h.data(), m->s_col_h.size(), stream))) return fail(st);
   if ((st = m->s_kind.upload(kind.data(), kind.size(), stream))) return fail(st);
