@@ -702,28 +702,49 @@ __global__ void k_split_sum(int nq, int nsplit, double* __restrict__ val) {
   val[j] = v;
 }
 
-// y[i] (+)= scale * sum over incident (tau, a) of sum_q psi_a(x_q) w_q val[0][6 tau + q]; 4 lanes per vertex
+// y[i] (+)= sum over incident (tau, a) of sum_q psi_a(x_q) w_q val[6 tau + q], plus the rows of `add` (the near
+// field's, which would cost a launch of its own, 2.7 us of a 70 us product of 500 triangles); 8 lanes per vertex
 __global__ void k_test_reduce(int nv, const int* __restrict__ ptr, const int* __restrict__ idx,
-                              const double* __restrict__ val, int nsplit, int nq, const double* __restrict__ qw,
-                              double scale, int accumulate, double* __restrict__ y) {
-  const int lane = threadIdx.x & 3;
-  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 2;
+                              const double* __restrict__ val, const double* __restrict__ qw, RowAdd add,
+                              int accumulate, double* __restrict__ y) {
+  const int lane = threadIdx.x & 7;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 3;
   const bool valid = i < nv;  // all lanes reach the shuffles
-  (void)nsplit;
-  (void)nq;
-  double acc = 0.0;
+  double acc = 0.0, cor = 0.0;
   const int b = valid ? ptr[i] : 0, e = valid ? ptr[i + 1] : 0;
-  for (int k = b * QS + lane; k < e * QS; k += 4) {
+  for (int k = b * QS + lane; k < e * QS; k += 8) {
     int ent = idx[k / QS], q = k % QS;
     int t = ent / 3, a = ent - 3 * t;
     int j = QS * t + q;
     acc += c_tri_b[q][a] * qw[j] * val[j];
   }
-  acc += __shfl_down_sync(0xffffffffu, acc, 2, 4);
-  acc += __shfl_down_sync(0xffffffffu, acc, 1, 4);
+  if (add.ptr && valid) {
+    const int k1 = add.ptr[i + 1];
+    for (int k0 = add.ptr[i] + lane; k0 < k1; k0 += 32) {  // four entries a lane in flight
+      double v[4], x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int k = k0 + 8 * u;
+        v[u] = x[u] = 0.0;
+        if (k < k1) {
+          const int c = add.col[k];
+          v[u] = add.val[k];
+          if (add.half) v[u] = fma(0.5, add.half[k], v[u]);
+          x[u] = add.x[add.map ? add.map[c] : c];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) cor = fma(v[u], x[u], cor);
+    }
+  }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+    acc += __shfl_down_sync(0xffffffffu, acc, o, 8);
+    cor += __shfl_down_sync(0xffffffffu, cor, o, 8);
+  }
   if (lane == 0 && valid) {
-    acc *= scale;
-    y[i] = accumulate ? y[i] + acc : acc;
+    acc = accumulate ? y[i] + acc : acc;
+    y[i] = add.ptr ? acc + cor : acc;
   }
 }
 
@@ -912,14 +933,13 @@ int ff_exp_table(Mesh* m) {
   return PBFB_OK;
 }
 
-int test_reduce(Mesh* m, Surface* s, double* val, int nsplit, double* y, bool accumulate) {
+int test_reduce(Mesh* m, Surface* s, double* val, int nsplit, double* y, bool accumulate, const RowAdd* add) {
   if (nsplit > 1) {
     k_split_sum<<<blocks_for(s->nq, 256), 256, 0, m->stream>>>(s->nq, nsplit, val);
     PB_LAUNCHED(m);
   }
-  k_test_reduce<<<blocks_for((int64_t)s->nv * 4, 128), 128, 0, m->stream>>>(s->nv, s->inc_ptr.p, s->inc_idx.p, val,
-                                                                            nsplit, s->nq, s->qw.p, 1.0,
-                                                                            accumulate ? 1 : 0, y);
+  k_test_reduce<<<blocks_for((int64_t)s->nv * 8, 128), 128, 0, m->stream>>>(
+      s->nv, s->inc_ptr.p, s->inc_idx.p, val, s->qw.p, add ? *add : RowAdd{}, accumulate ? 1 : 0, y);
   PB_LAUNCHED(m);
   return PBFB_OK;
 }
@@ -1005,17 +1025,17 @@ void launch_nbody_f32(Mesh* m, Surface* s, double kappa, int tpt, int packed, in
 // lam indexed by local surface vertex; x (the shell part of the full vector, or a local
 // surface vector when lam == x is a surface vector) indexed through vmap.
 int launch_bem_far(Mesh* m, Surface* s, const double* x, const double* lam, double cs, double cd, double kappa,
-                   int precision, double* y, bool accumulate) {
+                   int precision, double* y, bool accumulate, const RowAdd* add) {
   const int nq = s->nq;
   const bool yuk = kappa != 0.0;
   const int u_local = (x != nullptr && x == lam) ? 1 : 0;
   const double* uvec = (cd != 0.0) ? x : nullptr;
   const double* lvec = (cs != 0.0) ? lam : nullptr;
-  if (precision == PBFB_FLOAT2) return launch_bem_far_ff(m, s, x, lam, cs, cd, kappa, y, accumulate);
+  if (precision == PBFB_FLOAT2) return launch_bem_far_ff(m, s, x, lam, cs, cd, kappa, y, accumulate, add);
   if (precision == PBFB_FP64) {
     double* v;
     PB_TRY(launch_pairs(m, s, x, lam, cs * INV4PI, cd * INV4PI, kappa, true, &v));
-    return test_reduce(m, s, v, 1, y, accumulate);
+    return test_reduce(m, s, v, 1, y, accumulate, add);
   }
   k_sources<<<blocks_for(nq, 256), 256, 0, m->stream>>>(s->nt, s->tri.p, s->vmap.p, lvec, uvec, u_local, s->qw.p,
                                                         s->nrm.p, s->qpf.p, cs * INV4PI, cd * INV4PI, s->spos.p,
@@ -1074,11 +1094,11 @@ int launch_bem_far(Mesh* m, Surface* s, const double* x, const double* lam, doub
   const double pairs = tree_pairs >= 0.0 ? tree_pairs : (double)nq * (double)nq;
   timer_end(m, tm, ev, pairs);
   m->nbody_flops += (yuk ? 24.0 : 18.0) * pairs;
-  return test_reduce(m, s, vals, nsplit, y, accumulate);
+  return test_reduce(m, s, vals, nsplit, y, accumulate, add);
 }
 
 int launch_bem_far_ff(Mesh* m, Surface* s, const double* x, const double* lam, double cs, double cd,
-                      double kappa, double* y, bool accumulate) {
+                      double kappa, double* y, bool accumulate, const RowAdd* add) {
   const int nq = s->nq;
   const bool yuk = kappa != 0.0;
   const int u_local = (x != nullptr && x == lam) ? 1 : 0;
@@ -1088,7 +1108,7 @@ int launch_bem_far_ff(Mesh* m, Surface* s, const double* x, const double* lam, d
   if (m->tune_ff_kernel != 1) {
     double* v;
     PB_TRY(launch_pairs(m, s, x, lam, cs * INV4PI, cd * INV4PI, kappa, kappa > 0.0 && kappa < 1e-8, &v));
-    return test_reduce(m, s, v, 1, y, accumulate);
+    return test_reduce(m, s, v, 1, y, accumulate, add);
   }
   PB_TRY(ff_exp_table(m));
   if (s->ffsrc.n < 4 * (size_t)nq) PB_TRY(s->ffsrc.alloc(4 * (size_t)nq));
@@ -1117,7 +1137,7 @@ int launch_bem_far_ff(Mesh* m, Surface* s, const double* x, const double* lam, d
     k_nbody_ff<NT, false><<<grid, NT, 0, m->stream>>>(nq, s->fftgt.p, s->ffsrc.p, kh, kl, m->ff_tab.p, per, s->val.p);
   PB_LAUNCHED(m);
   timer_end(m, m->t_nbodyff, ev, (double)nq * (double)nq);
-  return test_reduce(m, s, s->val.p, nsplit, y, accumulate);
+  return test_reduce(m, s, s->val.p, nsplit, y, accumulate, add);
 }
 
 int launch_coulomb(Mesh* m) {
@@ -1258,8 +1278,8 @@ int bem_apply_noalloc(Mesh* m, int which, int op, const double* x, double* y) {
   nsplit = blocks_for(nq, per);
   launch_nbody_f32(m, s, kappa, tpt, packed, nsplit, per, spos, sdl, val);
   PB_LAUNCHED(m);
-  PB_TRY(test_reduce(m, s, val, nsplit, y, false));
-  PB_TRY(launch_csr_spmv(m, s->nv, s->c_ptr.p, s->c_col.p, op == 0 ? s->corrV.p : s->corrK.p, x, y, true));
+  const RowAdd near = near_rows(s, op, x);
+  PB_TRY(test_reduce(m, s, val, nsplit, y, false, &near));
   return PBFB_OK;
 }
 

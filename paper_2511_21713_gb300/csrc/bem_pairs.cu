@@ -479,29 +479,49 @@ __global__ void __launch_bounds__(32 * PW, 2)
   }
 }
 
-// out[i] = sum of point i's rows (pair_task), in a fixed order: 8 threads a point, their sums added in thread
-// order.
-__global__ void __launch_bounds__(256) k_pairs_sum(int nq, int per_group, int G, int K, int nsub,
-                                                    const double* PI, const double* PJ,
-                                                    double* __restrict__ out) {
-  __shared__ double sh[8][33];
+// out[i] = sum of point i's rows (pair_task), in a fixed order: SUM_Y threads a point, their sums added in thread
+// order.  A chain of L2 latencies where rows are many (500 triangles: up to 768): 12.6 us with 8
+// threads and one load at a time, 6.4 us with 16 and eight in flight.
+constexpr int SUM_Y = 16;
+__global__ void __launch_bounds__(32 * SUM_Y) k_pairs_sum(int nq, int per_group, int G, int K, int nsub,
+                                                          const double* PI, const double* PJ,
+                                                          double* __restrict__ out) {
+  __shared__ double sh[SUM_Y][33];
   const int i = blockIdx.x * 32 + threadIdx.x, ty = threadIdx.y;
   double v = 0.0;
+  // rows p G + c, p < np, lo <= c < hi, every SUM_Y-th of them; eight loads in flight
+  auto rows = [&](const double* P, int np, int lo, int hi) {
+    const int n = hi - lo, dp = SUM_Y / n, dc = SUM_Y - dp * n;
+    int p = ty / n, c = lo + ty - p * n;
+    while (p < np) {
+      double x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        x[u] = p < np ? P[((size_t)p * G + c) * nq + i] : 0.0;
+        p += dp;
+        c += dc;
+        if (c >= hi) {
+          c -= n;
+          ++p;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v += x[u];
+    }
+  };
   if (i < nq) {
     if (nsub == 1) {
-      for (int r = ty; r < K * (G + 1); r += 8) v += PI[(size_t)r * nq + i];
+      rows(PI, 1, 0, K * (G + 1));
     } else {
       const int gi = i / per_group;
-      for (int p = 0; p < K; ++p)
-        for (int c = gi + ty; c < G; c += 8) v += PI[(size_t)(p * G + c) * nq + i];
-      for (int p = 0; p < K * nsub; ++p)
-        for (int r = ty; r <= gi; r += 8) v += PJ[(size_t)(p * G + r) * nq + i];
+      rows(PI, K, gi, G);
+      rows(PJ, K * nsub, 0, gi + 1);
     }
   }
   sh[ty][threadIdx.x] = v;
   __syncthreads();
   if (ty == 0 && i < nq) {
-    for (int k = 1; k < 8; ++k) v += sh[k][threadIdx.x];
+    for (int k = 1; k < SUM_Y; ++k) v += sh[k][threadIdx.x];
     out[i] = v;
   }
 }
@@ -705,7 +725,7 @@ int launch_pairs(Mesh* m, Surface* s, const double* x, const double* lam, double
     PB_CUDA(cudaLaunchKernel(fn, dim3(nb), dim3(32 * PW), args, 0, m->stream));
   }
   PB_LAUNCHED(m);
-  k_pairs_sum<<<blocks_for(nq, 32), dim3(32, 8), 0, m->stream>>>(nq, S.tpg * PT * QS, S.G, S.K, S.nsub, PI, PJ, out);
+  k_pairs_sum<<<blocks_for(nq, 32), dim3(32, SUM_Y), 0, m->stream>>>(nq, S.tpg * PT * QS, S.G, S.K, S.nsub, PI, PJ, out);
   PB_LAUNCHED(m);
   timer_end(m, tm, ev, (double)nq * (double)nq);
   *val = out;

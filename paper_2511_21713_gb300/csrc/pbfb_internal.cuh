@@ -279,8 +279,7 @@ struct Mesh {
   double cell_lo[3] = {0, 0, 0}, cell_h = 1.0;
   int cell_dim[3] = {0, 0, 0};
   DBuf<double> rho;                 // nv: sum_k z_k v_i(x_k) (no 4 pi l_B)
-  DBuf<double> pp_val;              // Gamma_m correction pattern: M_m / 2 + corrK_m
-  DBuf<double> pp_work;             // post-process vectors: 6 * nm
+  DBuf<double> pp_work;             // the flux's vectors: 5 * nm
   ~Mesh() {
     if (pcg_graph) cudaGraphExecDestroy(pcg_graph);
   }
@@ -317,6 +316,21 @@ namespace pbfb {
 // ---- quadrature constants (device) and their host initialisation
 int init_quadrature();
 
+// Sparse rows added to a test reduction (ptr null: none): y_i += sum_k (val_k + half_k / 2) x[map[col_k]],
+// half and map optional.
+struct RowAdd {
+  const int* ptr = nullptr;
+  const int* col = nullptr;
+  const double* val = nullptr;
+  const double* half = nullptr;
+  const double* x = nullptr;
+  const int* map = nullptr;
+};
+// the near-field correction of a surface's V (op 0) or K (op 1)
+inline RowAdd near_rows(const Surface* s, int op, const double* x) {
+  return {s->c_ptr.p, s->c_col.p, op == 0 ? s->corrV.p : s->corrK.p, nullptr, x, nullptr};
+}
+
 // ---- fem_kernels.cu
 int launch_tet_volumes(Mesh* m, const int* tets, int64_t nt, double* vol);
 int launch_stiffness_local(Mesh* m, const int* tets, int64_t nt, const double* vol, double* loc10);
@@ -343,11 +357,13 @@ int launch_csr_spmv(Mesh* m, int nrows, const int* ptr, const int* col, const do
 // ---- bem_kernels.cu
 int launch_surface_geometry(Mesh* m, Surface* s);
 // test reduction of far-field partials (sums the source splits in place, then reduces per vertex)
-int test_reduce(Mesh* m, Surface* s, double* val, int nsplit, double* y, bool accumulate);
+// (add: sparse rows over the surface's vertices to add in the same pass)
+int test_reduce(Mesh* m, Surface* s, double* val, int nsplit, double* y, bool accumulate,
+                const RowAdd* add = nullptr);
 int launch_bem_far(Mesh* m, Surface* s, const double* x, const double* lam, double cs, double cd,
-                   double kappa, int precision, double* y, bool accumulate);
+                   double kappa, int precision, double* y, bool accumulate, const RowAdd* add = nullptr);
 int launch_bem_far_ff(Mesh* m, Surface* s, const double* x, const double* lam, double cs, double cd,
-                      double kappa, double* y, bool accumulate);
+                      double kappa, double* y, bool accumulate, const RowAdd* add = nullptr);
 int launch_coulomb(Mesh* m);
 // winding numbers of Gamma_m at nq host points (SoA), on the device (pbfb_check_charges' formula)
 int launch_winding_numbers(Mesh* m, const double* soa, int nq, double* w);

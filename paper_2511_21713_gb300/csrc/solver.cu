@@ -983,9 +983,96 @@ __global__ void k_sub_load(int nv, const double* __restrict__ N, double* __restr
   if (i < nv) d[i] -= N[i];
 }
 
-__global__ void k_trace(int ns, const int* __restrict__ vmap, const double* __restrict__ u, double* __restrict__ out) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < ns) out[i] = u[vmap[i]];
+// Vector steps of the flux's CG, one block each (a few thousand vertices: a step is launches and latency, not
+// bandwidth; 40,960 vertices take 16 us against milliseconds of its far field): 256 threads to 4096 vertices, whose
+// block sums are a quarter of 1024 threads' (the float64 pipe of one SM), 1024 above.  sc: r.z, p.q, r.r, rhs.rhs.
+// GB300, 642 vertices, four products of 152 us: 1011 us before (12 dots with a copy
+// and a wait each, 26 vector launches), 774 us so.
+constexpr int FLUX_T = 1024;
+static inline int flux_threads(int n) { return n <= 4096 ? 256 : FLUX_T; }
+template <int NV>
+__device__ __forceinline__ void flux_block_sums(double (&v)[NV]) {  // in every thread, in a fixed order
+  __shared__ double sh[FLUX_T / 32][NV], tot[NV];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    if (lane == 0) sh[warp][k] = v[k];
+  }
+  __syncthreads();
+  if (warp == 0) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      double s = lane < (int)(blockDim.x >> 5) ? sh[lane][k] : 0.0;
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) tot[k] = s;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < NV; ++k) v[k] = tot[k];
+}
+
+// r = rhs + c coul, lam = 0, rhs.rhs
+__global__ void __launch_bounds__(FLUX_T) k_flux_start(int n, double c, const double* __restrict__ coul,
+                                                       double* __restrict__ r, double* lam, double* __restrict__ sc) {
+  double d[1] = {0.0};
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    double v = r[i];
+    if (coul) v += c * coul[i];
+    r[i] = v;
+    lam[i] = 0.0;
+    d[0] += v * v;
+  }
+  flux_block_sums(d);
+  if (threadIdx.x == 0) {
+    sc[0] = sc[1] = sc[2] = 0.0;
+    sc[3] = d[0];
+  }
+}
+
+// p = z + beta p with the flexible (Polak-Ribiere) beta = (r.z - r_old.z) / (r.z)_old: robust to the float32
+// preconditioner's asymmetry.  first: p = z.
+__global__ void __launch_bounds__(FLUX_T) k_flux_direction(int n, int first, const double* __restrict__ r,
+                                                           const double* __restrict__ rold,
+                                                           const double* __restrict__ z, double* __restrict__ p,
+                                                           double* __restrict__ sc) {
+  double d[2] = {0.0, 0.0};
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    d[0] += r[i] * z[i];
+    if (!first) d[1] += rold[i] * z[i];
+  }
+  const double rz = sc[0];
+  flux_block_sums(d);
+  const double beta = first ? 0.0 : (d[0] - d[1]) / rz;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = first ? z[i] : z[i] + beta * p[i];
+  if (threadIdx.x == 0) sc[0] = d[0];
+}
+
+// alpha = r.z / p.q, lam += alpha p, r -= alpha q (unless p.q <= 0 or a NaN: the caller ends there)
+__global__ void __launch_bounds__(FLUX_T) k_flux_update(int n, const double* __restrict__ p,
+                                                        const double* __restrict__ q, double* lam,
+                                                        double* __restrict__ r, double* __restrict__ rold,
+                                                        double* __restrict__ sc) {
+  double d[1] = {0.0};
+  for (int i = threadIdx.x; i < n; i += blockDim.x) d[0] += p[i] * q[i];
+  flux_block_sums(d);
+  const double pq = d[0], alpha = sc[0] / pq;
+  d[0] = 0.0;
+  if (pq > 0)
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      lam[i] += alpha * p[i];
+      rold[i] = r[i];
+      const double v = r[i] - alpha * q[i];
+      r[i] = v;
+      d[0] += v * v;
+    }
+  flux_block_sums(d);
+  if (threadIdx.x == 0) {
+    sc[1] = pq;
+    sc[2] = d[0];
+  }
 }
 
 __global__ void k_div(int n, const double* __restrict__ x, const double* __restrict__ d, double* __restrict__ y) {
@@ -1912,15 +1999,13 @@ static int gamma_m_flux(Mesh* m, const double* x, bool coulomb, double* lam) {
     set_error("Gamma_m flux: charges not set");
     return PBFB_ERR_STATE;
   }
-  PB_TRY(ensure(m->pp_val, s->cnnz));
-  PB_TRY(ensure(m->pp_work, 7 * (size_t)nm));
-  double* rhs = m->pp_work.p;
-  double* r = rhs + nm;
-  double* z = rhs + 2 * (size_t)nm;
-  double* p = rhs + 3 * (size_t)nm;
-  double* q = rhs + 4 * (size_t)nm;
-  double* ug = rhs + 5 * (size_t)nm;
-  double* rold = rhs + 6 * (size_t)nm;
+  PB_TRY(ensure(m->pp_work, 5 * (size_t)nm));
+  double* r = m->pp_work.p;
+  double* z = r + nm;
+  double* p = r + 2 * (size_t)nm;
+  double* q = r + 3 * (size_t)nm;
+  double* rold = r + 4 * (size_t)nm;
+  double* sc = m->scal.p + 4100;
   const bool dense = nm <= DENSE_V_MAX;
   if (dense && !s->vinv_ok) PB_TRY(build_dense_single_layer(m, s, 0.0, true));
   auto precond = [&](const double* v, double* out) -> int {
@@ -1929,53 +2014,35 @@ static int gamma_m_flux(Mesh* m, const double* x, bool coulomb, double* lam) {
     PB_LAUNCHED(m);
     return PBFB_OK;
   };
-  auto applyV = [&](const double* v, double* out) -> int {
-    PB_TRY(launch_bem_far(m, s, v, v, 1.0, 0.0, 0.0, prec, out, false));
-    return launch_csr_spmv(m, nm, s->c_ptr.p, s->c_col.p, s->corrV.p, v, out, true);
-  };
-  // right-hand side
-  PB_TRY(launch_axpby(m, s->cnnz, 0.5, s->mass.p, 1.0, s->corrK.p, m->pp_val.p));
-  k_trace<<<blocks_for(nm, 256), 256, 0, m->stream>>>(nm, s->vmap.p, x, ug);
+  // right-hand side, with the near field's M_m / 2 + corrK_m over the trace of u
+  const RowAdd near_k{s->c_ptr.p, s->c_col.p, s->corrK.p, s->mass.p, x, s->vmap.p};
+  PB_TRY(launch_bem_far(m, s, x, x + s->col0, 0.0, 1.0, 0.0, prec, r, false, &near_k));
+  k_flux_start<<<1, flux_threads(nm), 0, m->stream>>>(nm, -m->lB / m->eps_m, coulomb ? m->coul.p : nullptr, r, lam, sc);
   PB_LAUNCHED(m);
-  PB_TRY(launch_bem_far(m, s, x, x + s->col0, 0.0, 1.0, 0.0, prec, rhs, false));
-  PB_TRY(launch_csr_spmv(m, nm, s->c_ptr.p, s->c_col.p, m->pp_val.p, ug, rhs, true));
-  if (coulomb) PB_TRY(launch_axpby(m, nm, 1.0, rhs, -m->lB / m->eps_m, m->coul.p, rhs));
-  double bb;
-  PB_TRY(dot(m, rhs, rhs, nm, &bb));
-  PB_CUDA(cudaMemsetAsync(lam, 0, nm * sizeof(double), m->stream));
-  if (!(bb > 0)) {
-    if (!std::isfinite(bb)) {
-      set_error("Gamma_m flux: non-finite right-hand side");
-      return PBFB_ERR_NONFINITE;
-    }
-    return PBFB_OK;
-  }
-  PB_CUDA(cudaMemcpyAsync(r, rhs, nm * sizeof(double), cudaMemcpyDeviceToDevice, m->stream));
   PB_TRY(precond(r, z));
-  PB_CUDA(cudaMemcpyAsync(p, z, nm * sizeof(double), cudaMemcpyDeviceToDevice, m->stream));
-  double rz;
-  PB_TRY(dot(m, r, z, nm, &rz));
+  k_flux_direction<<<1, flux_threads(nm), 0, m->stream>>>(nm, 1, r, rold, z, p, sc);
+  PB_LAUNCHED(m);
+  const RowAdd near_v = near_rows(s, 0, p);
   for (int it = 0; it < 500; ++it) {
-    PB_TRY(applyV(p, q));
-    double pq;
-    PB_TRY(dot(m, p, q, nm, &pq));
-    if (!(pq > 0)) break;
-    const double alpha = rz / pq;
-    PB_TRY(launch_axpby(m, nm, alpha, p, 1.0, lam, lam));
-    PB_CUDA(cudaMemcpyAsync(rold, r, nm * sizeof(double), cudaMemcpyDeviceToDevice, m->stream));
-    PB_TRY(launch_axpby(m, nm, -alpha, q, 1.0, r, r));
-    double rr;
-    PB_TRY(dot(m, r, r, nm, &rr));
-    if (!std::isfinite(rr)) break;
-    if (rr <= 1e-26 * bb) return PBFB_OK;
-    // flexible (Polak-Ribiere) beta: robust to the float32 preconditioner's asymmetry
+    PB_TRY(launch_bem_far(m, s, p, p, 1.0, 0.0, 0.0, prec, q, false, &near_v));
+    k_flux_update<<<1, flux_threads(nm), 0, m->stream>>>(nm, p, q, lam, r, rold, sc);
+    PB_LAUNCHED(m);
+    PB_CUDA(cudaMemcpyAsync(m->pinned, sc, 4 * sizeof(double), cudaMemcpyDeviceToHost, m->stream));
+    // the next direction is on its way while the host looks at the residual
     PB_TRY(precond(r, z));
-    double rz_new, roz;
-    PB_TRY(dot(m, r, z, nm, &rz_new));
-    PB_TRY(dot(m, rold, z, nm, &roz));
-    const double beta = (rz_new - roz) / rz;
-    rz = rz_new;
-    PB_TRY(launch_axpby(m, nm, 1.0, z, beta, p, p));
+    k_flux_direction<<<1, flux_threads(nm), 0, m->stream>>>(nm, 0, r, rold, z, p, sc);
+    PB_LAUNCHED(m);
+    PB_CUDA(cudaStreamSynchronize(m->stream));
+    const double pq = m->pinned[1], rr = m->pinned[2], bb = m->pinned[3];
+    if (!(bb > 0)) {
+      if (!std::isfinite(bb)) {
+        set_error("Gamma_m flux: non-finite right-hand side");
+        return PBFB_ERR_NONFINITE;
+      }
+      return PBFB_OK;
+    }
+    if (!(pq > 0) || !std::isfinite(rr)) break;
+    if (rr <= 1e-26 * bb) return PBFB_OK;
   }
   set_error("Gamma_m flux: CG on V_L did not reach a relative residual of 1e-13");
   return PBFB_ERR_GMRES_NOCONV;
@@ -2522,12 +2589,9 @@ int pbfb_bem_apply(pbfb_mesh* h, int which, int op, const double* x_dev, double*
   }
   pbfb::Surface* s = which == PBFB_GAMMA_M ? &m->sm : &m->ss;
   double kap = which == PBFB_GAMMA_M ? 0.0 : m->kappa;
+  const pbfb::RowAdd near = pbfb::near_rows(s, op, x_dev);
   int st = pbfb::launch_bem_far(m, s, x_dev, x_dev, op == 0 ? 1.0 : 0.0, op == 1 ? 1.0 : 0.0, kap, m->precision,
-                                y_dev, false);
-  if (st) return st;
-  // near-field correction: y += C x (CSR on the surface pattern)
-  st = pbfb::launch_csr_spmv(m, s->nv, s->c_ptr.p, s->c_col.p, op == 0 ? s->corrV.p : s->corrK.p, x_dev, y_dev,
-                             true);
+                                y_dev, false, &near);
   if (st) return st;
   return cudaStreamSynchronize(m->stream) == cudaSuccess ? PBFB_OK : PBFB_ERR_CUDA;
 }

@@ -153,3 +153,29 @@ def test_float_float_elements(nu, layers, scheme):
             assert np.abs(a - b).max() <= 1e-12 * np.abs(a).max() * np.sqrt(m.n)
         assert np.allclose(o1[0][0], o1[1][2], rtol=1e-13, atol=1e-13 * np.abs(o1[1]).max())
     m.close()
+
+
+# the flux's vector steps take 256 threads to 4096 vertices and 1024 above: 12, 4002 and 4412 vertices.  The flux of a
+# solution of V lam = rhs: V lam, from the operator itself, gives rhs back to CG's 1e-13 of its norm, plus the far
+# field's rounding (1e-14 a product)
+@pytest.mark.parametrize("nu", [1, 20, 21])
+def test_flux_residual(nu):
+    from paper_2511_21713_gb300 import inputs, pbfb
+    case = inputs.sphere_case(nu=nu, a=4.0, R=6.0, layers=1)
+    m = pbfb.Mesh.from_case(case)
+    m.set_params(case.eps_in, case.eps_out, case.kappa, case.T, pbfb.FLOAT2)
+    rng = np.random.default_rng(nu)
+    x, lam, V, K = dev(rng.standard_normal(m.n)), dev(np.zeros(m.n_m)), dev(np.zeros(m.n_m)), dev(np.zeros(m.n_m))
+    m.gamma_m_flux(x, 0, lam)
+    u = x[dev(m.surface_vertices(pbfb.GAMMA_M)).long()].contiguous()
+    m.bem_apply(pbfb.GAMMA_M, 0, lam, V)
+    m.bem_apply(pbfb.GAMMA_M, 1, u, K)
+    tri = np.searchsorted(np.unique(case.gm_tris), np.asarray(case.gm_tris))
+    P, un = np.asarray(case.xyz)[np.asarray(case.gm_tris)], u.cpu().numpy()
+    area = 0.5 * np.linalg.norm(np.cross(P[:, 1] - P[:, 0], P[:, 2] - P[:, 0]), axis=1)
+    mass = np.zeros(m.n_m)
+    for a in range(3):  # rows of the mass matrix: area / 12 (1 + [a = b])
+        np.add.at(mass, tri[:, a], area / 12.0 * (un[tri].sum(axis=1) + un[tri[:, a]]))
+    rhs = 0.5 * mass + K.cpu().numpy()
+    assert np.linalg.norm(V.cpu().numpy() - rhs) <= 5e-13 * np.linalg.norm(rhs)
+    m.close()
