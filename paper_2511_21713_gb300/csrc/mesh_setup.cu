@@ -833,6 +833,12 @@ int mesh_create(const double* xyz, int nv, const int* tets, int64_t nt, const in
   sm.col0 = nv;
   ss.col0 = nv + sm.nv;
   m->n = nv + sm.nv + ss.nv;
+  // the surfaces' device geometry and Gamma_m's corrections run while the host builds the pattern below (whose uploads
+  // wait for them: 2880 triangles, 6.6 ms of GPU time beside 5.7 ms of the host's)
+  if ((st = m->red2.alloc(9 * (size_t)std::max(sm.npair, ss.npair)))) return fail(st);
+  if ((st = launch_surface_geometry(m, &sm))) return fail(st);
+  if ((st = launch_surface_geometry(m, &ss))) return fail(st);
+  if ((st = launch_pair_corrections(m, &sm, 0.0))) return fail(st);
   // ---- sparse-part pattern of the coupled operator, row by row: a FEM row has the vertices of its tets, then the
   // surface unknowns of the vertices it shares a triangle with (mass coupling; an interior Gamma_m couples nothing:
   // its lam_m rows are the identity)
@@ -1018,7 +1024,6 @@ int mesh_create(const double* xyz, int nv, const int* tets, int64_t nt, const in
   if ((st = m->tloc.alloc(14 * (size_t)nti))) return fail(st);
   if ((st = m->red.alloc((size_t)152 * 7 * (OMEGA_MAX + 1) + 1024))) return fail(st);
   if ((st = m->scal.alloc(8192))) return fail(st);
-  if ((st = m->red2.alloc(9 * (size_t)std::max(sm.npair, ss.npair)))) return fail(st);
   if (cudaMallocHost((void**)&m->pinned, 4096 * sizeof(double)) != cudaSuccess) {
     set_error("cudaMallocHost failed");
     return fail(PBFB_ERR_OOM);
@@ -1040,9 +1045,6 @@ int mesh_create(const double* xyz, int nv, const int* tets, int64_t nt, const in
     build_charge_grid(m, tm_h);
     m->tets_m_h.swap(tm_h);
   }
-  if ((st = launch_surface_geometry(m, &sm))) return fail(st);
-  if ((st = launch_surface_geometry(m, &ss))) return fail(st);
-  if ((st = launch_pair_corrections(m, &sm, 0.0))) return fail(st);
   sm.kappa = 0.0;
   sm.built = true;
   if (cudaStreamSynchronize(stream) != cudaSuccess) {
