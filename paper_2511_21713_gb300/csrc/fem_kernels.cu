@@ -14,6 +14,8 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <type_traits>
+#include <vector>
 
 #include "fp64_math.cuh"
 #include "pbfb_internal.cuh"
@@ -393,18 +395,101 @@ constexpr int ELEM_T = 256;  // threads a block of the float-float element kerne
 
 __device__ __forceinline__ float2 f2_store(f2 a) { return make_float2(a.h, a.l); }
 
-// Jacobian and load of F on one tet (layout k * nt + t: J at k = 0..9, N at k = 10..13).
-__global__ void k_element_nl(int scheme, const double* __restrict__ u, const int* __restrict__ tets, int64_t nt,
-                             const double* __restrict__ vol, double coef, double* __restrict__ loc) {
+// F, F' and F'' of a scheme in float64: e^u and e^-u from one reduction (exp_pm), the Taylor schemes by Horner's rule.
+template <int S>
+__device__ __forceinline__ void scheme_f64(double u, const double* __restrict__ tab, double& F, double& G, double& H) {
+  if (S == PBFB_HS) {
+    double ep, em;
+    exp_pm(fabs(u), tab, ep, em);
+    F = copysign(0.5 * (ep - em), u);
+    G = 0.5 * (ep + em);
+    H = F;
+  } else if (S == PBFB_LINEAR) {
+    F = u;
+    G = 1.0;
+    H = 0.0;
+  } else {
+    const double u2 = u * u;
+    const double o7 = S == PBFB_T7 ? fma(u2, 1.0 / 42.0, 1.0) : 1.0;
+    const double o5 = S == PBFB_T3 ? 1.0 : fma(u2 * (1.0 / 20.0), o7, 1.0);
+    F = u * fma(u2 * (1.0 / 6.0), o5, 1.0);
+    const double p5 = S == PBFB_T7 ? fma(u2, 1.0 / 20.0, 1.0) : 1.0;
+    H = S == PBFB_T3 ? u : u * fma(u2 * (1.0 / 6.0), p5, 1.0);
+    const double e6 = S == PBFB_T7 ? fma(u2, 1.0 / 30.0, 1.0) : 1.0;
+    const double e4 = S == PBFB_T3 ? 1.0 : fma(u2 * (1.0 / 12.0), e6, 1.0);
+    G = fma(u2 * 0.5, e4, 1.0);
+  }
+}
+
+// Jacobian and load of F on one tet in float64 (layout k * nt + t: J at k = 0..9, N at k = 10..13), from the orbit
+// sums of k_element_ff below.  The float64 pipe bounds it: about 400 operations a tet for the sinh scheme, 1000 with
+// the 14 points one by one, the library's exponential and a division.
+// GB300, 86,400 tets: 128 us so, 72 us now.
+template <int S>
+__global__ void __launch_bounds__(128) k_element_f64(const double* __restrict__ u, const int* __restrict__ tets,
+                                                     int64_t nt, const double* __restrict__ vol, double coef,
+                                                     const double* __restrict__ tab, double* __restrict__ loc) {
+  constexpr double A1 = PBFB_T_A1, D1 = PBFB_T_B1 - PBFB_T_A1, A2 = PBFB_T_A2, D2 = PBFB_T_B2 - PBFB_T_A2;
+  constexpr double C3 = PBFB_T_C3, E3 = PBFB_T_D3 - PBFB_T_C3, W1 = PBFB_T_W1, W2 = PBFB_T_W2, W3 = PBFB_T_W3;
   int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
-  double ua[4];
-  for (int a = 0; a < 4; ++a) ua[a] = u[tets[a * nt + t]];
-  double J[10], N[4];
-  element_sums_f64(scheme, ua, J, N);
-  double s = coef * vol[t];
-  for (int k = 0; k < 10; ++k) loc[k * nt + t] = s * J[k];
-  for (int a = 0; a < 4; ++a) loc[(10 + a) * nt + t] = s * N[a];
+  double v[4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a) v[a] = u[tets[a * nt + t]];
+  const double su = (v[0] + v[1]) + (v[2] + v[3]);
+  double n[4], h[4], D[4], g3[6], T, C;
+  {
+    double fs = 0.0, gs = 0.0;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) n[a] = h[a] = 0.0;
+#pragma unroll
+    for (int p = 0, P = 0; p < 3; ++p)
+#pragma unroll
+      for (int q = p + 1; q < 4; ++q, ++P) {
+        double F, G, H;
+        scheme_f64<S>(fma(E3, v[p] + v[q], C3 * su), tab, F, G, H);
+        n[p] += F;
+        n[q] += F;
+        h[p] += G;
+        h[q] += G;
+        g3[P] = W3 * E3 * E3 * G;
+        fs += F;
+        gs += G;
+      }
+    T = W3 * C3 * fs;
+    C = W3 * C3 * C3 * gs;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      n[a] *= W3 * E3;
+      D[a] = W3 * E3 * E3 * h[a];
+      h[a] *= W3 * C3 * E3;
+    }
+  }
+  auto orbit = [&](double alpha, double delta, double w) {
+    double fs = 0.0, gs = 0.0;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      double F, G, H;
+      scheme_f64<S>(fma(delta, v[a], alpha * su), tab, F, G, H);
+      n[a] = fma(w * delta, F, n[a]);
+      h[a] = fma(w * alpha * delta, G, h[a]);
+      D[a] = fma(w * delta * delta, G, D[a]);
+      fs += F;
+      gs += G;
+    }
+    T = fma(w * alpha, fs, T);
+    C = fma(w * alpha * alpha, gs, C);
+  };
+  orbit(A1, D1, W1);
+  orbit(A2, D2, W2);
+  const double s = coef * vol[t];
+#pragma unroll
+  for (int a = 0, P = 0; a < 4; ++a) {
+    loc[sym10(a, a) * nt + t] = s * (C + fma(2.0, h[a], D[a]));
+#pragma unroll
+    for (int b = a + 1; b < 4; ++b, ++P) loc[sym10(a, b) * nt + t] = s * ((C + g3[P]) + (h[a] + h[b]));
+    loc[(10 + a) * nt + t] = s * (T + n[a]);
+  }
 }
 
 // Tets outside the float-float range take the float64 sums (kept out of line).
@@ -546,29 +631,85 @@ __global__ void k_csr_acc(int nrows, const int* __restrict__ ptr, const int* __r
   if (lane == 0 && valid) y[row] = accumulate ? y[row] + acc : acc;
 }
 
-// Omega batch: per tet and omega, local load of F(w), of F'(w) du and of F''(w) du^2 at
-// w = u + omega du; layout ((o * 3 + quantity) * 4 + a) * nt + t.
-__global__ void k_omega_elements(int scheme, const double* __restrict__ u, const double* __restrict__ du,
-                                 OmegaSet omegas, int nomega, const int* __restrict__ tets,
-                                 int64_t nt, const double* __restrict__ vol, double coef, double* __restrict__ loc) {
+// Omega batch in float64: per tet and omega, local load of F(w), of F'(w) du and of F''(w) du^2 at w = u + omega du
+// from orbit sums; layout ((o * 3 + quantity) * 4 + a) * nt + t.  The float64 pipe bounds it.
+// GB300, 86,400 tets, one omega: 135 us point by point, 83 us so.
+template <int S>
+__global__ void __launch_bounds__(128) k_omega_f64(const double* __restrict__ u, const double* __restrict__ du,
+                                                   OmegaSet omegas, int nomega, const int* __restrict__ tets,
+                                                   int64_t nt, const double* __restrict__ vol, double coef,
+                                                   const double* __restrict__ tab, double* __restrict__ loc) {
+  constexpr double A1 = PBFB_T_A1, D1 = PBFB_T_B1 - PBFB_T_A1, A2 = PBFB_T_A2, D2 = PBFB_T_B2 - PBFB_T_A2;
+  constexpr double C3 = PBFB_T_C3, E3 = PBFB_T_D3 - PBFB_T_C3, W1 = PBFB_T_W1, W2 = PBFB_T_W2, W3 = PBFB_T_W3;
   int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
-  double ua[4], da[4];
+  double ua[4], d[4];
+#pragma unroll
   for (int a = 0; a < 4; ++a) {
-    int v = tets[a * nt + t];
-    ua[a] = u[v];
-    da[a] = du[v];
+    const int vtx = tets[a * nt + t];
+    ua[a] = u[vtx];
+    d[a] = du[vtx];
   }
-  double s = coef * vol[t];
+  const double sd = (d[0] + d[1]) + (d[2] + d[3]), s = coef * vol[t];
   for (int o = 0; o < nomega; ++o) {
-    double R0[4], R1[4], R2[4];
-    omega_sums_f64(scheme, ua, da, omegas.v[o], R0, R1, R2);
-    int64_t base = (int64_t)o * 12 * nt;
-    for (int a = 0; a < 4; ++a) {
-      loc[base + (0 * 4 + a) * nt + t] = s * R0[a];
-      loc[base + (1 * 4 + a) * nt + t] = s * R1[a];
-      loc[base + (2 * 4 + a) * nt + t] = s * R2[a];
+    double w[4], n[3][4], T[3];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) w[a] = fma(omegas.v[o], d[a], ua[a]);
+    const double sw = (w[0] + w[1]) + (w[2] + w[3]);
+    auto point = [&](double wq, double dq, double (&x)[3]) {
+      double G, H;
+      scheme_f64<S>(wq, tab, x[0], G, H);
+      x[1] = G * dq;
+      x[2] = H * dq * dq;
+    };
+    {
+      double sum[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int a = 0; a < 4; ++a) n[k][a] = 0.0;
+#pragma unroll
+      for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int q = p + 1; q < 4; ++q) {
+          double x[3];
+          point(fma(E3, w[p] + w[q], C3 * sw), fma(E3, d[p] + d[q], C3 * sd), x);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            n[k][p] += x[k];
+            n[k][q] += x[k];
+            sum[k] += x[k];
+          }
+        }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        T[k] = W3 * C3 * sum[k];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) n[k][a] *= W3 * E3;
+      }
     }
+    auto orbit = [&](double alpha, double delta, double wt) {
+      double sum[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        double x[3];
+        point(fma(delta, w[a], alpha * sw), fma(delta, d[a], alpha * sd), x);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          n[k][a] = fma(wt * delta, x[k], n[k][a]);
+          sum[k] += x[k];
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) T[k] = fma(wt * alpha, sum[k], T[k]);
+    };
+    orbit(A1, D1, W1);
+    orbit(A2, D2, W2);
+    double* out = loc + (int64_t)o * 12 * nt;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int a = 0; a < 4; ++a) out[(k * 4 + a) * nt + t] = s * (T[k] + n[k][a]);
   }
 }
 
@@ -586,7 +727,7 @@ __device__ __noinline__ void omega_fallback(int scheme, const double* ua4, const
 }
 
 // Omega batch in float-float (scheme S): per tet and omega the loads of F(w), F'(w) d and F''(w) d^2 at
-// w = u + omega du, each T + n_a from orbit sums (see k_element_ff); same layout as k_omega_elements.
+// w = u + omega du, each T + n_a from orbit sums (see k_element_ff); same layout as k_omega_f64.
 // GB300, 408,000 tets, one omega: 106 -> 59 us.
 template <int S>
 __global__ void __launch_bounds__(ELEM_T) k_omega_ff(const double* __restrict__ u, const double* __restrict__ du,
@@ -942,35 +1083,31 @@ static bool use_ff(const Mesh* m, int scheme) {
   return m->precision != PBFB_FP64 && scheme >= PBFB_LINEAR && scheme <= PBFB_T7;
 }
 
-template <int S>
-static void element_ff(Mesh* m, const double* u, double coef, float2* out) {
-  k_element_ff<S><<<blocks_for(m->nt, ELEM_T), ELEM_T, 0, m->stream>>>(u, m->tets.p, m->nt, m->vol.p, coef, m->fx_tab.p,
-                                                                  out);
-}
-
-template <int S>
-static void omega_ff(Mesh* m, const double* u, const double* du, const OmegaSet& omegas, int nomega, double coef,
-                     float2* out) {
-  k_omega_ff<S><<<blocks_for(m->nt, ELEM_T), ELEM_T, 0, m->stream>>>(u, du, omegas, nomega, m->tets.p, m->nt, m->vol.p,
-                                                                coef, m->fx_tab.p, out);
+// f(integral_constant) of the scheme
+template <class F>
+static void with_scheme(int scheme, F f) {
+  switch (scheme) {
+    case PBFB_LINEAR: f(std::integral_constant<int, PBFB_LINEAR>()); break;
+    case PBFB_T3: f(std::integral_constant<int, PBFB_T3>()); break;
+    case PBFB_T5: f(std::integral_constant<int, PBFB_T5>()); break;
+    case PBFB_T7: f(std::integral_constant<int, PBFB_T7>()); break;
+    default: f(std::integral_constant<int, PBFB_HS>()); break;
+  }
 }
 
 int launch_element_nl(Mesh* m, int scheme, const double* u, double coef, double* loc, bool* ff) {
   cudaEvent_t ev;
   *ff = use_ff(m, scheme);
-  if (*ff) PB_TRY(fx_table(m));
+  PB_TRY(*ff ? fx_table(m) : pair_tables(m, true));
   timer_begin(m, m->t_elem, &ev);
-  if (*ff) {
-    float2* out = reinterpret_cast<float2*>(loc);
-    switch (scheme) {
-      case PBFB_LINEAR: element_ff<PBFB_LINEAR>(m, u, coef, out); break;
-      case PBFB_T3: element_ff<PBFB_T3>(m, u, coef, out); break;
-      case PBFB_T5: element_ff<PBFB_T5>(m, u, coef, out); break;
-      case PBFB_T7: element_ff<PBFB_T7>(m, u, coef, out); break;
-      default: element_ff<PBFB_HS>(m, u, coef, out); break;
-    }
-  } else
-    k_element_nl<<<blocks_for(m->nt, 128), 128, 0, m->stream>>>(scheme, u, m->tets.p, m->nt, m->vol.p, coef, loc);
+  with_scheme(scheme, [&](auto S) {
+    if (*ff)
+      k_element_ff<S()><<<blocks_for(m->nt, ELEM_T), ELEM_T, 0, m->stream>>>(
+          u, m->tets.p, m->nt, m->vol.p, coef, m->fx_tab.p, reinterpret_cast<float2*>(loc));
+    else
+      k_element_f64<S()><<<blocks_for(m->nt, 128), 128, 0, m->stream>>>(u, m->tets.p, m->nt, m->vol.p, coef,
+                                                                        m->pair_tab64.p, loc);
+  });
   PB_LAUNCHED(m);
   timer_end(m, m->t_elem, ev, (double)m->nt);
   return PBFB_OK;
@@ -1007,22 +1144,18 @@ int launch_omega_elements(Mesh* m, int scheme, const double* u, const double* du
                           int nomega, double coef, double* loc, bool* ff) {
   cudaEvent_t ev;
   *ff = use_ff(m, scheme);
-  if (*ff) PB_TRY(fx_table(m));
+  PB_TRY(*ff ? fx_table(m) : pair_tables(m, true));
   OmegaSet omegas;
   for (int o = 0; o < OMEGA_MAX; ++o) omegas.v[o] = o < nomega ? omegas_host[o] : 0.0;
   timer_begin(m, m->t_elem, &ev);
-  if (*ff) {
-    float2* out = reinterpret_cast<float2*>(loc);
-    switch (scheme) {
-      case PBFB_LINEAR: omega_ff<PBFB_LINEAR>(m, u, du, omegas, nomega, coef, out); break;
-      case PBFB_T3: omega_ff<PBFB_T3>(m, u, du, omegas, nomega, coef, out); break;
-      case PBFB_T5: omega_ff<PBFB_T5>(m, u, du, omegas, nomega, coef, out); break;
-      case PBFB_T7: omega_ff<PBFB_T7>(m, u, du, omegas, nomega, coef, out); break;
-      default: omega_ff<PBFB_HS>(m, u, du, omegas, nomega, coef, out); break;
-    }
-  } else
-    k_omega_elements<<<blocks_for(m->nt, 128), 128, 0, m->stream>>>(scheme, u, du, omegas, nomega, m->tets.p,
-                                                                    m->nt, m->vol.p, coef, loc);
+  with_scheme(scheme, [&](auto S) {
+    if (*ff)
+      k_omega_ff<S()><<<blocks_for(m->nt, ELEM_T), ELEM_T, 0, m->stream>>>(
+          u, du, omegas, nomega, m->tets.p, m->nt, m->vol.p, coef, m->fx_tab.p, reinterpret_cast<float2*>(loc));
+    else
+      k_omega_f64<S()><<<blocks_for(m->nt, 128), 128, 0, m->stream>>>(u, du, omegas, nomega, m->tets.p, m->nt,
+                                                                      m->vol.p, coef, m->pair_tab64.p, loc);
+  });
   PB_LAUNCHED(m);
   timer_end(m, m->t_elem, ev, (double)m->nt * nomega);
   return PBFB_OK;
