@@ -45,12 +45,9 @@ FLOP_PAIR = {"laplace": 20.0, "yukawa": 28.0}
 # pbfb_newton_opts.residual_far: PBFB_FLOAT2 (float-float direct sum) or PBFB_MIXED (float32 operator)
 RESIDUAL_FAR = {"float2": 2, "f32": 1}
 GOLDEN = os.path.join(ROOT, "tests", "golden", "multi_charge_sphere.json")
-# DRAM bytes (read + write) per launch on this workload, each from an ncu capture of the kernel
-# (dram__bytes_read.sum + dram__bytes_write.sum): the packed float32 far field (source records
-# read once) and the packed mutual float-float far field
+# DRAM bytes (read + write) per launch on this workload, from an ncu capture of the packed float32
+# far field (dram__bytes_read.sum + dram__bytes_write.sum; source records read once)
 NBODY_TRAFFIC = 2311424.0
-FF2_TRAFFIC = 15.17e6
-FF_TRAFFIC = 15.2e6
 # float32 lane operations (FADD, FMUL, FFMA each 1; a packed instruction 2) per ordered pair that
 # the float-float evaluation by pairs of triangles issues, counted in its source: the emulation's
 # cost, against 20 / 28 flops of the method's own arithmetic
