@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(32 * PW, NP == 3 ? 2 : 3)
     k_pairs_ff(int nt, int ntask, int nT, int tpg, int G, int K, const float* __restrict__ geo,
                const float* __restrict__ src, const float2* __restrict__ tab, double* PI,
                double* PJ) {
-  __shared__ float s_tile[PW][(FF_GEO + FF_SRC) * PT];
+  __shared__ __align__(16) float s_tile[PW][(FF_GEO + FF_SRC) * PT];  // filled by float4 stores
   __shared__ float2 s_acc[PW][QS][PT];
   __shared__ float2 s_tab[YUK ? FF_HI + FF_LO : 1];
   if (YUK) {
@@ -378,7 +378,7 @@ __global__ void __launch_bounds__(32 * PW, 2)
     k_pairs_f64(int nt, int ntask, int nT, int tpg, int G, int K, const double* __restrict__ geo,
                 const double* __restrict__ src, const double* __restrict__ tab, double kappa,
                 double* PI, double* PJ) {
-  extern __shared__ double smem[];
+  extern __shared__ __align__(16) double smem[];  // tiles filled by double2 stores
   double* s_tab = smem;  // 2^(-k / 2048) (Yukawa)
   double* s_warp = smem + (YUK ? EXP2_TAB : 0);
   if (YUK) {
