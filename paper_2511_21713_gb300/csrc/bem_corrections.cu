@@ -368,7 +368,7 @@ std::vector<Row> touching_rows(const double* x, const double* w) {
 
 }  // namespace
 
-// tables of the accurate rules, once (called by init_quadrature)
+// tables of the accurate rules on the current device (called by init_quadrature, once per device)
 int init_correction_rules() {
   double x[NGL], w[NGL];
   gauss_legendre01(NGL, x, w);

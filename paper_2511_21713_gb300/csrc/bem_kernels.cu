@@ -18,9 +18,9 @@
 
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 #include <vector>
 
+#include "device_once.h"
 #include "f32x2.cuh"
 #include "fp64_math.cuh"
 #include "pbfb_internal.cuh"
@@ -902,22 +902,24 @@ inline int blocks_for(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
 }  // namespace
 
+// Constant tables of the quadrature rules and of the float-float exponential, once per device (called by mesh
+// creation, before any launch)
 int init_quadrature() {
-  static std::mutex mu;
-  static bool done = false;
-  std::lock_guard<std::mutex> lk(mu);
-  if (done) return PBFB_OK;
-  PB_TRY(init_correction_rules());
-  // float-float exp tables: exp(-k0 / 256), k0 < 16 (constant memory)
-  float2 lo[16];
-  for (int k = 0; k < 16; ++k) {
-    double v = std::exp(-k / 256.0);
-    float h = (float)v;
-    lo[k] = make_float2(h, (float)(v - (double)h));
-  }
-  PB_CUDA(cudaMemcpyToSymbol(c_ff_exp_lo, lo, sizeof(lo)));
-  done = true;
-  return PBFB_OK;
+  static DeviceOnce once;
+  int dev = 0;
+  PB_CUDA(cudaGetDevice(&dev));
+  return once.run(dev, []() -> int {
+    PB_TRY(init_correction_rules());
+    // float-float exp tables: exp(-k0 / 256), k0 < 16 (constant memory)
+    float2 lo[16];
+    for (int k = 0; k < 16; ++k) {
+      double v = std::exp(-k / 256.0);
+      float h = (float)v;
+      lo[k] = make_float2(h, (float)(v - (double)h));
+    }
+    PB_CUDA(cudaMemcpyToSymbol(c_ff_exp_lo, lo, sizeof(lo)));
+    return PBFB_OK;
+  });
 }
 
 // exp(-16 k1 / 256), k1 < FF_TABLE_HI, as float-float pairs (host-computed in float64)
