@@ -22,8 +22,8 @@
 
 #include <algorithm>
 #include <cstdint>
-#include <mutex>
 
+#include "device_once.h"
 #include "f32x2.cuh"
 #include "pbfb_internal.cuh"
 #include "quad_tables.cuh"
@@ -512,20 +512,18 @@ int build_dense_single_layer(Mesh* m, Surface* s, double kappa, bool invert) {
 // then never change a kernel's attributes while another thread launches or captures it, and a
 // smaller matrix never lowers the limit a larger one needs.
 int init_dense_attributes() {
-  static std::mutex mu;
-  static uint64_t done = 0;
+  static DeviceOnce once;
   int dev = 0;
   PB_CUDA(cudaGetDevice(&dev));
-  std::lock_guard<std::mutex> lk(mu);
-  if (dev < 64 && ((done >> dev) & 1)) return PBFB_OK;
-  PB_CUDA(cudaFuncSetAttribute(k_sweep_update, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               2 * SW_B * SW_TILE * (int)sizeof(float)));
-  for (const void* f : {(const void*)k_dense_rows<true>, (const void*)k_dense_rows<false>})
-    PB_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, DW_SMEM));
-  PB_CUDA(cudaFuncSetAttribute(k_dense_apply, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               dense_ld(DENSE_V_MAX) * (int)sizeof(float)));
-  if (dev < 64) done |= 1ull << dev;
-  return PBFB_OK;
+  return once.run(dev, []() -> int {
+    PB_CUDA(cudaFuncSetAttribute(k_sweep_update, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 2 * SW_B * SW_TILE * (int)sizeof(float)));
+    for (const void* f : {(const void*)k_dense_rows<true>, (const void*)k_dense_rows<false>})
+      PB_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, DW_SMEM));
+    PB_CUDA(cudaFuncSetAttribute(k_dense_apply, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 dense_ld(DENSE_V_MAX) * (int)sizeof(float)));
+    return PBFB_OK;
+  });
 }
 
 int launch_dense_apply(Mesh* m, Surface* s, double scale, const double* v, double* z) {

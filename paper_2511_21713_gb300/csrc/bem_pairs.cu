@@ -34,6 +34,7 @@
 #include <cmath>
 #include <vector>
 
+#include "device_once.h"
 #include "f32x2.cuh"
 #include "fp64_math.cuh"
 #include "pbfb_internal.cuh"
@@ -732,12 +733,18 @@ int launch_pairs(Mesh* m, Surface* s, const double* x, const double* lam, double
   return PBFB_OK;
 }
 
-// Shared-memory limits of the float64 form, once per device (called by mesh creation, before any launch)
+// Shared-memory limits of the float64 form, once per device (called by mesh creation, before any launch): later mesh
+// creations leave the kernels' attributes alone while other host threads launch them
 int init_pair_attributes() {
-  const int smem = (EXP2_TAB + PW * (D_GEO + D_SRC + QS) * PT) * (int)sizeof(double);
-  for (const void* f : {(const void*)k_pairs_f64<true>, (const void*)k_pairs_f64<false>})
-    PB_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  return PBFB_OK;
+  static DeviceOnce once;
+  int dev = 0;
+  PB_CUDA(cudaGetDevice(&dev));
+  return once.run(dev, []() -> int {
+    const int smem = (EXP2_TAB + PW * (D_GEO + D_SRC + QS) * PT) * (int)sizeof(double);
+    for (const void* f : {(const void*)k_pairs_f64<true>, (const void*)k_pairs_f64<false>})
+      PB_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    return PBFB_OK;
+  });
 }
 
 }  // namespace pbfb

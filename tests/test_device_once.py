@@ -61,7 +61,7 @@ def body(name):
     raise AssertionError(name)
 
 
-@pytest.mark.parametrize("name", ["init_quadrature"])
+@pytest.mark.parametrize("name", ["init_quadrature", "init_pair_attributes", "init_dense_attributes"])
 def test_set_up_is_per_device(name):
     b = body(name)
     assert "DeviceOnce" in b and "cudaGetDevice" in b
