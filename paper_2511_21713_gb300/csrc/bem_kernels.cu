@@ -918,6 +918,8 @@ int init_quadrature() {
       lo[k] = make_float2(h, (float)(v - (double)h));
     }
     PB_CUDA(cudaMemcpyToSymbol(c_ff_exp_lo, lo, sizeof(lo)));
+    // the copies run on the legacy stream, which a mesh's own (non-blocking) stream does not wait for
+    PB_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
     return PBFB_OK;
   });
 }

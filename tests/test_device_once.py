@@ -70,3 +70,11 @@ def test_set_up_is_per_device(name):
 def test_no_flag_per_process():
     for path in glob.glob(os.path.join(CSRC, "*.cu")):
         assert not re.search(r"static\s+(?:std::atomic<)?bool>?\s+\w+\s*(?:=|;|\{)", open(path).read()), path
+
+
+def test_symbol_copies_are_waited_for():
+    """The tables are copied on the legacy stream from pageable memory, so that a copy may still be on its way when
+    the call returns; meshes run on non-blocking streams, which wait for no other."""
+    b = body("init_quadrature")
+    last = max(b.index("init_correction_rules"), b.rindex("cudaMemcpyToSymbol"))
+    assert "cudaStreamSynchronize(cudaStreamLegacy)" in b[last:]
