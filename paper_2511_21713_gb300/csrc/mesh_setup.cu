@@ -11,13 +11,12 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
-#include <exception>
 #include <string>
-#include <system_error>
 #include <thread>
 #include <unordered_map>
 #include <vector>
 
+#include "host_ranges.h"
 #include "pbfb_internal.cuh"
 #include "quad_tables.cuh"
 
@@ -27,35 +26,6 @@ namespace {
 
 thread_local std::string g_err;
 
-// f(k, i0, i1) for a partition of [0, n) into ranges k = 0, 1, ... on up to 16 host threads, each with `grain` items
-// or more; the same n and grain give the same partition.  An exception of a range is rethrown here.
-constexpr int HOST_THREADS = 16;
-template <class F>
-void parallel_ranges(int64_t n, int64_t grain, F f) {
-  const int64_t hw = std::max(1u, std::min((unsigned)HOST_THREADS, std::thread::hardware_concurrency()));
-  const int nth = (int)std::max<int64_t>(1, std::min(hw, n / grain));
-  std::exception_ptr err[HOST_THREADS];
-  auto run = [&](int k) {
-    try {
-      f(k, n * k / nth, n * (k + 1) / nth);
-    } catch (...) {
-      err[k] = std::current_exception();
-    }
-  };
-  std::thread th[HOST_THREADS];
-  int k = 1;
-  try {
-    for (; k < nth; ++k) th[k] = std::thread(run, k);
-  } catch (const std::system_error&) {  // no more threads: the rest runs here
-  }
-  const int started = k;
-  run(0);
-  for (; k < nth; ++k) run(k);
-  for (int q = 1; q < started; ++q) th[q].join();
-  for (int q = 0; q < nth; ++q)
-    if (err[q]) std::rethrow_exception(err[q]);
-}
-
 // counting sort of the values val(e), e = 0..n-1, by keys[e] in [0, nkeys): ptr (nkeys + 1) and the values, in
 // ascending e within a key.  A thread takes a range of the keys and reads all of them (sequentially: a fraction of
 // the scattered writes).
@@ -63,18 +33,18 @@ template <class V>
 void bucket(const int* keys, int64_t n, int nkeys, V val, std::vector<int>& ptr, std::vector<int>& out) {
   ptr.assign(nkeys + 1, 0);
   out.resize(n);
-  auto ranges = [&](auto f) { parallel_ranges(n < 40000 ? 1 : nkeys, n < 40000 ? 1 : std::max(1, nkeys / 16), f); };
+  const HostRanges ranges(n < 40000 ? 1 : nkeys, n < 40000 ? 1 : std::max(1, nkeys / 16));
   auto clip = [&](int64_t& k0, int64_t& k1) {
     if (n < 40000) k0 = 0, k1 = nkeys;
   };
-  ranges([&](int, int64_t k0, int64_t k1) {
+  ranges.run([&](int, int64_t k0, int64_t k1) {
     clip(k0, k1);
     for (int64_t e = 0; e < n; ++e)
       if (keys[e] >= k0 && keys[e] < k1) ptr[keys[e] + 1]++;
   });
   for (int i = 0; i < nkeys; ++i) ptr[i + 1] += ptr[i];
   std::vector<int> pos(ptr.begin(), ptr.end() - 1);
-  ranges([&](int, int64_t k0, int64_t k1) {
+  ranges.run([&](int, int64_t k0, int64_t k1) {
     clip(k0, k1);
     for (int64_t e = 0; e < n; ++e)
       if (keys[e] >= k0 && keys[e] < k1) out[pos[keys[e]]++] = val(e);
@@ -148,7 +118,7 @@ void classify_pairs(const HostSurface& hs, std::vector<int>& pptr, std::vector<i
   }
   // near pairs, both orientations, from per-thread buffers merged in thread (= triangle) order
   std::vector<int> found[HOST_THREADS];
-  parallel_ranges(nt, 32, [&](int k, int64_t t0, int64_t t1) {
+  HostRanges(nt, 32).run([&](int k, int64_t t0, int64_t t1) {
     std::vector<int> stamp(nt, -1);
     std::vector<int>& out = found[k];
     for (int t = (int)t0; t < (int)t1; ++t) {
@@ -202,7 +172,8 @@ void classify_pairs(const HostSurface& hs, std::vector<int>& pptr, std::vector<i
     std::vector<int> s, cls, perm;
   } rows[HOST_THREADS];
   pptr.assign(nt + 1, 0);
-  parallel_ranges(nt, 64, [&](int k, int64_t t0, int64_t t1) {
+  const HostRanges ranges(nt, 64);
+  ranges.run([&](int k, int64_t t0, int64_t t1) {
     std::vector<int> cnt(nt, 0), touched;
     std::vector<std::array<int, 2>> row;  // (s, class)
     Rows& out = rows[k];
@@ -264,7 +235,7 @@ void classify_pairs(const HostSurface& hs, std::vector<int>& pptr, std::vector<i
   ps.resize(np);
   cls.resize(np);
   perm.resize(6 * (size_t)np);
-  parallel_ranges(nt, 64, [&](int k, int64_t t0, int64_t t1) {
+  ranges.run([&](int k, int64_t t0, int64_t t1) {
     const int p0 = pptr[t0];
     std::copy(rows[k].s.begin(), rows[k].s.end(), ps.begin() + p0);
     std::copy(rows[k].cls.begin(), rows[k].cls.end(), cls.begin() + p0);
@@ -341,7 +312,8 @@ int build_surface(Mesh* m, Surface* s, const std::vector<int>& gtri, const std::
     // sizes, and the distinct columns (a marker per column), sorted
     std::vector<int> dptr(s->nv + 1, 0), eptr(s->nv + 1, 0), cols[HOST_THREADS];
     s->c_ptr_h.assign(s->nv + 1, 0);
-    parallel_ranges(s->nv, 32, [&](int k, int64_t i0, int64_t i1) {
+    const HostRanges ranges(s->nv, 32);
+    ranges.run([&](int k, int64_t i0, int64_t i1) {
       std::vector<int> mark(s->nv, -1);
       for (int i = (int)i0; i < (int)i1; ++i) {
         const size_t w0 = cols[k].size();
@@ -366,7 +338,7 @@ int build_surface(Mesh* m, Surface* s, const std::vector<int>& gtri, const std::
     s->c_col_h.resize(s->cnnz);
     std::vector<int> cgp(s->cnnz + 1), cgi(eptr[s->nv]), dgi(dptr[s->nv]);
     cgp[s->cnnz] = eptr[s->nv];
-    parallel_ranges(s->nv, 32, [&](int k, int64_t i0, int64_t i1) {
+    ranges.run([&](int k, int64_t i0, int64_t i1) {
       std::copy(cols[k].begin(), cols[k].end(), s->c_col_h.begin() + s->c_ptr_h[i0]);
       std::vector<int> rank(s->nv), pos;
       for (int i = (int)i0; i < (int)i1; ++i) {
@@ -485,7 +457,7 @@ static int validate(const double* xyz, int nv, const int* tets, int64_t nt, cons
   std::vector<uint64_t> fother(4 * (size_t)nt);
   int64_t degenerate[HOST_THREADS];
   std::fill(degenerate, degenerate + HOST_THREADS, nt);
-  parallel_ranges(nt, 4096, [&](int th, int64_t t0, int64_t t1) {
+  HostRanges(nt, 4096).run([&](int th, int64_t t0, int64_t t1) {
     for (int64_t t = t0; t < t1; ++t) {
       const int* T = tets + 4 * t;
       double e[3][3];
@@ -523,7 +495,7 @@ static int validate(const double* xyz, int nv, const int* tets, int64_t nt, cons
   std::vector<char> fcount(ford.size(), 0);
   size_t nbs[HOST_THREADS] = {}, nifs[HOST_THREADS] = {};
   bool more[HOST_THREADS] = {};
-  parallel_ranges(nv, 512, [&](int th, int64_t v0, int64_t v1) {
+  HostRanges(nv, 512).run([&](int th, int64_t v0, int64_t v1) {
     for (size_t q = fptr[v0]; q < (size_t)fptr[v1]; ++q) face[q] = {fother[ford[q]], ford[q]};
     for (int64_t v = v0; v < v1; ++v) {
       std::sort(face.begin() + fptr[v], face.begin() + fptr[v + 1]);
@@ -870,7 +842,8 @@ int mesh_create(const double* xyz, int nv, const int* tets, int64_t nt, const in
   // row sizes; the FEM columns, distinct (a marker per column) and sorted
   std::vector<int> cols[HOST_THREADS];
   m->s_ptr_h.assign(m->n + 1, 0);
-  parallel_ranges(nv, 256, [&](int k, int64_t v0, int64_t v1) {
+  const HostRanges ranges(nv, 256);
+  ranges.run([&](int k, int64_t v0, int64_t v1) {
     std::vector<int> mark(nv, -1);
     std::vector<int>& out = cols[k];
     for (int v = (int)v0; v < (int)v1; ++v) {
@@ -918,7 +891,7 @@ int mesh_create(const double* xyz, int nv, const int* tets, int64_t nt, const in
       jp[r].assign(m->snnz + 1, (int)(16 * tn[r]));
       ji[r].resize(16 * tn[r]);
     }
-    parallel_ranges(nv, 256, [&](int k, int64_t v0, int64_t v1) {
+    ranges.run([&](int k, int64_t v0, int64_t v1) {
       std::vector<int> rank(nv), pos;
       const int* src = cols[k].data();
       for (int v = (int)v0; v < (int)v1; ++v) {
