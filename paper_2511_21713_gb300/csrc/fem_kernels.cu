@@ -421,6 +421,21 @@ __device__ __forceinline__ void scheme_f64(double u, const double* __restrict__ 
   }
 }
 
+// The float64 loops' orbit sums hold where F stays finite.  Past |u| = 700 (upper word compared as integers; infinities
+// and NaN are above) a tet takes the rule point by point, whose weights are all positive: sums past the range are then
+// infinite with F's sign, where the second orbit's negative beta - alpha would make inf - inf of them.
+constexpr int ORBIT_MAX_HI = 0x4085E000;
+__device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7fffffff; }
+
+__device__ __noinline__ void element_wide(int scheme, const double* ua4, double sc, int64_t nt, int64_t t,
+                                          double* __restrict__ loc) {
+  const double ua[4] = {ua4[0], ua4[1], ua4[2], ua4[3]};
+  double J[10], N[4];
+  element_sums_f64(scheme, ua, J, N);
+  for (int k = 0; k < 10; ++k) loc[k * nt + t] = sc * J[k];
+  for (int a = 0; a < 4; ++a) loc[(10 + a) * nt + t] = sc * N[a];
+}
+
 // Jacobian and load of F on one tet in float64 (layout k * nt + t: J at k = 0..9, N at k = 10..13), from the orbit
 // sums of k_element_ff below.  The float64 pipe bounds it: about 400 operations a tet for the sinh scheme, 1000 with
 // the 14 points one by one, the library's exponential and a division.
@@ -434,8 +449,16 @@ __global__ void __launch_bounds__(128) k_element_f64(const double* __restrict__ 
   int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
   double v[4];
+  int vmax = 0;
 #pragma unroll
-  for (int a = 0; a < 4; ++a) v[a] = u[tets[a * nt + t]];
+  for (int a = 0; a < 4; ++a) {
+    v[a] = u[tets[a * nt + t]];
+    vmax = max(vmax, abs_hi(v[a]));
+  }
+  if (vmax >= ORBIT_MAX_HI) {
+    element_wide(S, v, coef * vol[t], nt, t, loc);
+    return;
+  }
   const double su = (v[0] + v[1]) + (v[2] + v[3]);
   double n[4], h[4], D[4], g3[6], T, C;
   {
@@ -631,6 +654,19 @@ __global__ void k_csr_acc(int nrows, const int* __restrict__ ptr, const int* __r
   if (lane == 0 && valid) y[row] = accumulate ? y[row] + acc : acc;
 }
 
+// one omega of a tet with a value or a step past the orbit sums' range
+__device__ __noinline__ void omega_wide(int scheme, const double* ua4, const double* da4, double om, double sc, int64_t nt,
+                                        int64_t t, double* __restrict__ out) {
+  const double ua[4] = {ua4[0], ua4[1], ua4[2], ua4[3]}, da[4] = {da4[0], da4[1], da4[2], da4[3]};
+  double R0[4], R1[4], R2[4];
+  omega_sums_f64(scheme, ua, da, om, R0, R1, R2);
+  for (int a = 0; a < 4; ++a) {
+    out[(0 * 4 + a) * nt + t] = sc * R0[a];
+    out[(1 * 4 + a) * nt + t] = sc * R1[a];
+    out[(2 * 4 + a) * nt + t] = sc * R2[a];
+  }
+}
+
 // Omega batch in float64: per tet and omega, local load of F(w), of F'(w) du and of F''(w) du^2 at w = u + omega du
 // from orbit sums; layout ((o * 3 + quantity) * 4 + a) * nt + t.  The float64 pipe bounds it.
 // GB300, 86,400 tets, one omega: 135 us point by point, 83 us so.
@@ -644,17 +680,28 @@ __global__ void __launch_bounds__(128) k_omega_f64(const double* __restrict__ u,
   int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
   double ua[4], d[4];
+  int dmax = 0;
 #pragma unroll
   for (int a = 0; a < 4; ++a) {
     const int vtx = tets[a * nt + t];
     ua[a] = u[vtx];
     d[a] = du[vtx];
+    dmax = max(dmax, abs_hi(d[a]));
   }
   const double sd = (d[0] + d[1]) + (d[2] + d[3]), s = coef * vol[t];
   for (int o = 0; o < nomega; ++o) {
+    double* out = loc + (int64_t)o * 12 * nt;
     double w[4], n[3][4], T[3];
+    int wmax = dmax;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) w[a] = fma(omegas.v[o], d[a], ua[a]);
+    for (int a = 0; a < 4; ++a) {
+      w[a] = fma(omegas.v[o], d[a], ua[a]);
+      wmax = max(wmax, abs_hi(w[a]));
+    }
+    if (wmax >= ORBIT_MAX_HI) {
+      omega_wide(S, ua, d, omegas.v[o], s, nt, t, out);
+      continue;
+    }
     const double sw = (w[0] + w[1]) + (w[2] + w[3]);
     auto point = [&](double wq, double dq, double (&x)[3]) {
       double G, H;
@@ -705,7 +752,6 @@ __global__ void __launch_bounds__(128) k_omega_f64(const double* __restrict__ u,
     };
     orbit(A1, D1, W1);
     orbit(A2, D2, W2);
-    double* out = loc + (int64_t)o * 12 * nt;
 #pragma unroll
     for (int k = 0; k < 3; ++k)
 #pragma unroll
