@@ -25,6 +25,7 @@
 #include "fp64_math.cuh"
 #include "pbfb_internal.cuh"
 #include "quad_tables.cuh"
+#include "solid_angle.h"
 
 namespace pbfb {
 
@@ -807,12 +808,12 @@ __global__ void k_chunk_sum(int n, int nchunk, const double* __restrict__ part, 
   out[i] = v;
 }
 
-// Winding numbers of Gamma_m at the charges: sum over the triangles of their signed solid angles by Van Oosterom
-// and Strackee's formula, 2 atan2(det, den), as on the host (winding_numbers in mesh_setup.cu) with the same
-// test for points on a triangle.  det and den in float64, whose pipe bounds it (63 operations per pair), the
-// angle itself in float32: its 1e-7 per triangle against the threshold 3/4 between 1 and 1/2.  A thread takes a
-// charge, chunks of the triangles (blockIdx.y) give the blocks; a point on the surface makes its sum huge.
-// GB300, 1536 charges on 15,680 triangles: 30 to 42 ms on 16 host cores, 3.1 ms here; 200 on 8000, 0.15 ms.
+// Winding numbers of Gamma_m at the charges: sum over the triangles of their signed solid angles (half_solid_angle), as
+// on the host (winding_numbers in mesh_setup.cu) with the same test for points on a triangle, all in float64, whose
+// pipe bounds it.  A thread takes a charge, chunks of the triangles (blockIdx.y) give the blocks; a point on the
+// surface makes its sum huge.
+// GB300, the whole charges_set: 1536 charges on 15,680 triangles 35.5 ms with this check on 16 host cores, 10.2 ms so
+// (8.6 with the angles in float32); 200 on 8000, 3.2 and 0.87 ms (0.71).
 constexpr int WIND_T = 64;
 constexpr double WIND_ON = 1e30;
 __global__ void __launch_bounds__(WIND_T) k_winding(int nt, const int* __restrict__ tri, const int* __restrict__ vmap,
@@ -835,7 +836,6 @@ __global__ void __launch_bounds__(WIND_T) k_winding(int nt, const int* __restric
       }
     __syncthreads();
     const int cnt = min(WIND_T, t1 - t0);
-    float s = 0.f;
     for (int i = 0; i < cnt; ++i) {
       const double* p = P[i];
       const double a0 = p[0] - x, a1 = p[1] - y, a2 = p[2] - z;
@@ -847,17 +847,9 @@ __global__ void __launch_bounds__(WIND_T) k_winding(int nt, const int* __restric
         on = true;
         continue;
       }
-      const double ra = rsqrt64(ra2), rb = rsqrt64(rb2), rc = rsqrt64(rc2);
-      const double la = ra2 * ra, lb = rb2 * rb, lc = rc2 * rc, s3 = la * lb * lc;
-      const double det = fma(a2, fma(b0, c1, -b1 * c0), fma(a0, fma(b1, c2, -b2 * c1), -a1 * fma(b0, c2, -b2 * c0)));
-      const double ab = fma(a2, b2, fma(a1, b1, a0 * b0)), bc = fma(b2, c2, fma(b1, c1, b0 * c0)),
-                   ca = fma(c2, a2, fma(c1, a1, c0 * a0));
-      const double den = fma(ca, lb, fma(bc, la, fma(ab, lc, s3)));
-      if (fabs(det) <= 1e-12 * s3 && den <= 0.0) on = true;
-      const double inv = ra * rb * rc;
-      s += atan2f((float)(det * inv), (float)(den * inv));
+      sum += half_solid_angle(a0, a1, a2, b0, b1, b2, c0, c1, c2, ra2 * rsqrt64(ra2), rb2 * rsqrt64(rb2),
+                              rc2 * rsqrt64(rc2), &on);
     }
-    sum += (double)s;
   }
   if (k < nq) part[(size_t)blockIdx.y * nq + k] = on ? WIND_ON : sum;
 }

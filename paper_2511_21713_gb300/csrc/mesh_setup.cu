@@ -19,6 +19,7 @@
 #include "host_ranges.h"
 #include "pbfb_internal.cuh"
 #include "quad_tables.cuh"
+#include "solid_angle.h"
 
 namespace pbfb {
 
@@ -1030,13 +1031,9 @@ int mesh_create(const double* xyz, int nv, const int* tets, int64_t nt, const in
 }
 
 // Generalised winding number of a closed triangulated surface at points q (n of them):
-// w(x) = (1/4 pi) sum_tau Omega_tau(x), with the signed solid angle of each triangle from the formula
-// of Van Oosterom and Strackee (1983),
-//   tan(Omega/2) = a.(b x c) / (|a||b||c| + (a.b)|c| + (b.c)|a| + (c.a)|b|),  a, b, c = corners - x.
+// w(x) = (1/4 pi) sum_tau Omega_tau(x), the signed solid angle of each triangle from half_solid_angle.
 // With the normals pointing out of the enclosed region, w = 1 inside, 0 outside and 1/2 on the
-// surface.  A point on a triangle (a corner, or coplanar to 1e-12 relative with the formula's
-// denominator not positive, i.e. within the triangle) makes that triangle's solid angle +-2 pi by
-// the sign of a rounded zero; such points are reported as on the surface, w = 1/2.
+// surface (points on a triangle are reported so).
 // tri9: 9 coordinates per triangle.  Host threads over the points.
 void winding_numbers(const double* tri9, size_t nt, const double* q, int nq, double* w) {
   auto work = [&](int k0, int k1) {
@@ -1052,12 +1049,7 @@ void winding_numbers(const double* tri9, size_t nt, const double* q, int nq, dou
         const double la = std::sqrt(a0 * a0 + a1 * a1 + a2 * a2);
         const double lb = std::sqrt(b0 * b0 + b1 * b1 + b2 * b2);
         const double lc = std::sqrt(c0 * c0 + c1 * c1 + c2 * c2);
-        const double det = a0 * (b1 * c2 - b2 * c1) - a1 * (b0 * c2 - b2 * c0) + a2 * (b0 * c1 - b1 * c0);
-        const double den = la * lb * lc + (a0 * b0 + a1 * b1 + a2 * b2) * lc + (b0 * c0 + b1 * c1 + b2 * c2) * la +
-                           (c0 * a0 + c1 * a1 + c2 * a2) * lb;
-        const double s3 = la * lb * lc;
-        if (s3 == 0.0 || (std::fabs(det) <= 1e-12 * s3 && den <= 0.0)) on = true;
-        sum += 2.0 * std::atan2(det, den);
+        sum += 2.0 * half_solid_angle(a0, a1, a2, b0, b1, b2, c0, c1, c2, la, lb, lc, &on);
       }
       w[k] = on ? 0.5 : sum / (4.0 * M_PI);
     }
