@@ -383,8 +383,9 @@ typedef struct pbfb_tuning {
                                         2: mutual pairs, each point pair evaluated once for
                                         both directions (4 targets per thread; blocks_per_sm
                                         counts one-warp blocks) */
-  int32_t ff_blocks_per_sm;          /* float-float far field: an eighth of its tasks per SM
-                                        (ff_kernel 1: source splits), 1..64 */
+  int32_t ff_blocks_per_sm;          /* float-float far field: an eighth of its tasks per SM,
+                                        values above 16 acting as 16 (ff_kernel 1: source
+                                        splits), 1..64 */
   int32_t ff_kernel;                 /* float-float far field: 1 one target per thread; 0, 2, 3
                                         and 4 pairs of triangles, each pair of points evaluated
                                         once for both directions (float2) */

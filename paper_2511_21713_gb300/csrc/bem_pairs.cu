@@ -37,6 +37,7 @@
 #include "device_once.h"
 #include "f32x2.cuh"
 #include "fp64_math.cuh"
+#include "pair_split.h"
 #include "pbfb_internal.cuh"
 #include "quad_tables.cuh"
 
@@ -44,7 +45,7 @@ namespace pbfb {
 
 namespace {
 
-constexpr int PT = 32;               // triangles per tile: one per lane
+constexpr int PT = PAIR_TILE;        // triangles per tile: one per lane
 constexpr int PW = 4;                // warps (independent tasks) per block
 constexpr int FF_GEO = 48;           // float rows of a tile: 18 hi, 18 lo coordinates, 3 hi, 3 lo normals, 6 plane offsets
 constexpr int FF_SRC = 24;           // s hi, s lo, mu hi, mu lo of the 6 points
@@ -628,38 +629,8 @@ int pair_tables(Mesh* m, bool f64) {
   return m->pair_tab.upload(t.data(), t.size(), m->stream);
 }
 
-// Split of a surface's tile pairs into tasks: G groups of tpg tiles, K parts of the 32 steps, and nsub
-// shares of a triangle's points (3: a packed pair per lane; 1: all six).  One tile per group while that
-// gives no more than `want` tasks; below some thousand tasks the chip is not full, and the steps are cut
-// into parts and (float-float) the points into shares, which cost 12 % more operations but a third of the
-// serial work of a lane.  GB300, one call of a K operator, us, (nsub, K) -- float-float, 320 triangles (10
-// tiles): (1, 8) 75, (3, 4) 72, (3, 8) 76; 980 (31): (1, 2) 145, (3, 4) 139; 1280 (40): (1, 2) 192, (3, 2) 192;
-// 2000 (63): (1, 2) 373, (3, 1) 371; 2880 (90): (1, 2) 683, (3, 1) 719; 3920 (123): (1, 1) 1209, (3, 1) 1266.
-// The float64 pipe is one unit per SM, so only the balance counts: 1620 triangles (51), Yukawa: K = 1 3694, 4
-// 3097, 8 2817.
-void pair_split(int nt, int want, bool f64, PairSplit* S) {
-  S->nT = std::max(1, (nt + PT - 1) / PT);
-  S->nsub = 1;
-  S->K = 1;
-  const int G = std::max(1, std::min((int)std::sqrt(2.0 * want), S->nT));
-  S->tpg = S->nT / G;
-  S->G = (S->nT + S->tpg - 1) / S->tpg;
-  auto tasks = [&] { return (int64_t)S->G * (S->G + 1) / 2 * S->K * S->nsub; };
-  if (S->tpg == 1) {
-    if (!f64 && tasks() <= 2048) S->nsub = 3;
-    while (tasks() * 2 <= (f64 ? 24000 : 8192) && S->K < (f64 ? 8 : 4)) S->K *= 2;
-  }
-  S->ntask = (int)tasks();
-  S->rows = S->nsub == 1 ? (size_t)S->K * (S->G + 1) : (size_t)S->K * S->G * (1 + S->nsub);
-}
-
 // doubles of partial sums and their total, the larger of the two forms
-size_t pair_work(int64_t nt) {
-  PairSplit a, b;
-  pair_split((int)nt, 152 * 32, true, &a);
-  pair_split((int)nt, 152 * 128, false, &b);
-  return (std::max(a.rows, b.rows) + 1) * QS * (size_t)nt;
-}
+size_t pair_work(int64_t nt) { return (pair_rows_max((int)nt) + 1) * QS * (size_t)nt; }
 
 int launch_pairs(Mesh* m, Surface* s, const double* x, const double* lam, double cs, double cd, double kappa, bool f64,
                  double** val) {
@@ -668,11 +639,7 @@ int launch_pairs(Mesh* m, Surface* s, const double* x, const double* lam, double
   const int u_local = (x != nullptr && x == lam) ? 1 : 0;
   const double* uvec = cd != 0.0 ? x : nullptr;
   const double* lvec = cs != 0.0 ? lam : nullptr;
-  // tasks: 128 a SM, ten waves of the resident warps or so, which keeps the last one short (8000 triangles,
-  // float-float: one tile per group 4.61 + 6.41 ms, two 4.67 + 6.50; 15,680: two 17.4 + 24.3, three 17.8 + 24.8)
-  const int want = 152 * (f64 ? 32 : 8 * (m->tune_ff_bps > 0 ? m->tune_ff_bps : 16));
-  PairSplit S;
-  pair_split(nt, want, f64, &S);
+  const PairSplit S = pair_split(nt, pair_want(f64, m->tune_ff_bps), f64);
   const int nT = S.nT, npad = nT * PT * QS;
   PB_TRY(pair_tables(m, f64));
   PB_TRY(ensure(s->mval, (S.rows + 1) * nq));

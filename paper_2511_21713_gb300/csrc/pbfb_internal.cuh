@@ -379,11 +379,6 @@ inline double ff_grid(const Surface* s, double scale) {
 }
 
 // ---- bem_pairs.cu: far fields of the accurate precisions by pairs of triangles
-struct PairSplit {
-  int nT, tpg, G, K, nsub, ntask;  // tiles, tiles per group, groups, step parts, point shares, tasks
-  size_t rows;                     // rows of partial sums
-};
-void pair_split(int nt, int want, bool f64, PairSplit* S);
 size_t pair_work(int64_t nt);
 // far-field potentials at the quadrature points (float64 if f64, else float-float); *val: device, nq
 int launch_pairs(Mesh* m, Surface* s, const double* x, const double* lam, double cs, double cd, double kappa, bool f64,
