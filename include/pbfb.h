@@ -432,8 +432,7 @@ int pbfb_apply_tuning(pbfb_mesh* mesh, const pbfb_tuning* t);
  * candidate shape of the float32 far field (targets per thread 1/2/4, packed
  * or not, 8/16/32 blocks per SM of source splits; or mutual pairs with
  * 16/32/64 one-warp blocks per SM) and of the float-float far
- * field (4/8/16/24 blocks per SM; one target per thread, or pairs of
- * triangles) on both
+ * field by pairs of triangles (ff_blocks_per_sm 4/8/16) on both
  * surfaces of this mesh at the current parameters, and of the operator's
  * SpMV (4/8/16 lanes per row x 128/256/512 threads) and of the cooperative
  * inner PCG of the block preconditioner (1/2/4/8 blocks per SM or all that

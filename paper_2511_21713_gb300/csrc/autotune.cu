@@ -150,25 +150,25 @@ int autotune(Mesh* m, int reps, pbfb_tuning* best_out, double* ms_out) {
       best.treecode = tc;
     }
   }
-  // float-float far field
-  for (int kind : {1, 4})
-    for (int bps : {4, 8, 16, 24}) {
-      pbfb_tuning t = best;
-      t.ff_kernel = kind;
-      t.ff_blocks_per_sm = bps;
-      write_tuning(m, &t);
-      double ms;
-      int st = time_ms(m, reps, far(PBFB_FLOAT2), &ms);
-      if (st) {
-        write_tuning(m, &cur);
-        return st;
-      }
-      if (ms < t_best[1]) {
-        t_best[1] = ms;
-        best.ff_kernel = kind;
-        best.ff_blocks_per_sm = bps;
-      }
+  // float-float far field: pairs of triangles (the one-target-per-thread sum, ff_kernel 1, is slower at every size, see
+  // launch_bem_far_ff)
+  for (int bps : {4, 8, 16}) {
+    pbfb_tuning t = best;
+    t.ff_kernel = 4;
+    t.ff_blocks_per_sm = bps;
+    write_tuning(m, &t);
+    double ms;
+    int st = time_ms(m, reps, far(PBFB_FLOAT2), &ms);
+    if (st) {
+      write_tuning(m, &cur);
+      return st;
     }
+    if (ms < t_best[1]) {
+      t_best[1] = ms;
+      best.ff_kernel = 4;
+      best.ff_blocks_per_sm = bps;
+    }
+  }
   // SpMV of the operator's sparse part (10 products per repetition)
   for (int L : {4, 8, 16})
     for (int B : {128, 256, 512}) {

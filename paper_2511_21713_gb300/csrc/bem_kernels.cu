@@ -1098,7 +1098,10 @@ int launch_bem_far_ff(Mesh* m, Surface* s, const double* x, const double* lam, d
   const int nq = s->nq;
   const bool yuk = kappa != 0.0;
   const int u_local = (x != nullptr && x == lam) ? 1 : 0;
-  // by pairs of triangles; ff_kernel = 1 asks for the one-target-per-thread sum.  Lengths are scaled by kappa
+  // by pairs of triangles; ff_kernel = 1 asks for the one-target-per-thread sum, which shares no pair formula with them
+  // (a check of either by the other) and is slower at every size (K operator, Laplace / Yukawa: 20 triangles 44 / 71
+  // against 36 / 40 us; 500, 119 / 241 and 58 / 68; 3920, 2.46 / 4.40 and 1.03 / 1.48 ms; 20,480, 66 / 119 and 26 /
+  // 37), so that neither the built-in shapes nor the autotuner take it.  Lengths are scaled by kappa
   // there: a Yukawa kernel with kappa below 1e-8 (no physical ionic strength; the scaled 1/r^3 nears the end of
   // float32's range) takes the float64 form.
   if (m->tune_ff_kernel != 1) {
