@@ -439,7 +439,9 @@ __device__ __noinline__ void element_wide(int scheme, const double* ua4, double 
 // Jacobian and load of F on one tet in float64 (layout k * nt + t: J at k = 0..9, N at k = 10..13), from the orbit
 // sums of k_element_ff below.  The float64 pipe bounds it: about 400 operations a tet for the sinh scheme, 1000 with
 // the 14 points one by one, the library's exponential and a division.
-// GB300, 86,400 tets: 128 us so, 72 us now.
+// GB300, 86,400 tets: 128 us so, 72 us now.  Against long double the loads' errors scatter alike (1.35e-16 of their
+// terms' magnitudes, rms over the vertices, both forms); the products of weights, rounded once at compile time, shift
+// all of them by 3e-17.
 template <int S>
 __global__ void __launch_bounds__(128) k_element_f64(const double* __restrict__ u, const int* __restrict__ tets,
                                                      int64_t nt, const double* __restrict__ vol, double coef,

@@ -201,8 +201,8 @@ struct Mesh {
   DBuf<double> tloc;        // 10 * nt Jacobian + 4 * nt load, tet-local
   DBuf<double> wloc;        // omega batch: nomega * 12 * nt
   DBuf<double> red;         // block partial sums
-  DBuf<double> scal;        // device scalars: [0,64) omegas, [64, 64+7*64+3) omega dots,
-                            // [1000] ion integral, [4000] dot result, [5000, 5502) PCG scalars
+  DBuf<double> scal;        // device scalars: [0, 7*64+3) omega dots, [1000, 1003) reaction energies and ion integral,
+                            // [4000] dot result, [4100, 4104) the flux's CG, [5000, 5502) PCG scalars
   DBuf<double> red2;        // pair-local mass entries during correction builds
   double* pinned = nullptr; // host pinned scratch (4096 doubles)
   // GMRES workspace
@@ -371,7 +371,7 @@ int launch_reaction_energy(Mesh* m, const double* xL, const double* xNL, double*
 int bem_apply_noalloc(Mesh* m, int which, int op, const double* x, double* y);
 
 // Grid of the float-float coordinates' high parts for lengths scaled by `scale` (a power of 2): differences
-// of two of them are below 2^24 steps, hence exact in float32.  Low parts lie on its 2^-25th part, within half
+// of two of them are below 2^24 steps, hence exact in float32.  Low parts lie on its 2^-24th part, within half
 // a step, so that they are float32 numbers and most differences of two of them are exact too: the pair
 // arithmetic then sees the same (rounded) points in every pair.
 inline double ff_grid(const Surface* s, double scale) {
