@@ -25,9 +25,10 @@
 // surface, 7.58 + 11.12 ms for mutual pairs of points with a dipole vector each (97.7 and 145.7 float32 lane
 // operations per ordered pair) to 3.9 + 5.7 ms (58 and 82 counted in the source; 82 to 86 % of the float32
 // pipes' rate); float64, 3380 triangles, 14.9 + 33.6 ms one-directionally with the library's root and
-// exponential to 7.0 + 11.6 ms (9.3 and 13.3 float64 operations per ordered pair, four fifths of the
-// float64 pipe's rate).  Errors of V and K against 64 bits: float64 unchanged (7e-16 to 1.7e-15), float-float
-// 2.5e-15 (V, from 4e-15) and 1.1e-14 (K, from 2e-14 to 7e-14).
+// exponential to 7.0 + 11.6 ms (9.3 and 13.3 float64 operations per ordered pair counted in the source; the float64
+// pipe 88 to 90 % busy).  Errors of V and K: float64 against long double (320 triangles) 0.9e-16 to 1.2e-16 (V, from
+// 1.5e-16 to 2.1e-16) and 1.4e-16 to 1.8e-16 (K, from 3.4e-16 to 6.1e-16); float-float against 64 bits 2.5e-15 (V, from
+// 4e-15) and 1.1e-14 (K, from 2e-14 to 7e-14).
 #include <cuda_runtime.h>
 
 #include <algorithm>
