@@ -229,7 +229,8 @@ int pbfb_surface_vertices(const pbfb_mesh* mesh, int which, int32_t* out);
  * shell mesh every charge must lie strictly inside Gamma_m (in Omega_m, as the
  * three-region model of Sec. 2.1 places them), checked by the winding number of
  * pbfb_check_charges before the charges are taken; PBFB_ERR_INVALID
- * otherwise, the mesh keeping its previous charges. */
+ * otherwise, the mesh keeping its previous charges.  An error past this check
+ * (out of memory) leaves the mesh without charges. */
 int pbfb_charges_set(pbfb_mesh* mesh, const double* xyz, const double* z, int32_t n_q);
 
 /* Host-only input check (no GPU needed): the generalised winding number

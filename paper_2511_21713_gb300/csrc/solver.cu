@@ -2341,6 +2341,8 @@ int charges_set(Mesh* m, const double* xyz, const double* z, int n_q) {
     for (int k = 0; k < n_q; ++k)
       if (!(w[k] > 0.75)) return charge_outside(k, xyz + 3 * (size_t)k, w[k]);
   }
+  // from here on the old set is overwritten: an error (out of memory) leaves the mesh without charges, not with a mixture
+  m->charges = false;
   if (m->full) PB_TRY(m->rho.upload(rho.data(), rho.size(), m->stream));
   PB_TRY(ensure(m->qxyz, soa.size()));
   PB_TRY(ensure(m->qz, n_q));
