@@ -10,8 +10,8 @@ namespace pbfb {
 
 constexpr int HOST_THREADS = 16;
 
-// A partition of [0, n) into at most HOST_THREADS ranges of `grain` items or more, made once and run any number of times:
-// what a pass keeps per range (sizes, buffers) fits every later pass of the same object, whatever the machine's
+// A partition of [0, n) into at most HOST_THREADS ranges of `grain` items or more, made once and run any number of
+// times: what a pass keeps per range (sizes, buffers) fits every later pass of the same object, whatever the machine's
 // processor count says by then.
 class HostRanges {
  public:

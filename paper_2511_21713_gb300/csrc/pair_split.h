@@ -33,8 +33,8 @@ inline int pair_want(bool f64, int ff_bps) {
 // fewer an uneven last wave (8000 triangles, 250 tiles, above; rounding up would take two tiles a group there).  Below
 // some thousand tasks the chip is not full, and the steps are cut into parts and (float-float) the points into shares,
 // which cost 12 % more operations but a third of the serial work of a lane.  GB300, one call of a K operator, us,
-// (nsub, K), before the pair loop was unrolled -- float-float, 320 triangles (10 tiles): (1, 8) 75, (3, 4) 72, (3, 8) 76;
-// 980 (31): (1, 2) 145, (3, 4) 139; 1280 (40): (1, 2) 192, (3, 2) 192; 2000 (63): (1, 2) 373, (3, 1) 371; 2880 (90):
+// (nsub, K), before the pair loop was unrolled -- float-float, 320 triangles (10 tiles): (1, 8) 75, (3, 4) 72, (3, 8)
+// 76; 980 (31): (1, 2) 145, (3, 4) 139; 1280 (40): (1, 2) 192, (3, 2) 192; 2000 (63): (1, 2) 373, (3, 1) 371; 2880 (90):
 // (1, 2) 683, (3, 1) 719; 3920 (123): (1, 1) 1209, (3, 1) 1266.  The float64 pipe is one unit per SM, so only the
 // balance counts: 1620 triangles (51), Yukawa: K = 1 3694, 4 3097, 8 2817.
 inline PairSplit pair_split(int nt, int want, bool f64) {

@@ -12,8 +12,8 @@
 
 namespace pbfb {
 
-// Half the signed solid angle that the triangle with corners a, b, c (relative to the point, of lengths la, lb, lc) takes
-// up, Van Oosterom and Strackee (1983):
+// Half the signed solid angle that the triangle with corners a, b, c (relative to the point, of lengths la, lb, lc)
+// takes up, Van Oosterom and Strackee (1983):
 //   tan(Omega / 2) = a.(b x c) / (|a||b||c| + (a.b)|c| + (b.c)|a| + (c.a)|b|).
 // *on: the point lies on the triangle (a corner, or coplanar to 1e-12 relative with the denominator not positive,
 // i.e. within the triangle), where the sign of a rounded zero would make the angle +-2 pi.
